@@ -199,7 +199,8 @@ bst_status bst_plan_get_stacks(const bst_plan *plan, int32_t *mnk, int64_t *buck
                                int32_t *a_off, int32_t *b_off, int32_t *c_off);
 
 /* Work units of the native-FP64 staged kernel: hist[s] (s = 1..16) = row tiles of C
- * whose inner dimension is split over s lane groups (choice of BST_TUNE_F64_SPLIT and
+ * whose inner dimension is split over s lane groups, for all their outputs or for the
+ * last partial round of 32 (choice of BST_TUNE_F64_SPLIT and
  * the built-in cost rule, as of the last execute or plan build); hist[0] = C blocks
  * run by the direct-load kernel instead (plans whose blocks do not fit the staged
  * tiles).  hist has 17 entries.  Synchronises. */
@@ -294,10 +295,10 @@ bst_status bst_plan_destroy(bst_plan *plan);
  *     -1 = back to the built-in rule (fewer 16 x 8 tiles wins).  Row-scaled mode only.
  *   BST_TUNE_F64_SPLIT (per (m, n) C block class): the largest number of lane groups
  *     over which the native-FP64 staged kernel may split the inner dimension of one
- *     C tile (1 = never split; 2..16); -1 = back to the built-in bound.  Within the
- *     bound each tile takes the split that needs the fewest FP64 instructions, and
- *     only when that saves at least 1/16 of them; the s partial sums of an output are
- *     added in a fixed order, so results stay deterministic.
+ *     C tile, or of its last partial round of 32 outputs (1 = never split; 2..16); -1 =
+ *     back to the built-in bound.  Within the bound each tile takes the split that needs
+ *     the fewest FP64 instructions; the partial sums of an output are added in a fixed
+ *     order, so results stay deterministic.
  *   BST_TUNE_CONTRACT_SLAB (m, n ignored): 1 = when a contraction's first tensor is
  *     stored as (outer contracted modes, free modes, inner contracted modes), e.g.
  *     T(P, mu, nu) contracted over (P, nu), its matrix view is read in place as

@@ -36,7 +36,7 @@ struct bst_batch {
   size_t pbytes = 0;
   int grid = 0;
   int stage_elems = 0;  // staged FP64 kernel slot size (0: some plan needs direct loads)
-  bool stage_strided = false;
+  bool stage_strided = false, stage_wide = false;
   int64_t n_titems = 0;
   int64_t *titems = nullptr;  // staged kernel: every plan's tiles by decreasing cost
   // emulated FP64 schedule (item = plan << 32 | C block)
@@ -154,7 +154,10 @@ bst_status bst_batch_create(bst_ctx *ctx, int32_t n, bst_plan *const *plans, bst
           mx = std::max(mx, (int)p->stage_elems);
         }
         if (all) b->stage_elems = std::max(mx, 1);
-        for (auto *p : b->plans) b->stage_strided = b->stage_strided || p->stage_strided;
+        for (auto *p : b->plans) {
+          b->stage_strided = b->stage_strided || p->stage_strided;
+          b->stage_wide = b->stage_wide || p->stage_wide;
+        }
       }
       if (b->stage_elems > 0) {
         for (auto *p : b->plans) b->n_titems += p->n_tiles;
@@ -267,7 +270,7 @@ bst_status bst_batch_execute(bst_batch *b, const double *alpha, const double *be
       }
       if (b->stage_elems > 0)
         bst::launch_fp64_staged(b->d_params, b->titems, b->n_titems, b->stage_elems,
-                                b->stage_strided, split, b->ctx->num_sms, b->counter, s);
+                                b->stage_strided, split, b->stage_wide, b->ctx->num_sms, b->counter, s);
       else
         bst::launch_fp64_persist(b->d_params, b->items, b->n_items, b->counter, b->grid, s);
     } else {

@@ -334,7 +334,8 @@ struct bst_plan {
   int64_t *titems = nullptr;   // tiles by decreasing cost
   int32_t *tkeys = nullptr;    // each tile's cost key
   int64_t split_version = -1;  // tune_version the tiles' inner splits were chosen for
-  bool stage_split = false;    // some tile splits its inner dimension
+  bool stage_split = false;    // some whole tile splits its inner dimension
+  bool stage_wide = false;     // tiles up to 544 elements (else 320)
   bst::Arena sched_ar;         // the staged schedule's arrays (rebuilt for slab reading)
   // Slab reading of a contraction operand (set by the contraction before the staged
   // schedule is built): A's stored block (m x k, k = k_o * k_i) is k_o contiguous m x k_i
@@ -427,7 +428,7 @@ constexpr int kF64DescWords = 8;  // descriptor words per staged tile
 void build_plan_tile_items(bst_plan *p, int64_t base, int64_t *items, int32_t *keys,
                            cudaStream_t s);
 void launch_fp64_staged(const void *params, const int64_t *items, int64_t nitems,
-                        int slot_elems, bool strided, bool split, int num_sms,
+                        int slot_elems, bool strided, bool split, bool wide, int num_sms,
                         unsigned long long *counter, cudaStream_t s);
 // persistent emulated-FP64 numeric (numeric_emu.cu)
 size_t emu_params_bytes();

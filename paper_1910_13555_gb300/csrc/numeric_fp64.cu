@@ -274,9 +274,9 @@ __global__ void __launch_bounds__(256, 2)
 
 // ---- staged persistent kernel ---------------------------------------------------------
 //
-// The work units are row tiles of C blocks (whole blocks up to 32 * kMaxR elements) and
+// The work units are row tiles of C blocks (whole blocks up to 32 MR elements) and
 // their entries are (product, inner panel) pairs, both cut on the host so that one
-// entry's operands always fit a shared-memory slot (kStageMax doubles).  A warp walks a
+// entry's operands always fit a shared-memory slot.  A warp walks a
 // stream of jobs (the entries of its tiles, tile by tile) and keeps two slots: while it
 // multiplies the op(A) and op(B) panels of job j from one slot, those of job j + 1 --
 // possibly the first job of its next tile -- arrive in the other through cp.async, so
@@ -292,22 +292,30 @@ __global__ void __launch_bounds__(256, 2)
 // value is needed, so the atomic's latency is hidden too.  Which warp runs a tile does
 // not change its result: every tile is summed by one warp in its entry order.
 
-constexpr int kMaxR = 17;         // accumulators per lane: tiles up to 544 elements
-constexpr int kTile = 32 * kMaxR;
-// doubles per slot (two slots per warp): at most 1184 keeps three 4-warp CTAs resident
-// per SM (3 x (2 x 4 x 1184 x 8 B + 1 KB) <= 228 KB); the panels get narrower, but with
-// 1536 the contraction plans ran 2 CTAs per SM and lost 8-9 % (FP64 pipe 68-82 % busy)
-constexpr int kStageMax = 1184;
+// Two shapes of the kernel (MR accumulators per lane, tiles up to 32 MR elements):
+// * MR = 10, slots of at most 896 doubles: four 4-warp CTAs per SM (at most 128
+//   registers, 4 x (2 x 4 x 896 x 8 B + 1 KB) <= 228 KB).  The FP64 pipe takes 16 SM
+//   cycles per warp FMA and idles when no resident warp has one ready: with 17
+//   accumulators and 1184-double slots 12 warps fitted and the pipe was 94 % busy on the
+//   banded product (20.8 ms); 16 warps keep it 96 % busy (18.9 ms with the tail split).  A
+//   23 x 23 block is then cut into tiles of 13 and 10 rows.
+// * MR = 17, slots of 1184 doubles, three CTAs per SM ("wide"): for plans with rows of C
+//   of 321 to 544 elements, and for contractions read in place as slabs (which need whole
+//   C blocks) with blocks of 321 to 544 elements.
+constexpr int kNarrowR = 10, kWideR = 17;
+constexpr int kNarrowSlot = 896, kWideSlot = 1184;
 constexpr int kStageWarps = 4;    // warps per CTA
 constexpr int kF64Desc = kF64DescWords;
 
-// Work unit: a row tile of a C block (the whole block when it has at most 32 * kMaxR
+// Work unit: a row tile of a C block (the whole block when it has at most 32 MR
 // elements).  Descriptor: 0 element offset of the tile in C, 1 first entry, 2 entry
 // count, 3 tile rows m | n << 12, 4 C_in block (-1: none), 5 element offset of the tile
-// inside the C_in block, 6 C block, 7 inner split s (>= 1).
+// inside the C_in block, 6 C block, 7 inner split s (>= 1) | tail split << 8 (>= 1, taken
+// when s = 1; see slot_tail).
 struct F64Blk {
   int off, eb, ne, m, n, cin, cio, s;
 };
+__device__ __forceinline__ int f64_split_word(int s, int tail) { return s | (tail << 8); }
 
 __device__ __forceinline__ F64Blk f64_blk(int dw) {
   F64Blk b;
@@ -317,7 +325,7 @@ __device__ __forceinline__ F64Blk f64_blk(int dw) {
   const int mn = __shfl_sync(0xffffffffu, dw, 3);
   b.cin = __shfl_sync(0xffffffffu, dw, 4);
   b.cio = __shfl_sync(0xffffffffu, dw, 5);
-  b.s = max(__shfl_sync(0xffffffffu, dw, 7), 1);
+  b.s = __shfl_sync(0xffffffffu, dw, 7);
   b.m = mn & 0xfff;
   b.n = (mn >> 12) & 0xfff;
   return b;
@@ -335,19 +343,33 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_grou
 // panels and tiles of large products take it).  stride < len: the source is len / stride
 // consecutive slabs of rows x stride doubles (a slab-read operand), one contiguous range
 // whose slab j supplies columns j stride .. (j + 1) stride - 1 of every row.
-__device__ __noinline__ void stage_strided(double *dst, const double *src, int rows, int len,
+//
+// A lane's elements i = lane, lane + 32, ... are located by mixed-radix digits (slab j,
+// row r, column c) decoded once and advanced by the digits of 32 with carries, with no
+// division per element.
+__device__ __forceinline__ void stage_strided(double *dst, const double *src, int rows, int len,
                                            int stride) {
-  const int lane = threadIdx.x & 31;
-  if (stride < len) {
-    const int per = rows * stride;
-    for (int i = lane; i < rows * len; i += 32) {
-      const int j = i / per, rem = i - j * per, r = rem / stride;
-      cp_async8(dst + r * len + j * stride + (rem - r * stride), src + i);
+  const int lane = threadIdx.x & 31, total = rows * len;
+  const bool slabs = stride < len;
+  const int w = slabs ? stride : len;         // columns of one slab
+  const int64_t rs = slabs ? w : stride;      // source row stride
+  const int dr0 = 32 / w, dc = 32 - dr0 * w, dj = dr0 / rows, dr = dr0 - dj * rows;
+  const int r0 = lane / w;
+  int c = lane - r0 * w, j = r0 / rows, r = r0 - j * rows;
+  for (int i = lane; i < total; i += 32) {
+    cp_async8(dst + r * len + j * w + c, src + (int64_t)j * rows * w + r * rs + c);
+    c += dc;
+    r += dr;
+    j += dj;
+    if (c >= w) {
+      c -= w;
+      ++r;
     }
-    return;
+    if (r >= rows) {
+      r -= rows;
+      ++j;
+    }
   }
-  for (int r = 0; r < rows; ++r)
-    for (int c = lane; c < len; c += 32) cp_async8(dst + r * len + c, src + (int64_t)r * stride + c);
 }
 
 template <bool STRIDED>
@@ -380,49 +402,131 @@ __device__ __forceinline__ void stage_product(double *slot, const double *a, con
     stage_2d<STRIDED>(slot + m * w, b, w, n, sb);
 }
 
-// acc[r] += op(A)(p_r, :) . op(B)(:, q_r) from a slot for o = lane + 32 r = p_r n + q_r:
-// any (m, n) with m n <= 32 kMaxR, runtime sizes, one body for every size.  Bodies
-// specialised at compile time per (m, n) in {5, 13, 23}^2 and k in {5, 13, 23} were no
-// faster on GB300 (the FP64 pipe, not the index arithmetic, bounds the product) and their
-// code cost instruction-fetch stalls; one body per accumulator count thrashed the
-// instruction cache outright.
-__device__ __forceinline__ void slot_product_rt(const NumParams &P, const double *__restrict__ As,
-                                                int m, int n, int k, double (&acc)[kMaxR]) {
+// How a lane finds its outputs o = lane + 32 r = p n + q of a tile: row and column of
+// output `lane`, and of the step of 32; computed once per tile.
+struct LaneMap {
+  int p, q, dp, dq;
+};
+
+__device__ __forceinline__ LaneMap lane_map(int n) {
+  const int lane = threadIdx.x & 31;
+  LaneMap L;
+  L.p = lane / n;
+  L.q = lane - L.p * n;
+  L.dp = 32 / n;
+  L.dq = 32 - L.dp * n;
+  return L;
+}
+
+__device__ __forceinline__ void lane_step(const LaneMap &L, int n, int &p, int &q) {
+  p += L.dp;
+  q += L.dq;
+  if (q >= n) {
+    q -= n;
+    ++p;
+  }
+}
+
+// a double at a shared-memory address: the operand addresses advance by one integer add
+// per load, with no pointer arithmetic
+__device__ __forceinline__ double lds(unsigned a) {
+  double v;
+  asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
+  return v;
+}
+
+// acc[r] += op(A)(p_r, :) . op(B)(:, q_r) from a slot for o = lane + 32 r = p_r n + q_r,
+// rounds r < F: any (m, n) with m n <= 32 MR, runtime sizes, one body for every size.
+// The FP64 pipe bounds it (a warp FMA every 16 cycles of an SM); what costs is the time in
+// which no resident warp has an FMA ready, so the code is kept small and rolled: bodies
+// specialised at compile time per (m, n, k), one body per accumulator count, the inner
+// loop unrolled by 2 or 4, and two or four outputs at a time as independent FMA chains all
+// measured the same or slower (banded 4000 x 4000: 19.0 ms rolled with one chain or two,
+// 20.7 ms unrolled by four with two).
+template <int MR>
+__device__ __forceinline__ void slot_product_rt(const NumParams &P, const double *As, int m, int n,
+                                                int k, int F, const LaneMap &L,
+                                                double (&acc)[MR]) {
   const int lane = threadIdx.x & 31, mn = m * n;
-  const double *__restrict__ Bs = As + m * k;
-  const int a_sp = P.ta ? 1 : k, a_sl = P.ta ? m : 1;
-  const int b_sl = P.tb ? 1 : n, b_sq = P.tb ? k : 1;
-  const int R = (mn + 31) >> 5;
-  // output by output: the element's row and column are found once (incrementally from
-  // the previous accumulator's: o grows by 32), then its whole dot product runs
-  int p = lane / n, q = lane - p * n;
-  const int dp = 32 / n, dq = 32 - dp * n;
+  const unsigned A0 = (unsigned)__cvta_generic_to_shared(As), B0 = A0 + 8 * m * k;
+  const int a_sp = 8 * (P.ta ? 1 : k), a_sl = 8 * (P.ta ? m : 1);
+  const int b_sl = 8 * (P.tb ? 1 : n), b_sq = 8 * (P.tb ? k : 1);
+  int p = L.p, q = L.q;
 #pragma unroll
-  for (int r = 0; r < kMaxR; ++r) {
-    if (r >= R) break;
+  for (int r = 0; r < MR; ++r) {
+    if (r >= F) break;
     if (lane + 32 * r < mn) {
-      const double *a = As + p * a_sp, *b = Bs + q * b_sq;
+      unsigned a = A0 + p * a_sp, b = B0 + q * b_sq;
       double s = acc[r];
-#pragma unroll 4
-      for (int l = 0; l < k; ++l) s = fma(a[l * a_sl], b[l * b_sl], s);
+#pragma unroll 1
+      for (int l = 0; l < k; ++l) {
+        s = fma(lds(a), lds(b), s);
+        a += a_sl;
+        b += b_sl;
+      }
       acc[r] = s;
     }
-    p += dp;
-    q += dq;
-    if (q >= n) {
-      q -= n;
-      ++p;
-    }
+    lane_step(L, n, p, q);
   }
+}
+
+// The last, partial round of a tile (rem = m n mod 32 outputs on 32 lanes) with its inner
+// dimension split over t lane groups: lane g rem + o sums l = g, g + t, ... < k for output
+// o of the round.  A warp FMA occupies the FP64 pipe for 16 cycles however few lanes are
+// active, so a 13 x 13 tile's sixth round (9 outputs) costs as much as a full one unless
+// three groups share it.  The partial sums are added once per tile (tail_reduce).  On the
+// banded product this takes the FP64 instructions from 189.0 M to 175.2 M (2000 x 2000
+// blocks), 27.9 to 30.8 useful lanes per instruction.
+struct TailMap {
+  int g, p, q;  // group (>= t: idle lane), row and column of the lane's output
+};
+
+__device__ __forceinline__ TailMap tail_map(int mn, int n, int t) {
+  const int lane = threadIdx.x & 31, rem = mn & 31;
+  TailMap T;
+  T.g = lane / rem;
+  const int o = (mn & ~31) + lane - T.g * rem;
+  T.p = o / n;
+  T.q = o - T.p * n;
+  if (T.g >= t) T.g = 1 << 20;
+  return T;
+}
+
+__device__ __forceinline__ double slot_tail(const NumParams &P, const double *As, int m, int n,
+                                            int k, int t, const TailMap &T, double acc) {
+  const int a_sl = 8 * (P.ta ? m : 1), b_sl = 8 * (P.tb ? 1 : n);
+  unsigned a = (unsigned)__cvta_generic_to_shared(As), b = a + 8 * m * k;
+  a += 8 * T.p * (P.ta ? 1 : k) + T.g * a_sl;
+  b += 8 * T.q * (P.tb ? k : 1) + T.g * b_sl;
+#pragma unroll 1
+  for (int l = T.g; l < k; l += t) {
+    acc = fma(lds(a), lds(b), acc);
+    a += t * a_sl;
+    b += t * b_sl;
+  }
+  return acc;
+}
+
+// the t partial sums of every output of the tail added in a fixed tree, into group 0
+__device__ __forceinline__ double tail_reduce(int rem, int t, const TailMap &T, double v) {
+  const int lane = threadIdx.x & 31;
+  for (int s = t; s > 1;) {
+    const int h = (s + 1) >> 1;
+    const double w = __shfl_sync(0xffffffffu, v, (lane + h * rem) & 31);
+    if (T.g + h < s) v += w;
+    s = h;
+  }
+  return v;
 }
 
 // The inner dimension split s ways over the lanes, for tiles whose m n leaves lanes idle
 // (65 outputs on 3 x 32 lanes): virtual output v = lane + 32 r = g m n + o (o = p n + q)
 // accumulates op(A)(p, l) op(B)(l, q) over l = g, g + s, g + 2s, ... < k.  The s partial
 // sums of an output are added once, at the end of the tile (split_reduce).
+template <int MR>
 __device__ __forceinline__ void slot_product_split(const NumParams &P,
                                                    const double *__restrict__ As, int m, int n,
-                                                   int k, int s, double (&acc)[kMaxR]) {
+                                                   int k, int s, double (&acc)[MR]) {
   const int lane = threadIdx.x & 31, nv = s * m * n;
   const double *__restrict__ Bs = As + m * k;
   const int a_sp = P.ta ? 1 : k, a_sl = P.ta ? m : 1;
@@ -434,7 +538,7 @@ __device__ __forceinline__ void slot_product_split(const NumParams &P,
   const int dp = 32 / n, dq = 32 - dp * n;
   const int da = s * a_sl, db = s * b_sl;
 #pragma unroll
-  for (int r = 0; r < kMaxR; ++r) {
+  for (int r = 0; r < MR; ++r) {
     if (32 * r >= nv) break;
     if (lane + 32 * r < nv) {
       const double *a = As + p * a_sp + g * a_sl, *b = Bs + q * b_sq + g * b_sl;
@@ -463,14 +567,15 @@ __device__ __forceinline__ void slot_product_split(const NumParams &P,
 
 // acc[r] <- sum over g = 0 .. s - 1 (in that order) of the partial sums of output
 // o = lane + 32 r, through `red` (s m n doubles of a free slot)
-__device__ __forceinline__ void split_reduce(double *red, int mn, int s, double (&acc)[kMaxR]) {
+template <int MR>
+__device__ __forceinline__ void split_reduce(double *red, int mn, int s, double (&acc)[MR]) {
   const int lane = threadIdx.x & 31, nv = s * mn;
 #pragma unroll
-  for (int r = 0; r < kMaxR; ++r)
+  for (int r = 0; r < MR; ++r)
     if (lane + 32 * r < nv) red[lane + 32 * r] = acc[r];
   __syncwarp();
 #pragma unroll
-  for (int r = 0; r < kMaxR; ++r) {
+  for (int r = 0; r < MR; ++r) {
     const int o = lane + 32 * r;
     if (o < mn) {
       double t = red[o];
@@ -481,20 +586,16 @@ __device__ __forceinline__ void split_reduce(double *red, int mn, int s, double 
   __syncwarp();
 }
 
-__device__ __forceinline__ void slot_dispatch(const NumParams &P, const double *As, int m, int n,
-                                              int k, double (&acc)[kMaxR]) {
-  slot_product_rt(P, As, m, n, k, acc);
-}
-
 // C = alpha * acc + beta * C_in for one C block (C_in unread when beta == 0)
+template <int MR>
 __device__ __forceinline__ void store_block(const NumParams &P, const F64Blk &b,
-                                            const double (&acc)[kMaxR]) {
+                                            const double (&acc)[MR]) {
   const int lane = threadIdx.x & 31, mn = b.m * b.n;
   const double *ci = (P.has_beta && b.cin >= 0) ? P.Cin + P.cin_off[b.cin] + b.cio : nullptr;
   double *C = P.C + b.off;
   if (!P.alpha_one || ci) {
 #pragma unroll
-    for (int r = 0; r < kMaxR; ++r) {
+    for (int r = 0; r < MR; ++r) {
       const int o = lane + 32 * r;
       if (o < mn) {
         double v = P.alpha * acc[r];
@@ -504,7 +605,7 @@ __device__ __forceinline__ void store_block(const NumParams &P, const F64Blk &b,
     }
   } else {
 #pragma unroll
-    for (int r = 0; r < kMaxR; ++r)
+    for (int r = 0; r < MR; ++r)
       if (lane + 32 * r < mn) C[lane + 32 * r] = acc[r];
   }
 }
@@ -513,16 +614,17 @@ __device__ __forceinline__ void store_block(const NumParams &P, const F64Blk &b,
 // items[i / ksplit]; the part takes its share of the tile's entries (contiguous, in
 // entry order) and writes its partial sums, without alpha, to W + part * nelem(C), which
 // k_splitk_reduce adds in part order.
+template <int MR>
 __device__ __forceinline__ void store_part(const NumParams &P, const F64Blk &b, int part,
-                                           const double (&acc)[kMaxR]) {
+                                           const double (&acc)[MR]) {
   const int lane = threadIdx.x & 31, mn = b.m * b.n;
   double *W = P.W + (int64_t)part * P.nelemC + b.off;
 #pragma unroll
-  for (int r = 0; r < kMaxR; ++r)
+  for (int r = 0; r < MR; ++r)
     if (lane + 32 * r < mn) W[lane + 32 * r] = acc[r];
 }
 
-template <bool STRIDED, bool SPLIT, class GetP>
+template <bool STRIDED, bool SPLIT, int MR, class GetP>
 __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, int64_t nitems,
                                             int slot_elems, unsigned long long *__restrict__ counter,
                                             int chunk, int ksplit, GetP get) {
@@ -594,9 +696,17 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
                     P.tb);
       cp_commit();
     }
-    double acc[kMaxR];
+    // the C_in block is read when the tile ends: bring its lines into L2 now
+    if (P.has_beta && b.cin >= 0 && ksplit <= 1 && lane * 16 < b.m * b.n)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(P.Cin + P.cin_off[b.cin] + b.cio + lane * 16));
+    double acc[MR], acct = 0.0;
 #pragma unroll
-    for (int r = 0; r < kMaxR; ++r) acc[r] = 0.0;
+    for (int r = 0; r < MR; ++r) acc[r] = 0.0;
+    const int bs = SPLIT ? b.s & 0xff : 1;  // whole-tile split, else the tail's
+    const int ts = bs > 1 ? 1 : b.s >> 8, mn = b.m * b.n;
+    const int F = ts > 1 ? mn >> 5 : (mn + 31) >> 5;
+    const LaneMap L = lane_map(b.n);
+    const TailMap T = ts > 1 ? tail_map(mn, b.n, ts) : TailMap{0, 0, 0};
     int g0 = 0;
     for (int e = 0; e < b.ne; ++e) {
       if (e - g0 == 32) {
@@ -628,16 +738,25 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
       cp_commit();
       cp_wait_prev();
       __syncwarp();
-      if (SPLIT && b.s > 1)
-        slot_product_split(P, slots + slot * slot_elems, b.m, b.n, k, b.s, acc);
-      else
-        slot_dispatch(P, slots + slot * slot_elems, b.m, b.n, k, acc);
+      const double *cur = slots + slot * slot_elems;
+      if (SPLIT && bs > 1) {
+        slot_product_split(P, cur, b.m, b.n, k, bs, acc);
+      } else {
+        slot_product_rt(P, cur, b.m, b.n, k, F, L, acc);
+        if (ts > 1) acct = slot_tail(P, cur, b.m, b.n, k, ts, T, acct);
+      }
       __syncwarp();
       slot ^= 1;
     }
     staged = b.ne > 0 && vn >= 0 && bn.ne > 0;
     // the slot of the tile's last job is free: the next tile's first job went to the other
-    if (SPLIT && b.s > 1 && b.ne > 0) split_reduce(slots + (slot ^ 1) * slot_elems, b.m * b.n, b.s, acc);
+    if (SPLIT && bs > 1 && b.ne > 0) split_reduce(slots + (slot ^ 1) * slot_elems, mn, bs, acc);
+    if (ts > 1) {
+      acct = tail_reduce(mn & 31, ts, T, acct);
+#pragma unroll
+      for (int r = 0; r < MR; ++r)
+        if (r == F) acc[r] = acct;
+    }
     if (ksplit > 1)
       store_part(P, b, (int)(v >> 32), acc);
     else
@@ -657,29 +776,29 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
 // SPLIT: some tile spreads its inner dimension over lane groups.  Each is a separate
 // instance so that plans without them run none of their code (a larger loop body costs
 // instruction-fetch stalls on every tile).
-template <bool STRIDED, bool SPLIT>
-__global__ void __launch_bounds__(32 * kStageWarps, 3)
+template <bool STRIDED, bool SPLIT, int MR>
+__global__ void __launch_bounds__(32 * kStageWarps, MR == kNarrowR ? 4 : 3)
     k_num_fp64_staged1(NumParams P, const int64_t *__restrict__ items, int64_t nitems,
                        int slot_elems, unsigned long long *counter, int chunk, int ksplit) {
-  staged_loop<STRIDED, SPLIT>(items, nitems, slot_elems, counter, chunk, ksplit,
+  staged_loop<STRIDED, SPLIT, MR>(items, nitems, slot_elems, counter, chunk, ksplit,
                               [&](int64_t) -> const NumParams & { return P; });
 }
 
-template <bool STRIDED, bool SPLIT>
-__global__ void __launch_bounds__(32 * kStageWarps, 3)
+template <bool STRIDED, bool SPLIT, int MR>
+__global__ void __launch_bounds__(32 * kStageWarps, MR == kNarrowR ? 4 : 3)
     k_num_fp64_staged(const NumParams *__restrict__ plans, const int64_t *__restrict__ items,
                       int64_t nitems, int slot_elems, unsigned long long *counter, int chunk,
                       int ksplit) {
-  staged_loop<STRIDED, SPLIT>(items, nitems, slot_elems, counter, chunk, 1,
+  staged_loop<STRIDED, SPLIT, MR>(items, nitems, slot_elems, counter, chunk, 1,
                               [&](int64_t pl) -> const NumParams & { return plans[pl]; });
 }
 
 // ---- schedule of the staged kernel (built with the plan) ----------------------------
 //
 // Work units ("tiles") are row ranges of C blocks: a block of m x n elements with
-// m n > 32 * kMaxR is cut into tiles of floor(32 kMaxR / n) rows.  A product whose
-// tile operands exceed a slot ((tile rows + n) k > kStageMax) is cut into panels of the
-// inner dimension of width floor(kStageMax / (tile rows + n)).  Each tile lists its
+// m n > T = 32 MR is cut into tiles of floor(T / n) rows.  A product whose
+// tile operands exceed a slot of S doubles ((tile rows + n) k > S) is cut into panels of
+// the inner dimension, as few as fit and of about equal width.  Each tile lists its
 // (product, panel) entries {first A element, first B element, panel width w, row
 // strides}, in the product order of the stacks; per (m, n) class the host passes the
 // tile rows, and per (class, k class) the panel width.
@@ -744,30 +863,27 @@ __global__ void k_f64_ent_count(int64_t nc, const int32_t *__restrict__ c_cls,
 constexpr int kMaxSplit = 16;
 constexpr int kSplitMinInner = 48;
 constexpr int kSplitLongInner = 128;
+constexpr unsigned long long kSplitGate = 100;
 
 __device__ int f64_split_of(int32_t *__restrict__ d, const int4 *__restrict__ ents, int smax,
-                            int slot_elems, long long &c1, long long &saved) {
+                            int tile, int slot_elems, long long c1,
+                            long long &saved) {
   const int mn = (d[3] & 0xfff) * ((d[3] >> 12) & 0xfff), ne = d[2];
   // s m n partial sums fit the accumulators and, for the final sums, one slot
-  smax = min(min(smax, kMaxSplit), min(kTile, slot_elems) / max(mn, 1));
+  smax = min(min(smax, kMaxSplit), min(tile, slot_elems) / max(mn, 1));
   const long long v1 = (mn + 31) / 32;
   int best = 1;
-  c1 = 0;
   saved = 0;
   // short tiles (most of a plan of small products) never split: one pass over the widths
   long long w1 = 0;
   for (int e = 0; e < ne; ++e) w1 += ents[(int64_t)d[1] + e].z;
-  if (w1 < kSplitMinInner || smax < 2) {
-    c1 = v1 * w1;
-    return 1;
-  }
+  if (w1 < kSplitMinInner || smax < 2) return 1;
   long long W[kMaxSplit + 1];
   for (int s = 1; s <= max(smax, 1); ++s) W[s] = 0;
   for (int e = 0; e < ne; ++e) {
     const int w = ents[(int64_t)d[1] + e].z;
     for (int s = 1; s <= max(smax, 1); ++s) W[s] += (w + s - 1) / s;
   }
-  c1 = v1 * W[1];
   long long cb = c1;
   for (int s = 2; s <= smax; ++s) {
     const long long c = (long long)((s * mn + 31) / 32) * W[s] + (s - 1) * v1;
@@ -781,6 +897,43 @@ __device__ int f64_split_of(int32_t *__restrict__ d, const int4 *__restrict__ en
   return best;
 }
 
+// Tail split of a tile (descriptor word 7, bits 8 and up): the t <= 32 / rem lane groups
+// over which its last partial round of rem outputs spreads the inner dimension, by FP64
+// warp instructions: sum of ceil(w / t) over the entries plus ceil(log2 t) adds, against
+// the unsplit sum of w.  The most groups that fit and half of them are compared (13 x 13,
+// one product of 13: 6 against 13; 5 x 13: 1 + 4 against 13), bounded like the tile's
+// inner split.
+struct TailCost {
+  int t[2];
+  long long c[2], w1;
+};
+
+__device__ __forceinline__ TailCost tail_cost(int mn, int smax) {
+  TailCost C;
+  const int rem = mn & 31;
+  C.t[0] = rem ? min(32 / rem, min(smax, kMaxSplit)) : 1;
+  C.t[1] = (C.t[0] + 1) >> 1;
+  C.w1 = 0;
+  for (int i = 0; i < 2; ++i) C.c[i] = 32 - __clz(C.t[i] - 1);  // ceil(log2 t)
+  return C;
+}
+
+__device__ __forceinline__ void tail_add(TailCost &C, int w) {
+  C.w1 += w;
+  C.c[0] += (w + C.t[0] - 1) / C.t[0];
+  C.c[1] += (w + C.t[1] - 1) / C.t[1];
+}
+
+// FP64 instructions of the unsplit tile
+__device__ __forceinline__ long long tail_total(const TailCost &C, int mn) {
+  return (mn >> 5) * C.w1 + ((mn & 31) ? min(C.w1, min(C.c[0], C.c[1])) : 0);
+}
+
+__device__ __forceinline__ int tail_of(const TailCost &C) {
+  const int i = C.c[1] < C.c[0] ? 1 : 0;
+  return C.t[i] > 1 && C.c[i] < C.w1 ? C.t[i] : 1;
+}
+
 // descriptors and entries of every tile of C block c, each tile's cost key
 // (63 - floor(log2(flops)): a stable partition on it lists costly tiles first) and its
 // inner split, with its FP64 instruction counts added to c1_sum / saved_sum
@@ -791,7 +944,7 @@ __device__ __forceinline__ void f64_tiles_of(
     const int32_t *__restrict__ c_cin, const int64_t *__restrict__ tbeg,
     const int64_t *__restrict__ ebeg, const SchedTabs &S, int32_t *__restrict__ desc,
     int4 *__restrict__ ents, int32_t *__restrict__ key, const int32_t *__restrict__ cls_smax,
-    int slot_elems, long long &c1_sum, long long &saved_sum) {
+    int tile_max, int slot_elems, long long &c1_sum, long long &saved_sum) {
   const int cls = c_cls[c];
   const int m = S.cls_m[cls], n = S.cls_n[cls], tr = S.tile_rows[cls];
   const int nt = (m + tr - 1) / tr;
@@ -800,7 +953,7 @@ __device__ __forceinline__ void f64_tiles_of(
     const int p0 = t * tr, mt = min(tr, m - p0);
     int64_t q = ebeg[tile];
     unsigned long long flops = 0;
-    long long w1 = 0;  // the tile's inner elements (sum of its entries' panel widths)
+    TailCost tc = tail_cost(mt * n, cls_smax[cls]);
     for (int kc = 0; kc < S.Dk; ++kc) {
       const int len = run_len[c * S.Dk + kc];
       if (len == 0) continue;
@@ -820,7 +973,7 @@ __device__ __forceinline__ void f64_tiles_of(
             for (int l0 = 0; l0 < k; l0 += ws) {
               const int b = s_b[e] + (S.tb ? l0 : l0 * n);
               ents[q++] = make_int4((int)(ab + (int64_t)(l0 / ki) * m * ki), b, min(ws, k - l0), st);
-              w1 += min(ws, k - l0);
+              tail_add(tc, min(ws, k - l0));
             }
           } else {
             for (int l0 = 0; l0 < k; l0 += ki)
@@ -828,7 +981,7 @@ __device__ __forceinline__ void f64_tiles_of(
                 const int b = s_b[e] + (S.tb ? l0 + c0 : (l0 + c0) * n);
                 ents[q++] = make_int4((int)(ab + (int64_t)(l0 / ki) * m * ki + c0), b,
                                       min(w, ki - c0), st);
-                w1 += min(w, ki - c0);
+                tail_add(tc, min(w, ki - c0));
               }
           }
           continue;
@@ -838,7 +991,7 @@ __device__ __forceinline__ void f64_tiles_of(
           const int a = s_a[e] + (S.ta ? l0 * m + p0 : p0 * k + l0);
           const int b = s_b[e] + (S.tb ? l0 : l0 * n);
           ents[q++] = make_int4(a, b, wl, strides);
-          w1 += wl;
+          tail_add(tc, wl);
         }
       }
       flops += (unsigned long long)len * mt * n * k;
@@ -849,17 +1002,17 @@ __device__ __forceinline__ void f64_tiles_of(
     dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)ebeg[tile],
                       (int32_t)(q - ebeg[tile]), mt | (n << 12));
     key[tile] = __clzll(flops + 1ull);
+    const long long w1 = tc.w1;  // the tile's inner elements
     // a short tile never splits (the test f64_split_of starts with), decided here
     // without reading its entries back
     const int mn = mt * n;
-    const int smax = min(min(cls_smax[cls], kMaxSplit), min(kTile, slot_elems) / max(mn, 1));
-    long long c1, saved = 0;
+    const int smax = min(min(cls_smax[cls], kMaxSplit), min(tile_max, slot_elems) / max(mn, 1));
+    const long long c1 = tail_total(tc, mn);
+    long long saved = 0;
     int split = 1;
-    if (w1 < kSplitMinInner || smax < 2)
-      c1 = (long long)((mn + 31) / 32) * w1;
-    else
-      split = f64_split_of(d, ents, cls_smax[cls], slot_elems, c1, saved);
-    dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, split);
+    if (w1 >= kSplitMinInner && smax >= 2)
+      split = f64_split_of(d, ents, cls_smax[cls], tile_max, slot_elems, c1, saved);
+    dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, f64_split_word(split, tail_of(tc)));
     c1_sum += c1;
     saved_sum += saved;
   }
@@ -873,11 +1026,11 @@ __global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
                             const int64_t *__restrict__ tbeg, const int64_t *__restrict__ ebeg,
                             SchedTabs S, int32_t *__restrict__ desc, int4 *__restrict__ ents,
                             int32_t *__restrict__ key, const int32_t *__restrict__ cls_smax,
-                            int slot_elems, unsigned long long *__restrict__ sums) {
+                            int tile_max, int slot_elems, unsigned long long *__restrict__ sums) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   long long c1_sum = 0, saved_sum = 0;
   if (c < nc) f64_tiles_of(c, c_cls, run_start, run_len, s_a, s_b, c_off, c_cin, tbeg, ebeg, S,
-                           desc, ents, key, cls_smax, slot_elems, c1_sum, saved_sum);
+                           desc, ents, key, cls_smax, tile_max, slot_elems, c1_sum, saved_sum);
   for (int o = 16; o > 0; o >>= 1) {
     c1_sum += __shfl_down_sync(0xffffffffu, c1_sum, o);
     saved_sum += __shfl_down_sync(0xffffffffu, saved_sum, o);
@@ -891,13 +1044,18 @@ __global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
 // sums[0] += unsplit FP64 instruction counts, sums[1] += savings of the chosen splits
 __global__ void k_f64_split(int64_t ntiles, const int4 *__restrict__ ents,
                             const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_smax,
-                            int slot_elems, int32_t *__restrict__ desc,
+                            int tile_max, int slot_elems, int32_t *__restrict__ desc,
                             unsigned long long *__restrict__ sums) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   long long c1 = 0, saved = 0;
   if (t < ntiles) {
     int32_t *d = desc + t * kF64Desc;
-    d[7] = f64_split_of(d, ents, cls_smax[c_cls[d[6]]], slot_elems, c1, saved);
+    const int smax = cls_smax[c_cls[d[6]]];
+    const int mn = (d[3] & 0xfff) * ((d[3] >> 12) & 0xfff);
+    TailCost tc = tail_cost(mn, smax);
+    for (int e = 0; e < d[2]; ++e) tail_add(tc, ents[(int64_t)d[1] + e].z);
+    c1 = tail_total(tc, mn);
+    d[7] = f64_split_word(f64_split_of(d, ents, smax, tile_max, slot_elems, c1, saved), tail_of(tc));
   }
   for (int o = 16; o > 0; o >>= 1) {
     c1 += __shfl_down_sync(0xffffffffu, c1, o);
@@ -911,7 +1069,7 @@ __global__ void k_f64_split(int64_t ntiles, const int4 *__restrict__ ents,
 
 __global__ void k_f64_nosplit(int64_t ntiles, int32_t *__restrict__ desc) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < ntiles) desc[t * kF64Desc + 7] = 1;
+  if (t < ntiles) desc[t * kF64Desc + 7] = f64_split_word(1, desc[t * kF64Desc + 7] >> 8);
 }
 
 __global__ void k_plan_items(int64_t nc, int64_t base, int64_t *__restrict__ item) {
@@ -1054,20 +1212,30 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   if (nc == 0 || p->T == 0) return false;
   const int32_t ncls = p->Dm * p->Dn, Dk = p->Dk;
   std::vector<int32_t> tile_rows((size_t)ncls, 1), wpanel((size_t)ncls * Dk, 1);
+  // the wide shape: rows of C, or whole C blocks of a slab-read operand, above a narrow tile
+  const bool slab_wanted = !p->a_slab_kin.empty() && !p->ta && p->a_slab_toff;
+  bool wide = false;
   for (int32_t c = 0; c < ncls; ++c) {
     if (p->h_class_ptr[c + 1] == p->h_class_ptr[c]) continue;
     const int64_t m = p->m_vals[c / p->Dn], n = p->n_vals[c % p->Dn];
-    if (m >= 4096 || n >= 4096 || n > kTile) return false;
-    const int64_t tr = m * n <= kTile ? m : kTile / n;
-    if (tr + n > kStageMax) return false;
+    wide = wide || n > 32 * kNarrowR ||
+           (slab_wanted && m * n > 32 * kNarrowR && m * n <= 32 * kWideR);
+  }
+  const int tile = 32 * (wide ? kWideR : kNarrowR), slot_max = wide ? kWideSlot : kNarrowSlot;
+  for (int32_t c = 0; c < ncls; ++c) {
+    if (p->h_class_ptr[c + 1] == p->h_class_ptr[c]) continue;
+    const int64_t m = p->m_vals[c / p->Dn], n = p->n_vals[c % p->Dn];
+    if (m >= 4096 || n >= 4096 || n > tile) return false;
+    const int64_t tr = m * n <= tile ? m : tile / n;
+    if (tr + n > slot_max) return false;
     tile_rows[(size_t)c] = (int32_t)tr;
   }
-  bool strided = false;
+  bool strided = false, tiled = false;
   for (int32_t c = 0; c < ncls; ++c)
     if (p->h_class_ptr[c + 1] > p->h_class_ptr[c] && tile_rows[(size_t)c] < p->m_vals[c / p->Dn])
-      strided = true;
+      (p->ta ? strided : tiled) = true;
   // slab reading of A: whole C blocks only (a slab holds all m rows), op(A) = A
-  const bool slab = !p->a_slab_kin.empty() && !strided && !p->ta && p->a_slab_toff;
+  const bool slab = slab_wanted && !strided && !tiled;
   if (slab) strided = true;
   int64_t slot = 1;
   for (int32_t b = 0; b < p->nb_all; ++b) {
@@ -1075,7 +1243,10 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
     const int32_t kc = b % Dk, ncl = (b / Dk) % p->Dn, mc = b / (Dk * p->Dn);
     const int32_t cls = mc * p->Dn + ncl;
     const int64_t n = p->n_vals[ncl], k = p->k_vals[kc], tr = tile_rows[(size_t)cls];
-    const int64_t w = (tr + n) * k <= kStageMax ? k : kStageMax / (tr + n);
+    // panels of about equal width (a narrow last one would cost a whole job); of whole
+    // slabs when read in place
+    const int64_t wmax = slot_max / (tr + n), np = (k + wmax - 1) / wmax;
+    const int64_t w = k <= wmax ? k : slab ? wmax : (k + np - 1) / np;
     wpanel[(size_t)cls * Dk + kc] = (int32_t)w;
     if (w < k) strided = true;
     slot = std::max(slot, (tr + n) * w);
@@ -1136,7 +1307,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   p->tkeys = ar.alloc_n<int32_t>((size_t)ntiles);
   k_f64_tiles<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->run_start, p->run_len, p->s_a,
                                             p->s_b, p->C->off, p->c_cin, tbeg, ebeg, S, p->fdesc,
-                                            p->fents, p->tkeys, d_smax, (int)slot, d_sums);
+                                            p->fents, p->tkeys, d_smax, tile, (int)slot, d_sums);
   BST_CHECK_LAUNCH();
   // tiles by decreasing cost
   int64_t *it0 = scratch.alloc_n<int64_t>((size_t)ntiles);
@@ -1154,6 +1325,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   p->n_tiles = ntiles;
   p->stage_elems = (int32_t)slot;
   p->stage_strided = strided;
+  p->stage_wide = wide;
   p->a_slab = slab;
   apply_split_gate(p, sums, s);
   return true;
@@ -1171,11 +1343,11 @@ static std::vector<int32_t> class_split_bounds(const bst_plan *p) {
   return smax;
 }
 
-// The plan runs the split instance only when the chosen splits save at least 1/25 of all
+// The plan runs the split instance only when the chosen splits save at least 1 % of all
 // its FP64 instructions (a safeguard: a longer loop body once cost every tile a few per
 // cent); otherwise every tile is set back to s = 1.
 static void apply_split_gate(bst_plan *p, const unsigned long long sums[2], cudaStream_t s) {
-  p->stage_split = sums[1] > 0 && 25 * sums[1] >= sums[0];
+  p->stage_split = sums[1] > 0 && kSplitGate * sums[1] >= sums[0];
   if (!p->stage_split && sums[1] > 0) {  // with no saving every tile already has s = 1
     k_f64_nosplit<<<nblk(p->n_tiles, 256), 256, 0, s>>>(p->n_tiles, p->fdesc);
     BST_CHECK_LAUNCH();
@@ -1205,6 +1377,7 @@ void refresh_f64_split(bst_plan *p, cudaStream_t s) {
   unsigned long long *d_sums = scratch.alloc_n<unsigned long long>(2);
   BST_CUDA(cudaMemsetAsync(d_sums, 0, 2 * sizeof(unsigned long long), s));
   k_f64_split<<<nblk(p->n_tiles, 128), 128, 0, s>>>(p->n_tiles, p->fents, p->c_cls, d_smax,
+                                                   32 * (p->stage_wide ? kWideR : kNarrowR),
                                                    p->stage_elems, p->fdesc, d_sums);
   BST_CHECK_LAUNCH();
   unsigned long long sums[2] = {0, 0};
@@ -1249,8 +1422,9 @@ void build_plan_tile_items(bst_plan *p, int64_t base, int64_t *items, int32_t *k
 // resident CTAs per SM of a staged kernel instance for a slot size; raises its dynamic
 // shared-memory limit on first use
 template <class K>
-static int staged_ctas_per_sm(K kernel, bool &attr_set, int slot_elems, size_t &smem) {
-  const size_t max_smem = sizeof(double) * 2 * kStageMax * kStageWarps;
+static int staged_ctas_per_sm(K kernel, bool &attr_set, int max_slot, int slot_elems,
+                              size_t &smem) {
+  const size_t max_smem = sizeof(double) * 2 * max_slot * kStageWarps;
   if (!attr_set) {
     BST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)max_smem));
@@ -1267,12 +1441,12 @@ static int staged_ctas_per_sm(K kernel, bool &attr_set, int slot_elems, size_t &
 // items (1 .. 32 items): one counter request per chunk, fine enough that the last
 // chunks are small.  The counter is cleared on the launch's stream.
 template <class K, class Arg>
-static void staged_launch(K kernel, bool &attr_set, Arg params, const int64_t *items,
+static void staged_launch(K kernel, bool &attr_set, int max_slot, Arg params, const int64_t *items,
                           int64_t nitems, int slot_elems, int num_sms,
                           unsigned long long *counter, cudaStream_t s, int ksplit = 1) {
   BST_REQUIRE(counter, BST_ERR_STATE, "staged kernel without a work counter");
   size_t smem = 0;
-  const int per = staged_ctas_per_sm(kernel, attr_set, slot_elems, smem);
+  const int per = staged_ctas_per_sm(kernel, attr_set, max_slot, slot_elems, smem);
   const int64_t full = (int64_t)per * num_sms * kStageWarps;
   const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, nitems / (64 * full)));
   const int64_t nchunks = (nitems + chunk - 1) / chunk;
@@ -1284,19 +1458,28 @@ static void staged_launch(K kernel, bool &attr_set, Arg params, const int64_t *i
   BST_CHECK_LAUNCH();
 }
 
-static bool g_attr[2][4] = {};  // [batch, single plan][strided | split << 1]
+static bool g_attr[2][5] = {};  // [batch, single plan][instance]
+
+// instance of the staged kernel: strided | split << 1, or 4 for the wide shape
+static int staged_instance(bool strided, bool split, bool wide) {
+  return wide ? 4 : (strided ? 1 : 0) | (split ? 2 : 0);
+}
 
 void launch_fp64_staged(const void *params, const int64_t *items, int64_t nitems,
-                        int slot_elems, bool strided, bool split, int num_sms,
+                        int slot_elems, bool strided, bool split, bool wide, int num_sms,
                         unsigned long long *counter, cudaStream_t s) {
   if (nitems == 0) return;
   const NumParams *P = static_cast<const NumParams *>(params);
-  const int v = (strided ? 1 : 0) | (split ? 2 : 0);
+  const int v = staged_instance(strided, split, wide);
+  auto go = [&](auto kernel, int max_slot) {
+    staged_launch(kernel, g_attr[0][v], max_slot, P, items, nitems, slot_elems, num_sms, counter, s);
+  };
   switch (v) {
-    case 0: staged_launch(k_num_fp64_staged<false, false>, g_attr[0][v], P, items, nitems, slot_elems, num_sms, counter, s); break;
-    case 1: staged_launch(k_num_fp64_staged<true, false>, g_attr[0][v], P, items, nitems, slot_elems, num_sms, counter, s); break;
-    case 2: staged_launch(k_num_fp64_staged<false, true>, g_attr[0][v], P, items, nitems, slot_elems, num_sms, counter, s); break;
-    default: staged_launch(k_num_fp64_staged<true, true>, g_attr[0][v], P, items, nitems, slot_elems, num_sms, counter, s); break;
+    case 0: go(k_num_fp64_staged<false, false, kNarrowR>, kNarrowSlot); break;
+    case 1: go(k_num_fp64_staged<true, false, kNarrowR>, kNarrowSlot); break;
+    case 2: go(k_num_fp64_staged<false, true, kNarrowR>, kNarrowSlot); break;
+    case 3: go(k_num_fp64_staged<true, true, kNarrowR>, kNarrowSlot); break;
+    default: go(k_num_fp64_staged<true, true, kWideR>, kWideSlot); break;
   }
 }
 
@@ -1361,14 +1544,17 @@ void launch_direct_splitk(bst_plan *p, const NumParams &P, cudaStream_t s) {
 // The staged kernel over every tile (split = 1: into C), or over every (tile, K part)
 // into W followed by the fixed-order reduction of the parts (split > 1).
 static void staged_single(bst_plan *p, const NumParams &P, int split, cudaStream_t s) {
-  const int v = (p->stage_strided ? 1 : 0) | (p->stage_split ? 2 : 0);
-  const int ns = p->ctx->num_sms, se = p->stage_elems;
-  const int64_t nt = p->n_tiles * split;
+  const int v = staged_instance(p->stage_strided, p->stage_split, p->stage_wide);
+  auto go = [&](auto kernel, int max_slot) {
+    staged_launch(kernel, g_attr[1][v], max_slot, P, p->titems, p->n_tiles * split, p->stage_elems,
+                  p->ctx->num_sms, p->items_counter, s, split);
+  };
   switch (v) {
-    case 0: staged_launch(k_num_fp64_staged1<false, false>, g_attr[1][v], P, p->titems, nt, se, ns, p->items_counter, s, split); break;
-    case 1: staged_launch(k_num_fp64_staged1<true, false>, g_attr[1][v], P, p->titems, nt, se, ns, p->items_counter, s, split); break;
-    case 2: staged_launch(k_num_fp64_staged1<false, true>, g_attr[1][v], P, p->titems, nt, se, ns, p->items_counter, s, split); break;
-    default: staged_launch(k_num_fp64_staged1<true, true>, g_attr[1][v], P, p->titems, nt, se, ns, p->items_counter, s, split); break;
+    case 0: go(k_num_fp64_staged1<false, false, kNarrowR>, kNarrowSlot); break;
+    case 1: go(k_num_fp64_staged1<true, false, kNarrowR>, kNarrowSlot); break;
+    case 2: go(k_num_fp64_staged1<false, true, kNarrowR>, kNarrowSlot); break;
+    case 3: go(k_num_fp64_staged1<true, true, kNarrowR>, kNarrowSlot); break;
+    default: go(k_num_fp64_staged1<true, true, kWideR>, kWideSlot); break;
   }
   if (split > 1) {
     const int wpb = 8;
