@@ -417,6 +417,7 @@ int choose_split(const bst_plan *p, int num_sms);
 size_t num_params_bytes();
 void fill_num_params(bst_plan *p, const NumArgs &a, void *out, bool staged);
 void build_plan_items(bst_plan *p, int64_t base, int64_t *items, int32_t *keys, cudaStream_t s);
+void plan_items(int64_t n, int64_t *items, cudaStream_t s);  // 0 .. n - 1
 void sort_items(const int64_t *items, const int32_t *keys, int64_t n, int64_t *out, Arena &scratch,
                 cudaStream_t s);
 int persist_grid(int num_sms);
@@ -430,6 +431,18 @@ void build_plan_tile_items(bst_plan *p, int64_t base, int64_t *items, int32_t *k
 void launch_fp64_staged(const void *params, const int64_t *items, int64_t nitems,
                         int slot_elems, bool strided, bool split, bool wide, int num_sms,
                         unsigned long long *counter, cudaStream_t s);
+// A schedule of the staged kernel over output blocks that are not C's (the adjoint's):
+// tiles, their entries and whether they are parts of blocks or of products (tiled)
+struct TileLaunch {
+  const int64_t *items = nullptr;
+  int64_t nitems = 0;
+  const int32_t *desc = nullptr;
+  const int4 *ents = nullptr;
+  int slot = 0;
+  bool tx = false, ty = false, tiled = false;
+};
+void launch_fp64_tiles(const TileLaunch &t, const double *X, const double *Y, double *out,
+                       double alpha, int num_sms, unsigned long long *counter, cudaStream_t s);
 // persistent emulated-FP64 numeric (numeric_emu.cu)
 size_t emu_params_bytes();
 int64_t emu_item_count(bst_plan *p, cudaStream_t s);

@@ -26,6 +26,7 @@
 #include <cstring>
 
 #include "bst_internal.h"
+#include "fp64_tiles.h"
 
 namespace bst {
 
@@ -292,31 +293,16 @@ __global__ void __launch_bounds__(256, 2)
 // value is needed, so the atomic's latency is hidden too.  Which warp runs a tile does
 // not change its result: every tile is summed by one warp in its entry order.
 
-// Two shapes of the kernel (MR accumulators per lane, tiles up to 32 MR elements):
-// * MR = 10, slots of at most 896 doubles: four 4-warp CTAs per SM (at most 128
-//   registers, 4 x (2 x 4 x 896 x 8 B + 1 KB) <= 228 KB).  The FP64 pipe takes 16 SM
-//   cycles per warp FMA and idles when no resident warp has one ready: with 17
-//   accumulators and 1184-double slots 12 warps fitted and the pipe was 94 % busy on the
-//   banded product (20.8 ms); 16 warps keep it 96 % busy (18.9 ms with the tail split).  A
-//   23 x 23 block is then cut into tiles of 13 and 10 rows.
-// * MR = 17, slots of 1184 doubles, three CTAs per SM ("wide"): for plans with rows of C
-//   of 321 to 544 elements, and for contractions read in place as slabs (which need whole
-//   C blocks) with blocks of 321 to 544 elements.
-constexpr int kNarrowR = 10, kWideR = 17;
-constexpr int kNarrowSlot = 896, kWideSlot = 1184;
-constexpr int kStageWarps = 4;    // warps per CTA
-constexpr int kF64Desc = kF64DescWords;
-
 // Work unit: a row tile of a C block (the whole block when it has at most 32 MR
 // elements).  Descriptor: 0 element offset of the tile in C, 1 first entry, 2 entry
 // count, 3 tile rows m | n << 12, 4 C_in block (-1: none), 5 element offset of the tile
 // inside the C_in block, 6 C block, 7 inner split s (>= 1) | tail split << 8 (>= 1, taken
-// when s = 1; see slot_tail).
+// when s = 1; see slot_tail).  In a schedule of rectangular tiles (the adjoint's, TILED
+// below) the entries are those of the whole output block, shared by its tiles: word 4 holds
+// the tile's first row and column p0 | q0 << 16, word 5 the row length of the output block.
 struct F64Blk {
   int off, eb, ne, m, n, cin, cio, s;
 };
-__device__ __forceinline__ int f64_split_word(int s, int tail) { return s | (tail << 8); }
-
 __device__ __forceinline__ F64Blk f64_blk(int dw) {
   F64Blk b;
   b.off = __shfl_sync(0xffffffffu, dw, 0);
@@ -586,6 +572,20 @@ __device__ __forceinline__ void split_reduce(double *red, int mn, int s, double 
   __syncwarp();
 }
 
+// a rectangular tile of an output block with rows of b.cio elements: alpha * acc
+template <int MR>
+__device__ __forceinline__ void store_tile(const NumParams &P, const F64Blk &b, const LaneMap &L,
+                                           const double (&acc)[MR]) {
+  const int lane = threadIdx.x & 31, mn = b.m * b.n;
+  double *C = P.C + b.off;
+  int p = L.p, q = L.q;
+#pragma unroll
+  for (int r = 0; r < MR; ++r) {
+    if (lane + 32 * r < mn) C[p * b.cio + q] = P.alpha_one ? acc[r] : P.alpha * acc[r];
+    lane_step(L, b.n, p, q);
+  }
+}
+
 // C = alpha * acc + beta * C_in for one C block (C_in unread when beta == 0)
 template <int MR>
 __device__ __forceinline__ void store_block(const NumParams &P, const F64Blk &b,
@@ -624,7 +624,7 @@ __device__ __forceinline__ void store_part(const NumParams &P, const F64Blk &b, 
     if (lane + 32 * r < mn) W[lane + 32 * r] = acc[r];
 }
 
-template <bool STRIDED, bool SPLIT, int MR, class GetP>
+template <bool STRIDED, bool SPLIT, int MR, bool TILED = false, class GetP>
 __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, int64_t nitems,
                                             int slot_elems, unsigned long long *__restrict__ counter,
                                             int chunk, int ksplit, GetP get) {
@@ -675,6 +675,18 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
     return (v >= 0 && g0 + lane < b.ne) ? get(v >> 32).fents[(int64_t)b.eb + g0 + lane]
                                         : make_int4(0, 0, 0, 0);
   };
+  // the operands of entry j of `src` for a tile of block b into `dst`
+  auto stage = [&](double *dst, const NumParams &P, const F64Blk &b, const int4 &src, int j) {
+    int64_t x = __shfl_sync(0xffffffffu, src.x, j), y = __shfl_sync(0xffffffffu, src.y, j);
+    const int strides = __shfl_sync(0xffffffffu, src.w, j);
+    if (TILED) {  // the entry locates the whole block: go to the tile's first row and column
+      const int p0 = b.cin & 0xffff, q0 = b.cin >> 16;
+      x += P.ta ? p0 : p0 * (strides & 0xffff);
+      y += P.tb ? q0 * (strides >> 16) : q0;
+    }
+    stage_product<STRIDED>(dst, P.A + x, P.B + y, b.m, b.n, __shfl_sync(0xffffffffu, src.z, j),
+                           strides, P.ta, P.tb);
+  };
   int64_t v = item(next_pos());
   if (v < 0) return;
   int64_t vn = item(next_pos());
@@ -690,14 +702,11 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
     const int64_t vnn = vn >= 0 ? item(next_pos()) : -1;
     const int dwnn = word(vnn);
     if (!staged && b.ne > 0) {
-      stage_product<STRIDED>(slots + slot * slot_elems, P.A + __shfl_sync(0xffffffffu, ent.x, 0),
-                    P.B + __shfl_sync(0xffffffffu, ent.y, 0), b.m, b.n,
-                    __shfl_sync(0xffffffffu, ent.z, 0), __shfl_sync(0xffffffffu, ent.w, 0), P.ta,
-                    P.tb);
+      stage(slots + slot * slot_elems, P, b, ent, 0);
       cp_commit();
     }
     // the C_in block is read when the tile ends: bring its lines into L2 now
-    if (P.has_beta && b.cin >= 0 && ksplit <= 1 && lane * 16 < b.m * b.n)
+    if (!TILED && P.has_beta && b.cin >= 0 && ksplit <= 1 && lane * 16 < b.m * b.n)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(P.Cin + P.cin_off[b.cin] + b.cio + lane * 16));
     double acc[MR], acct = 0.0;
 #pragma unroll
@@ -724,16 +733,9 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
           src = group(v, b, g0 + 32);
           j = 0;
         }
-        stage_product<STRIDED>(nxt, P.A + __shfl_sync(0xffffffffu, src.x, j),
-                      P.B + __shfl_sync(0xffffffffu, src.y, j), b.m, b.n,
-                      __shfl_sync(0xffffffffu, src.z, j), __shfl_sync(0xffffffffu, src.w, j), P.ta,
-                      P.tb);
+        stage(nxt, P, b, src, j);
       } else if (vn >= 0 && bn.ne > 0) {
-        const NumParams &Pn = get(vn >> 32);
-        stage_product<STRIDED>(nxt, Pn.A + __shfl_sync(0xffffffffu, entn.x, 0),
-                      Pn.B + __shfl_sync(0xffffffffu, entn.y, 0), bn.m, bn.n,
-                      __shfl_sync(0xffffffffu, entn.z, 0), __shfl_sync(0xffffffffu, entn.w, 0),
-                      Pn.ta, Pn.tb);
+        stage(nxt, get(vn >> 32), bn, entn, 0);
       }
       cp_commit();
       cp_wait_prev();
@@ -757,7 +759,9 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
       for (int r = 0; r < MR; ++r)
         if (r == F) acc[r] = acct;
     }
-    if (ksplit > 1)
+    if (TILED)
+      store_tile(P, b, L, acc);
+    else if (ksplit > 1)
       store_part(P, b, (int)(v >> 32), acc);
     else
       store_block(P, b, acc);
@@ -775,13 +779,13 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
 // STRIDED: the plan has row tiles or inner panels (staging copies strided rows);
 // SPLIT: some tile spreads its inner dimension over lane groups.  Each is a separate
 // instance so that plans without them run none of their code (a larger loop body costs
-// instruction-fetch stalls on every tile).
-template <bool STRIDED, bool SPLIT, int MR>
+// instruction-fetch stalls on every tile).  TILED: rectangular tiles of output blocks.
+template <bool STRIDED, bool SPLIT, int MR, bool TILED = false>
 __global__ void __launch_bounds__(32 * kStageWarps, MR == kNarrowR ? 4 : 3)
     k_num_fp64_staged1(NumParams P, const int64_t *__restrict__ items, int64_t nitems,
                        int slot_elems, unsigned long long *counter, int chunk, int ksplit) {
-  staged_loop<STRIDED, SPLIT, MR>(items, nitems, slot_elems, counter, chunk, ksplit,
-                              [&](int64_t) -> const NumParams & { return P; });
+  staged_loop<STRIDED, SPLIT, MR, TILED>(items, nitems, slot_elems, counter, chunk, ksplit,
+                                     [&](int64_t) -> const NumParams & { return P; });
 }
 
 template <bool STRIDED, bool SPLIT, int MR>
@@ -852,87 +856,7 @@ __global__ void k_f64_ent_count(int64_t nc, const int32_t *__restrict__ c_cls,
   for (int t = 0; t < nt; ++t) cnt[tbeg[c] + t] = s;
 }
 
-// Inner split of every tile (descriptor word 7): the s <= smax of the tile's class that
-// needs the fewest FP64 warp instructions -- ceil(s mt n / 32) for each of the
-// ceil(w / s) steps of a panel of width w, plus (s - 1) ceil(mt n / 32) adds for the
-// final sums -- when it saves anything on a tile with at least kSplitLongInner inner
-// elements in all, at least 1/8 of the unsplit count on one with kSplitMinInner or more,
-// else 1 (on short tiles the final sums cost more than the idle lanes).  The plan-wide
-// sums of the unsplit counts and of the savings decide whether the plan splits at all
-// (refresh_f64_split).
-constexpr int kMaxSplit = 16;
-constexpr int kSplitMinInner = 48;
-constexpr int kSplitLongInner = 128;
 constexpr unsigned long long kSplitGate = 100;
-
-__device__ int f64_split_of(int32_t *__restrict__ d, const int4 *__restrict__ ents, int smax,
-                            int tile, int slot_elems, long long c1,
-                            long long &saved) {
-  const int mn = (d[3] & 0xfff) * ((d[3] >> 12) & 0xfff), ne = d[2];
-  // s m n partial sums fit the accumulators and, for the final sums, one slot
-  smax = min(min(smax, kMaxSplit), min(tile, slot_elems) / max(mn, 1));
-  const long long v1 = (mn + 31) / 32;
-  int best = 1;
-  saved = 0;
-  // short tiles (most of a plan of small products) never split: one pass over the widths
-  long long w1 = 0;
-  for (int e = 0; e < ne; ++e) w1 += ents[(int64_t)d[1] + e].z;
-  if (w1 < kSplitMinInner || smax < 2) return 1;
-  long long W[kMaxSplit + 1];
-  for (int s = 1; s <= max(smax, 1); ++s) W[s] = 0;
-  for (int e = 0; e < ne; ++e) {
-    const int w = ents[(int64_t)d[1] + e].z;
-    for (int s = 1; s <= max(smax, 1); ++s) W[s] += (w + s - 1) / s;
-  }
-  long long cb = c1;
-  for (int s = 2; s <= smax; ++s) {
-    const long long c = (long long)((s * mn + 31) / 32) * W[s] + (s - 1) * v1;
-    if (c < cb) {
-      cb = c;
-      best = s;
-    }
-  }
-  if ((W[1] >= kSplitLongInner ? cb >= c1 : 8 * cb > 7 * c1) || W[1] < kSplitMinInner) best = 1;
-  if (best > 1) saved = c1 - cb;
-  return best;
-}
-
-// Tail split of a tile (descriptor word 7, bits 8 and up): the t <= 32 / rem lane groups
-// over which its last partial round of rem outputs spreads the inner dimension, by FP64
-// warp instructions: sum of ceil(w / t) over the entries plus ceil(log2 t) adds, against
-// the unsplit sum of w.  The most groups that fit and half of them are compared (13 x 13,
-// one product of 13: 6 against 13; 5 x 13: 1 + 4 against 13), bounded like the tile's
-// inner split.
-struct TailCost {
-  int t[2];
-  long long c[2], w1;
-};
-
-__device__ __forceinline__ TailCost tail_cost(int mn, int smax) {
-  TailCost C;
-  const int rem = mn & 31;
-  C.t[0] = rem ? min(32 / rem, min(smax, kMaxSplit)) : 1;
-  C.t[1] = (C.t[0] + 1) >> 1;
-  C.w1 = 0;
-  for (int i = 0; i < 2; ++i) C.c[i] = 32 - __clz(C.t[i] - 1);  // ceil(log2 t)
-  return C;
-}
-
-__device__ __forceinline__ void tail_add(TailCost &C, int w) {
-  C.w1 += w;
-  C.c[0] += (w + C.t[0] - 1) / C.t[0];
-  C.c[1] += (w + C.t[1] - 1) / C.t[1];
-}
-
-// FP64 instructions of the unsplit tile
-__device__ __forceinline__ long long tail_total(const TailCost &C, int mn) {
-  return (mn >> 5) * C.w1 + ((mn & 31) ? min(C.w1, min(C.c[0], C.c[1])) : 0);
-}
-
-__device__ __forceinline__ int tail_of(const TailCost &C) {
-  const int i = C.c[1] < C.c[0] ? 1 : 0;
-  return C.t[i] > 1 && C.c[i] < C.w1 ? C.t[i] : 1;
-}
 
 // descriptors and entries of every tile of C block c, each tile's cost key
 // (63 - floor(log2(flops)): a stable partition on it lists costly tiles first) and its
@@ -1182,6 +1106,12 @@ void build_plan_items(bst_plan *p, int64_t base, int64_t *items, int32_t *keys, 
                                                    p->cls_m, p->cls_n, keys);
     BST_CHECK_LAUNCH();
   }
+}
+
+void plan_items(int64_t n, int64_t *items, cudaStream_t s) {
+  if (n == 0) return;
+  k_plan_items<<<nblk(n, 256), 256, 0, s>>>(n, 0, items);
+  BST_CHECK_LAUNCH();
 }
 
 // items reordered by their keys (stable): costly C blocks first
@@ -1458,7 +1388,7 @@ static void staged_launch(K kernel, bool &attr_set, int max_slot, Arg params, co
   BST_CHECK_LAUNCH();
 }
 
-static bool g_attr[2][5] = {};  // [batch, single plan][instance]
+static bool g_attr[2][6] = {};  // [batch, single plan][instance]
 
 // instance of the staged kernel: strided | split << 1, or 4 for the wide shape
 static int staged_instance(bool strided, bool split, bool wide) {
@@ -1563,6 +1493,32 @@ static void staged_single(bst_plan *p, const NumParams &P, int split, cudaStream
                                                        p->C->csz);
     BST_CHECK_LAUNCH();
   }
+}
+
+// out = alpha X Y over the tiles of an output-block schedule (adjoint.cu); tx, ty: X, Y are
+// stored transposed
+void launch_fp64_tiles(const TileLaunch &t, const double *X, const double *Y, double *out,
+                       double alpha, int num_sms, unsigned long long *counter, cudaStream_t s) {
+  if (t.nitems == 0) return;
+  NumParams P{};
+  P.A = X;
+  P.B = Y;
+  P.C = out;
+  P.alpha = alpha;
+  P.alpha_one = alpha == 1.0;
+  P.split = 1;
+  P.ta = t.tx;
+  P.tb = t.ty;
+  P.fdesc = t.desc;
+  P.fents = t.ents;
+  auto go = [&](auto kernel, int v) {
+    staged_launch(kernel, g_attr[1][v], kNarrowSlot, P, t.items, t.nitems, t.slot, num_sms,
+                  counter, s);
+  };
+  if (t.tiled)
+    go(k_num_fp64_staged1<true, true, kNarrowR, true>, 5);
+  else
+    go(k_num_fp64_staged1<false, true, kNarrowR>, 2);
 }
 
 void execute_fp64(bst_plan *p, const NumArgs &a, int split, cudaStream_t s) {
