@@ -58,10 +58,7 @@ struct EmuState {
   int64_t *a_doff = nullptr, *b_doff = nullptr, *a_toff = nullptr, *b_toff = nullptr;
   int64_t *a_eoff = nullptr, *b_eoff = nullptr;
   int64_t a_dsize = 0, b_dsize = 0, a_tsize = 0, b_tsize = 0, a_esize = 0, b_esize = 0;
-  int64_t nwarps = 0;            // 3xTF32 warps (one per 16 x 16 tile)
   int64_t nitems_b = 0;          // BF16 work items (one per C block)
-  int64_t *wstart = nullptr;    // per (m,n) class: first warp, 16 x 16 tiles (3xTF32)
-  int32_t ncls = 0;
   // global start of every op(A) row block / op(B) column block, and the largest
   // exponent of every op(A) row / op(B) column over all blocks
   int64_t *a_rowstart = nullptr, *b_colstart = nullptr;
@@ -71,7 +68,10 @@ struct EmuState {
   __nv_bfloat16 *a_dig = nullptr, *b_dig = nullptr;
   float *a_tf = nullptr, *b_tf = nullptr;
   int32_t *a_exp = nullptr, *b_exp = nullptr;
-  bool dig_alloc = false, tf_alloc = false;
+  bool dig_alloc = false, tf_alloc = false, tf_lists = false;
+  // 3xTF32: C-major entries and C block descriptors (k_tf32_ents, k_tf32_desc)
+  int4 *tents = nullptr;
+  int32_t *tdesc = nullptr;
   // C-major stack entries of the BF16 kernel (int4 each) and where each C block's start
   int4 *ents = nullptr;
   int64_t *ebeg = nullptr;
@@ -96,12 +96,6 @@ __device__ __forceinline__ int exp_of(double x) {
   return ex == 0 ? kExpNone : ex - 1022;
 }
 
-// same for m16n8k8 TF32 (thread t holds k = t, t+4 -> positions 2t, 2t+1)
-__device__ __forceinline__ int perm8(int l) {
-  const int j = l & 7;
-  return (l & ~7) + 2 * (j & 3) + (j >> 2);
-}
-
 struct SideArgs {
   int64_t nblocks;
   const int32_t *row, *col, *rsz, *csz;  // stored block index and sizes
@@ -119,23 +113,8 @@ struct SideArgs {
   float *tf;
 };
 
-// decompose stored element e of block b into op coordinates: (r, l) for the A side
-// (op row r, inner l), (l, q) for the B side (inner l, op column q); `outer` is r or q
-__device__ __forceinline__ void op_coords(const SideArgs &S, int rs, int cs, int &outer,
-                                          int &inner) {
-  // stored element (rs, cs); op(X) element = (rs, cs) or (cs, rs)
-  const int opr = S.trans ? cs : rs, opc = S.trans ? rs : cs;
-  if (S.is_b) {
-    inner = opr;
-    outer = opc;
-  } else {
-    outer = opr;
-    inner = opc;
-  }
-}
-
-// Both side kernels run one warp per stored block; four lanes share one 16-wide chunk of
-// one op row (A side) or op column (B side) and lane t of the four takes the inner
+// The side kernels run one warp per stored block; in the digit kernels four lanes share one
+// 16-wide chunk of one op row (A side) or op column (B side) and lane t of the four takes the inner
 // indices 2t, 2t+1, 2t+8, 2t+9 of the chunk -- the four values that the digit layout
 // stores next to each other (positions 4t..4t+3).  Elements are read in the stored
 // block's layout: element (outer, inner) sits at outer * Cc + inner when the op keeps
@@ -249,26 +228,28 @@ __device__ __forceinline__ float to_tf32(float x) {
   return __uint_as_float(r);
 }
 
+// TF32 high and low parts of a block, chunks of 8 inner elements of an op row (column) in the
+// order the m16n8k8 fragments take them: lane t of four holds inner t and t + 4, so its 16
+// bytes are {high t, high t + 4, low t, low t + 4} and a fragment is one 16-byte load.  The
+// padding of the last chunk is written as zeros with it (no clearing pass).
 __global__ void k_tf32_split(SideArgs S) {
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, t = lane & 3;
   const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (b >= S.nblocks) return;
-  const int R = S.rsz[S.row[b]], Cc = S.csz[S.col[b]];
-  const int nouter = S.is_b ? (S.trans ? R : Cc) : (S.trans ? Cc : R);
-  const int ninner = S.is_b ? (S.trans ? Cc : R) : (S.trans ? R : Cc);
-  const int kp = (ninner + 7) & ~7;
-  const int64_t plane = (int64_t)nouter * kp;
-  const double *x = S.data + S.off[b];
-  float *t = S.tf + S.doff[b];
-  for (int e = lane; e < R * Cc; e += 32) {
-    int outer, inner;
-    op_coords(S, e / Cc, e % Cc, outer, inner);
-    const double v = x[e];
-    const float hi = to_tf32((float)v);
-    const float lo = to_tf32((float)(v - (double)hi));
-    const int64_t pos = (int64_t)outer * kp + perm8(inner);
-    t[pos] = hi;
-    t[plane + pos] = lo;
+  const SideBlock B = side_block(S, b);
+  const int nch = (B.ninner + 7) >> 3;
+  float4 *dst = reinterpret_cast<float4 *>(S.tf + S.doff[b]);
+  const int64_t total = (int64_t)B.nouter * nch;
+  for (int64_t q = lane >> 2; q < total; q += 8) {
+    const int outer = (int)(q / nch), l = (int)(q - (int64_t)outer * nch) * 8 + t;
+    float hi[2], lo[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const double v = side_value(B, outer, l + 4 * u);
+      hi[u] = to_tf32((float)v);
+      lo[u] = to_tf32((float)(v - (double)hi[u]));
+    }
+    dst[q * 4 + t] = make_float4(hi[0], hi[1], lo[0], lo[1]);
   }
 }
 
@@ -315,6 +296,41 @@ __global__ void k_emu_ents(int64_t nc, int32_t Dk, const int32_t *__restrict__ r
     for (int e = e0; e < e0 + len; ++e)
       ents[q++] = make_int4((int)(unsigned)(a_doff[s_ab[e]] >> 4),
                             (int)(unsigned)(b_doff[s_bb[e]] >> 4), nch, e);
+  }
+}
+
+constexpr int kTfCols = 3;  // 16 x 8 tiles side by side in a pass of the 3xTF32 kernel
+
+// 3xTF32: the C-major entry list (at ebeg[c] too), {A and B offsets / 16 floats, 8-wide
+// chunks of the inner size, 0}, and the C block descriptors: 0 element offset, 1 first
+// entry, 2 entry count, 3 C_in block (-1: none), 4 m, 5 n, 6 swap (tile rows run over the
+// C block's columns when that takes fewer passes, or as many of fewer 16 x 8 tiles)
+__global__ void k_tf32_ents(int64_t nc, int32_t Dk, const int32_t *__restrict__ run_start,
+                            const int32_t *__restrict__ run_len, const int32_t *__restrict__ kval,
+                            const int32_t *__restrict__ s_ab, const int32_t *__restrict__ s_bb,
+                            const int64_t *__restrict__ a_toff, const int64_t *__restrict__ b_toff,
+                            const int64_t *__restrict__ ebeg, const int64_t *__restrict__ c_off,
+                            const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_m,
+                            const int32_t *__restrict__ cls_n, const int32_t *__restrict__ c_cin,
+                            int4 *__restrict__ ents, int32_t *__restrict__ desc) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nc) return;
+  int64_t q = ebeg[c];
+  int4 *d = reinterpret_cast<int4 *>(desc + c * kDescWords);
+  const int m = cls_m[c_cls[c]], n = cls_n[c_cls[c]];
+  auto cost = [](int r, int c) {
+    const int64_t mt = (r + 15) / 16, nt = (c + 7) / 8;
+    return (mt * ((nt + kTfCols - 1) / kTfCols) << 32) + mt * nt;
+  };
+  d[0] = make_int4((int)c_off[c], (int)q, (int)(ebeg[c + 1] - q), c_cin[c]);
+  d[1] = make_int4(m, n, cost(n, m) < cost(m, n), 0);
+  for (int kc = 0; kc < Dk; ++kc) {
+    const int len = run_len[c * Dk + kc];
+    if (len == 0) continue;
+    const int e0 = run_start[c * Dk + kc], nch = (kval[kc] + 7) >> 3;
+    for (int e = e0; e < e0 + len; ++e)
+      ents[q++] = make_int4((int)(unsigned)(a_toff[s_ab[e]] >> 4),
+                            (int)(unsigned)(b_toff[s_bb[e]] >> 4), nch, 0);
   }
 }
 
@@ -397,55 +413,23 @@ struct EmuParams {
   const double *Cin;
   double *C;
   double alpha, beta;
-  int32_t Dk, ncls;
-  const int64_t *wstart;
-  int32_t tiles_n;  // N-tiles of 8 columns per warp (1 or 2)
+  int32_t Dk;
   int32_t alpha_one, has_beta;  // alpha == 1, beta != 0 (set on the host: FP64 compares
                                 // would occupy GB300's slow FP64 pipe in every tile)
   int32_t row_scale;  // 1: digits scaled per whole op row / column (shared by all products)
   const int64_t *a_rowstart, *b_colstart;
   const int32_t *row_exp, *col_exp;
-  const int32_t *class_ptr, *task_c, *cls_m, *cls_n, *kval;
+  const int32_t *cls_m, *cls_n, *kval;
   const int32_t *c_row, *c_col, *c_cin, *c_cls;
   const int64_t *c_off, *cin_off;
   const int32_t *run_start, *run_len, *s_ab, *s_bb;
-  const int32_t *desc;  // BF16 kernel: C block descriptors (kDescWords each)
-  const int4 *ents;     // BF16 kernel: C-major entries
+  const int32_t *desc;  // C block descriptors (kDescWords each)
+  const int4 *ents;     // C-major entries
   const int64_t *a_doff, *b_doff, *a_eoff, *b_eoff;
   const __nv_bfloat16 *a_dig, *b_dig;
   const float *a_tf, *b_tf;
   const int32_t *a_exp, *b_exp;
 };
-
-struct WarpTask {
-  int c, m, n, mt, ng, ntn;
-  int sw = 0;  // 1: tile rows run over the C block's columns (C^T = op(B)^T op(A)^T)
-};
-
-__device__ __forceinline__ WarpTask find_task(const EmuParams &P, int64_t gw) {
-  // class of this warp: last class whose start <= gw (classes with no warps are skipped)
-  int lo = 0, hi = P.ncls;  // wstart has ncls + 1 entries, wstart[ncls] = total
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (P.wstart[mid] <= gw)
-      lo = mid;
-    else
-      hi = mid;
-  }
-  WarpTask w;
-  const int cls = lo;
-  w.m = P.cls_m[cls];
-  w.n = P.cls_n[cls];
-  const int MT = (w.m + 15) >> 4, NT = (w.n + 7) >> 3, NG = (NT + P.tiles_n - 1) / P.tiles_n;
-  // warps of one class number below 2^31 (a class holds < 2^31 C blocks x a few tiles)
-  const unsigned local = (unsigned)(gw - P.wstart[cls]), per = (unsigned)(MT * NG);
-  const unsigned task = local / per, sub = local - task * per;
-  w.mt = (int)(sub / (unsigned)NG);
-  w.ng = (int)(sub - (unsigned)w.mt * (unsigned)NG);
-  w.ntn = min(P.tiles_n, NT - P.tiles_n * w.ng);
-  w.c = P.task_c[P.class_ptr[cls] + (int)task];
-  return w;
-}
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                          uint32_t b1) {
@@ -467,13 +451,6 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1
 
 __device__ __forceinline__ uint2 ld8(const void *p) {
   return __ldg(reinterpret_cast<const uint2 *>(p));
-}
-
-// element (row, col) of this warp's tile owned by accumulator slot h of N-tile nt
-__device__ __forceinline__ void slot_rc(const WarpTask &w, int nt, int h, int &r, int &c) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  r = w.mt * 16 + g + (h >= 2 ? 8 : 0);
-  c = (2 * w.ng + nt) * 8 + 2 * t + (h & 1);
 }
 
 // ---- the BF16 slice kernel: one warp per C block -----------------------------------
@@ -875,13 +852,14 @@ static_assert(kChunk * kDescWords == 32, "one descriptor word per lane");
 // take the pipelined loop
 constexpr double kPipeMinInner = 64.0;
 
-template <int ROWS, class GetP>
+template <class GetP, class Run>
 __device__ __forceinline__ void emu_persist(const int64_t *__restrict__ items, int64_t nitems,
-                                            unsigned long long *counter, GetP get) {
+                                            unsigned long long *counter, GetP get, Run run,
+                                            int take = kChunk) {
   const int lane = threadIdx.x & 31;
   // lane 0 issues the atomic; the result is shuffled to the warp only when needed
   auto request = [&]() -> unsigned long long {
-    return lane == 0 ? atomicAdd(counter, (unsigned long long)kChunk) : 0ull;
+    return lane == 0 ? atomicAdd(counter, (unsigned long long)take) : 0ull;
   };
   auto item = [&](int64_t i) -> int64_t { return i < nitems ? (items ? items[i] : i) : -1; };
   // lane l: word l % 8 of the descriptor of item c0 + l / 8
@@ -896,10 +874,10 @@ __device__ __forceinline__ void emu_persist(const int64_t *__restrict__ items, i
     const unsigned long long req = request();  // the next chunk, in flight during block 0
     int64_t cn = 0;
     int dwn = 0;
-    for (int q = 0; q < kChunk && c0 + q < nitems; ++q) {
+    for (int q = 0; q < take && c0 + q < nitems; ++q) {
       const int64_t v = item(c0 + q);
       const int w = __shfl_sync(kFull, dw, q * kDescWords + (lane & (kDescWords - 1)));
-      emu_block<ROWS>(get(v >> 32), emu_blk(w));
+      run(get(v >> 32), w);
       if (q == 0) {
         cn = (int64_t)__shfl_sync(kFull, req, 0);
         dwn = words(cn);
@@ -914,92 +892,210 @@ __device__ __forceinline__ void emu_persist(const int64_t *__restrict__ items, i
 template <int ROWS>
 __global__ void __launch_bounds__(256, 2)
     k_num_emu_bf16_persist1(EmuParams P, int64_t nitems, unsigned long long *counter) {
-  emu_persist<ROWS>(nullptr, nitems, counter, [&](int64_t) -> const EmuParams & { return P; });
+  emu_persist(
+      nullptr, nitems, counter, [&](int64_t) -> const EmuParams & { return P; },
+      [](const EmuParams &Q, int w) { emu_block<ROWS>(Q, emu_blk(w)); });
 }
 
 template <int ROWS>
 __global__ void __launch_bounds__(256, 2)
     k_num_emu_bf16_persist(const EmuParams *__restrict__ plans, const int64_t *__restrict__ items,
                            int64_t nitems, unsigned long long *counter) {
-  emu_persist<ROWS>(items, nitems, counter,
-                    [&](int64_t pl) -> const EmuParams & { return plans[pl]; });
+  emu_persist(
+      items, nitems, counter, [&](int64_t pl) -> const EmuParams & { return plans[pl]; },
+      [](const EmuParams &Q, int w) { emu_block<ROWS>(Q, emu_blk(w)); });
 }
 
-__global__ void __launch_bounds__(256) k_num_tf32x3(EmuParams P, int64_t nwarps) {
-  const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (gw >= nwarps) return;
-  const WarpTask w = find_task(P, gw);
+// ---- the 3xTF32 kernel: one warp per C block ----------------------------------------
+//
+// Its products are short (about two per C block, two or three 8-wide chunks each), so it is
+// bound by instruction issue and by the chain of dependent index reads in front of the
+// operand loads, not by the tensor pipe.  A warp takes whole C blocks from the counter and
+// runs each in passes of 16 rows x 24 columns of the (possibly transposed) block, where one
+// 16-byte load gives a lane the high and low parts of a fragment.  There is one pass body of
+// runtime size: bodies per tile count filled the instruction cache (5.6 of 13 cycles per
+// instruction waited for it; 5.86 ms on the 2000 x 2000 banded product at 2 % against 3.58
+// now, and 7.74 with a warp per 16 x 16 tile walking the stacks); loading the next fragments
+// during the current MMAs costs spills (4.24 ms), three CTAs per SM measure the same (3.65).
+// The sums leave through shared memory, so that the FP64 adds,
+// 16 cycles a warp instruction, run on full warps and the stores are contiguous.  Per element
+// the MMAs and sums run in the order entry, chunk, {a_lo b_hi, a_hi b_lo, a_hi b_hi}
+// whatever the tile orientation.
+constexpr int kTfPitch = 8 * kTfCols + 1;  // float2 per row of the pass in shared memory
+
+__device__ __forceinline__ float4 ld16f(const float4 *p, bool ok) {
+  return ok ? __ldg(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+__device__ __forceinline__ void mma_tf32f(float (&d)[4], float a0, float a1, float a2, float a3,
+                                          float b0, float b1) {
+  mma_tf32(d, __float_as_uint(a0), __float_as_uint(a1), __float_as_uint(a2), __float_as_uint(a3),
+           __float_as_uint(b0), __float_as_uint(b1));
+}
+
+struct TfBlk {
+  int off, eb, ne, cin, m, n, sw;
+};
+
+struct TfFrag {
+  float4 a0, a1, b[kTfCols];
+};
+
+// the pass from row r00, column c00 of the block (of its transpose when it runs swapped)
+__device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, int r00, int c00,
+                                          const int4 &ent0, float2 *__restrict__ sm) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int r0 = w.mt * 16 + g, r1 = r0 + 8;
-  const bool v0 = r0 < w.m, v1 = r1 < w.m;
-  int colB[2];
-  bool vB[2];
-#pragma unroll
-  for (int nt = 0; nt < 2; ++nt) {
-    colB[nt] = (2 * w.ng + nt) * 8 + g;
-    vB[nt] = nt < w.ntn && colB[nt] < w.n;
-  }
+  const int RM = b.sw ? b.n : b.m, RN = b.sw ? b.m : b.n;
+  const int rows = min(16, RM - r00), cols = min(8 * kTfCols, RN - c00);
+  const float4 *X = reinterpret_cast<const float4 *>(b.sw ? P.b_tf : P.a_tf);
+  const float4 *Y = reinterpret_cast<const float4 *>(b.sw ? P.a_tf : P.b_tf);
   // running sum over the block products as an unevaluated FP32 pair (hi + lo), each
   // product added with an error-free TwoSum, so the sum over many products keeps about
   // twice FP32's precision
-  float hi[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-  float lo[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-  for (int kc = 0; kc < P.Dk; ++kc) {
-    const int64_t rr = (int64_t)w.c * P.Dk + kc;
-    const int len = P.run_len[rr];
-    if (len == 0) continue;
-    const int e0 = P.run_start[rr];
-    const int k = P.kval[kc], kp = (k + 7) & ~7, nch = kp >> 3;
-    for (int e = e0; e < e0 + len; ++e) {
-      const float *At = P.a_tf + P.a_doff[P.s_ab[e]];
-      const float *Bt = P.b_tf + P.b_doff[P.s_bb[e]];
-      const int64_t pa = (int64_t)w.m * kp, pb = (int64_t)w.n * kp;
-      float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-      for (int ch = 0; ch < nch; ++ch) {
-        const uint2 ah0 = v0 ? ld8(At + (int64_t)r0 * kp + ch * 8 + 2 * t) : make_uint2(0, 0);
-        const uint2 ah1 = v1 ? ld8(At + (int64_t)r1 * kp + ch * 8 + 2 * t) : make_uint2(0, 0);
-        const uint2 al0 = v0 ? ld8(At + pa + (int64_t)r0 * kp + ch * 8 + 2 * t) : make_uint2(0, 0);
-        const uint2 al1 = v1 ? ld8(At + pa + (int64_t)r1 * kp + ch * 8 + 2 * t) : make_uint2(0, 0);
+  float hi[kTfCols][4], lo[kTfCols][4], acc[kTfCols][4];
 #pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          if (nt >= w.ntn) break;
-          const uint2 bh = vB[nt] ? ld8(Bt + (int64_t)colB[nt] * kp + ch * 8 + 2 * t) : make_uint2(0, 0);
-          const uint2 bl = vB[nt] ? ld8(Bt + pb + (int64_t)colB[nt] * kp + ch * 8 + 2 * t) : make_uint2(0, 0);
-          mma_tf32(acc[nt], al0.x, al1.x, al0.y, al1.y, bh.x, bh.y);
-          mma_tf32(acc[nt], ah0.x, ah1.x, ah0.y, ah1.y, bl.x, bl.y);
-          mma_tf32(acc[nt], ah0.x, ah1.x, ah0.y, ah1.y, bh.x, bh.y);
+  for (int j = 0; j < kTfCols; ++j)
+#pragma unroll
+    for (int h = 0; h < 4; ++h) hi[j][h] = lo[j][h] = acc[j][h] = 0.f;
+  const float4 *x0, *y0;
+  int rs = 0;  // float4 per operand row: 4 per chunk of 8
+  auto entry = [&](const int4 &e, int j) {
+    const unsigned ea = (unsigned)__shfl_sync(kFull, e.x, j);
+    const unsigned eb = (unsigned)__shfl_sync(kFull, e.y, j);
+    rs = 4 * __shfl_sync(kFull, e.z, j);
+    x0 = X + 4 * (size_t)(b.sw ? eb : ea) + ((int64_t)(r00 + g) * rs + t);
+    y0 = Y + 4 * (size_t)(b.sw ? ea : eb) + ((int64_t)(c00 + g) * rs + t);
+  };
+  auto load = [&](TfFrag &f, int ch) {
+    const float4 *x = x0 + 4 * ch, *y = y0 + 4 * ch;
+    f.a0 = ld16f(x, g < rows);
+    f.a1 = ld16f(x + 8 * (int64_t)rs, g + 8 < rows);
+#pragma unroll
+    for (int j = 0; j < kTfCols; ++j) {
+      f.b[j] = ld16f(y, g + 8 * j < cols);
+      y += 8 * (int64_t)rs;
+    }
+  };
+  if (b.ne > 0) {
+    int4 ent = ent0;
+    int left = b.ne, g0 = 0, j = 0, ch = 0;
+    entry(ent, 0);
+    int nch = rs >> 2;
+    TfFrag cur;
+    load(cur, 0);
+#pragma unroll 1
+    for (;;) {
+      const bool last = ch + 1 == nch;  // last chunk of this product
+      if (last) {
+        ch = 0;
+        if (--left > 0) {
+          if (++j == 32) {
+            g0 += 32;
+            j = 0;
+            ent = g0 + lane < b.ne ? P.ents[(int64_t)b.eb + g0 + lane] : make_int4(0, 0, 0, 0);
+          }
+          entry(ent, j);
+          nch = rs >> 2;
         }
+      } else {
+        ++ch;
       }
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const float a = hi[nt][h], b = acc[nt][h];
-          const float s = __fadd_rn(a, b);
-          const float bb = __fsub_rn(s, a);
-          const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-          hi[nt][h] = s;
-          lo[nt][h] = __fadd_rn(lo[nt][h], err);
+      for (int q = 0; q < kTfCols; ++q) {
+        if (8 * q >= cols) break;
+        const float4 &a0 = cur.a0, &a1 = cur.a1, &bb = cur.b[q];
+        if (b.sw) {  // rows are op(B)'s: its high part times op(A)'s low part first
+          mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, bb.z, bb.w);
+          mma_tf32f(acc[q], a0.z, a1.z, a0.w, a1.w, bb.x, bb.y);
+        } else {
+          mma_tf32f(acc[q], a0.z, a1.z, a0.w, a1.w, bb.x, bb.y);
+          mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, bb.z, bb.w);
         }
+        mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, bb.x, bb.y);
+      }
+      if (last) {
+#pragma unroll
+        for (int q = 0; q < kTfCols; ++q) {
+          if (8 * q >= cols) break;
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const float a = hi[q][h], v = acc[q][h];
+            const float sum = __fadd_rn(a, v);
+            const float bb = __fsub_rn(sum, a);
+            const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bb)), __fsub_rn(v, bb));
+            hi[q][h] = sum;
+            lo[q][h] = __fadd_rn(lo[q][h], err);
+            acc[q][h] = 0.f;
+          }
+        }
+      }
+      if (left == 0) break;
+      load(cur, ch);
     }
   }
-  const int64_t off = P.c_off[w.c];
-  const int cin = P.c_cin[w.c];
-  const double *ci = (P.has_beta && cin >= 0) ? P.Cin + P.cin_off[cin] : nullptr;
-  const bool scale = !P.alpha_one;
 #pragma unroll
-  for (int nt = 0; nt < 2; ++nt)
+  for (int q = 0; q < kTfCols; ++q) {
+    if (8 * q >= cols) break;
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      int r, c;
-      slot_rc(w, nt, h, r, c);
-      if (nt < w.ntn && r < w.m && c < w.n) {
-        double v = f32_to_f64(hi[nt][h]) + f32_to_f64(lo[nt][h]);
-        if (scale) v *= P.alpha;
-        if (ci) v = fma(P.beta, ci[r * w.n + c], v);
-        P.C[off + r * w.n + c] = v;
-      }
+    for (int h = 0; h < 4; ++h)
+      sm[(g + 8 * (h >> 1)) * kTfPitch + 8 * q + 2 * t + (h & 1)] = make_float2(hi[q][h], lo[q][h]);
+  }
+  __syncwarp();
+  // outputs in C order: (outer, inner) = (row, column) of the pass, or swapped
+  const double *ci = (P.has_beta && b.cin >= 0) ? P.Cin + P.cin_off[b.cin] : nullptr;
+  const int64_t c0 = b.sw ? (int64_t)c00 * b.n + r00 : (int64_t)r00 * b.n + c00;
+  const int ni = b.sw ? rows : cols, total = rows * cols;
+  const int so = b.sw ? 1 : kTfPitch, si = b.sw ? kTfPitch : 1;
+  const int di = 32 % ni, dO = 32 / ni;
+  int y = lane / ni, x = lane - y * ni;
+#pragma unroll 1
+  for (int o = lane; o - lane < total; o += 32) {
+    const float2 v2 = o < total ? sm[y * so + x * si] : make_float2(0.f, 0.f);
+    // the FP64 add only where some low part is not zero (a NaN is not): blocks of one
+    // product have none
+    double v = f32_to_f64(v2.x);
+    if (__any_sync(kFull, v2.y != 0.f)) v += f32_to_f64(v2.y);
+    if (o < total) {
+      const int64_t at = c0 + (int64_t)y * b.n + x;
+      if (!P.alpha_one) v *= P.alpha;
+      if (ci) v = fma(P.beta, ci[at], v);
+      P.C[b.off + at] = v;
     }
+    y += dO;
+    x += di;
+    if (x >= ni) {
+      x -= ni;
+      ++y;
+    }
+  }
+  __syncwarp();
+}
+
+__device__ __forceinline__ void tf32_block(const EmuParams &P, int dw, float2 *sm) {
+  const int lane = threadIdx.x & 31;
+  TfBlk b;
+  b.off = __shfl_sync(kFull, dw, 0);
+  b.eb = __shfl_sync(kFull, dw, 1);
+  b.ne = __shfl_sync(kFull, dw, 2);
+  b.cin = __shfl_sync(kFull, dw, 3);
+  b.m = __shfl_sync(kFull, dw, 4);
+  b.n = __shfl_sync(kFull, dw, 5);
+  b.sw = __shfl_sync(kFull, dw, 6);
+  const int4 ent0 = lane < b.ne ? P.ents[(int64_t)b.eb + lane] : make_int4(0, 0, 0, 0);
+  const int RM = b.sw ? b.n : b.m, RN = b.sw ? b.m : b.n;
+#pragma unroll 1
+  for (int r = 0; r < RM; r += 16)
+#pragma unroll 1
+    for (int c = 0; c < RN; c += 8 * kTfCols) tf32_pass(P, b, r, c, ent0, sm);
+}
+
+__global__ void __launch_bounds__(256, 2)
+    k_num_tf32x3(EmuParams P, int64_t nitems, unsigned long long *counter, int take) {
+  __shared__ float2 sums[8][16 * kTfPitch];
+  float2 *sm = sums[threadIdx.x >> 5];
+  emu_persist(
+      nullptr, nitems, counter, [&](int64_t) -> const EmuParams & { return P; },
+      [&](const EmuParams &Q, int w) { tf32_block(Q, w, sm); }, take);
 }
 
 SideArgs side_args(const bst_matrix *X, bool trans, bool is_b) {
@@ -1072,18 +1168,6 @@ void emu_index(bst_plan *p, EmuState &E, cudaStream_t s) {
       BST_CHECK_LAUNCH();
     }
   }
-  // 3xTF32 warps per (m,n) class: one per 16-row x 16-column tile of each C block
-  const int32_t ncls = p->Dm * p->Dn;
-  std::vector<int64_t> ws((size_t)ncls + 1, 0);
-  for (int32_t c = 0; c < ncls; ++c) {
-    const int64_t cnt = (int64_t)p->h_class_ptr[c + 1] - p->h_class_ptr[c];
-    const int m = p->m_vals.empty() ? 0 : p->m_vals[c / p->Dn];
-    const int n = p->n_vals.empty() ? 0 : p->n_vals[c % p->Dn];
-    const int64_t mt = (m + 15) / 16, nt = (n + 7) / 8;
-    ws[c + 1] = ws[c] + cnt * mt * ((nt + 1) / 2);
-  }
-  E.ncls = ncls;
-  E.nwarps = ws.back();
   // global element starts of op(A) row blocks and op(B) column blocks
   auto starts = [&](const std::vector<int32_t> &sz, int64_t &total) {
     std::vector<int64_t> h(sz.size() + 1, 0);
@@ -1094,7 +1178,6 @@ void emu_index(bst_plan *p, EmuState &E, cudaStream_t s) {
   {
     const std::vector<int64_t> ha = starts(p->oa.h_rs, E.nrows), hb = starts(p->ob.h_cs, E.ncols);
     Upload up(p->ctx, s);
-    E.wstart = up.add_vector(ar, ws);
     E.a_rowstart = up.add_vector(ar, ha);
     E.b_colstart = up.add_vector(ar, hb);
     up.done();
@@ -1123,15 +1206,10 @@ EmuParams emu_params(bst_plan *p, const EmuState &E, const NumArgs &a) {
   P.has_beta = a.beta != 0.0;
   P.beta = a.beta;
   P.Dk = p->Dk;
-  P.ncls = E.ncls;
-  P.wstart = E.wstart;
-  P.tiles_n = 2;
   P.a_rowstart = E.a_rowstart;
   P.b_colstart = E.b_colstart;
   P.row_exp = E.row_exp;
   P.col_exp = E.col_exp;
-  P.class_ptr = p->class_ptr;
-  P.task_c = p->task_c;
   P.cls_m = p->cls_m;
   P.cls_n = p->cls_n;
   P.kval = p->kval;
@@ -1207,7 +1285,6 @@ static EmuParams bf16_params(bst_plan *p, const EmuState &E, const NumArgs &a) {
   EmuParams P = emu_params(p, E, a);
   P.a_doff = E.a_doff;
   P.b_doff = E.b_doff;
-  P.tiles_n = 1;
   P.row_scale = p->ctx->tune_emu_row_scale;
   return P;
 }
@@ -1392,13 +1469,30 @@ void emu_costs(bst_plan *p, cudaStream_t s, double *tensor_flops, double *bytes,
 void execute_tf32x3(bst_plan *p, const NumArgs &a, cudaStream_t s) {
   if (p->C->nblocks == 0) return;
   EmuState &E = emu_state(p, s);
+  const int64_t nc = p->C->nblocks;
   if (!E.tf_alloc) {
     E.a_tf = E.ar.alloc_n<float>((size_t)E.a_tsize);
     E.b_tf = E.ar.alloc_n<float>((size_t)E.b_tsize);
+    E.tents = E.ar.alloc_n<int4>((size_t)std::max<int64_t>(p->T, 1));
+    E.tdesc = E.ar.alloc_n<int32_t>((size_t)nc * kDescWords);
+    if (!E.counter) E.counter = E.ar.alloc_n<unsigned long long>(1);
     E.tf_alloc = true;
   }
-  BST_CUDA(cudaMemsetAsync(E.a_tf, 0, 4 * (size_t)std::max<int64_t>(E.a_tsize, 1), s));
-  BST_CUDA(cudaMemsetAsync(E.b_tf, 0, 4 * (size_t)std::max<int64_t>(E.b_tsize, 1), s));
+  if (!E.tf_lists) {
+    k_tf32_ents<<<nblk(nc, 256), 256, 0, s>>>(nc, p->Dk, p->run_start, p->run_len, p->kval, p->s_ab,
+                                              p->s_bb, E.a_toff, E.b_toff, E.ebeg, p->C->off,
+                                              p->c_cls, p->cls_m, p->cls_n, p->c_cin, E.tents,
+                                              E.tdesc);
+    BST_CHECK_LAUNCH();
+    // the lists serve later executes on any stream; an execute captured before they are
+    // built builds them in its graph, on every replay
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    BST_CUDA(cudaStreamIsCapturing(s, &cap));
+    if (cap == cudaStreamCaptureStatusNone) {
+      BST_CUDA(cudaStreamSynchronize(s));
+      E.tf_lists = true;
+    }
+  }
   const int wpb = 8;
   for (int side = 0; side < 2; ++side) {
     const bst_matrix *X = side ? p->B : p->A;
@@ -1411,12 +1505,17 @@ void execute_tf32x3(bst_plan *p, const NumArgs &a, cudaStream_t s) {
     BST_CHECK_LAUNCH();
   }
   EmuParams P = emu_params(p, E, a);
-  P.a_doff = E.a_toff;
-  P.b_doff = E.b_toff;
-  if (E.nwarps > 0) {
-    k_num_tf32x3<<<nblk(E.nwarps, wpb), 32 * wpb, 0, s>>>(P, E.nwarps);
-    BST_CHECK_LAUNCH();
-  }
+  P.desc = E.tdesc;
+  P.ents = E.tents;
+  int per = 0;
+  BST_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_num_tf32x3, 32 * wpb, 0));
+  const int64_t full = (int64_t)std::max(per, 1) * p->ctx->num_sms;
+  // few C blocks: one at a time, so that every warp gets some
+  const int take = nc >= 4 * kChunk * wpb * full ? kChunk : 1;
+  const int g = (int)std::min<int64_t>(full, (nc + wpb * take - 1) / (wpb * take));
+  BST_CUDA(cudaMemsetAsync(E.counter, 0, sizeof(unsigned long long), s));
+  k_num_tf32x3<<<g, 32 * wpb, 0, s>>>(P, nc, E.counter, take);
+  BST_CHECK_LAUNCH();
 }
 
 }  // namespace bst
