@@ -549,6 +549,7 @@ static void adj_build(bst_plan *p, AdjState &S, cudaStream_t s) {
   Arena scratch;
   scratch.ctx = S.ar.ctx;
   scratch.stream = s;
+  scratch.chunk = kScratchChunk;
   S.counters = S.ar.alloc_n<unsigned long long>(kAdjCounters);
   SideBuild sides[2] = {{true, &S.a, p->A}, {false, &S.b, p->B}};
   for (SideBuild &B : sides) side_begin(p, B, S, scratch, s);

@@ -24,6 +24,19 @@ void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 void set_error(const std::string &msg) { g_last_error = msg; }
 
 void *Arena::alloc(size_t bytes) {
+  if (4 * bytes > chunk) return alloc_own(bytes);
+  const size_t need = (std::max<size_t>(bytes, 8) + 255) & ~(size_t)255;
+  if (left < need) {
+    next = static_cast<char *>(alloc_own(chunk));
+    left = chunk;
+  }
+  void *p = next;
+  next += need;
+  left -= need;
+  return p;
+}
+
+void *Arena::alloc_own(size_t bytes) {
   void *p = nullptr;
   if (bytes == 0) bytes = 8;
   if (ctx && ctx->alloc) {
@@ -53,6 +66,7 @@ void Arena::release_all() {
       (void)cudaFreeAsync(b.p, stream);
   }
   bufs.clear();
+  left = 0;
 }
 
 }  // namespace bst
@@ -71,6 +85,63 @@ void use_device(const bst_ctx *ctx) {
 }
 
 }  // namespace
+
+namespace bst {
+
+bst_plan *make_plan(bst_ctx *ctx, char transa, char transb, const bst_matrix *A,
+                    const bst_matrix *B, const bst_matrix *C_in, double eps, cudaStream_t s,
+                    bool schedule) {
+  const bool ta = transa == 'T' || transa == 't', tb = transb == 'T' || transb == 't';
+  BST_REQUIRE(ta || transa == 'N' || transa == 'n', BST_ERR_INVALID_ARG, "transa must be N or T");
+  BST_REQUIRE(tb || transb == 'N' || transb == 'n', BST_ERR_INVALID_ARG, "transb must be N or T");
+  BST_REQUIRE(eps >= 0.0, BST_ERR_INVALID_ARG, "eps must be >= 0");
+  BST_REQUIRE(A->nblocks == 0 || A->data, BST_ERR_STATE, "A data not bound");
+  BST_REQUIRE(B->nblocks == 0 || B->data, BST_ERR_STATE, "B data not bound");
+  // shapes: block columns of op(A) == block rows of op(B), with equal sizes
+  const std::vector<int32_t> &a_rs = ta ? A->h_csz : A->h_rsz, &a_cs = ta ? A->h_rsz : A->h_csz;
+  const std::vector<int32_t> &b_rs = tb ? B->h_csz : B->h_rsz, &b_cs = tb ? B->h_rsz : B->h_csz;
+  BST_REQUIRE(a_cs == b_rs, BST_ERR_SHAPE_MISMATCH,
+              "inner block sizes of op(A) and op(B) differ");
+  if (C_in) {
+    BST_REQUIRE(C_in->h_rsz == a_rs && C_in->h_csz == b_cs, BST_ERR_SHAPE_MISMATCH,
+                "C_in block grid differs from op(A) rows x op(B) columns");
+  }
+  use_device(ctx);
+  auto *p = new bst_plan();
+  try {
+    p->ctx = ctx;
+    p->arena.ctx = static_cast<Ctx *>(ctx);
+    p->arena.stream = s;
+    p->arena.chunk = kPlanChunk;
+    p->work.ctx = static_cast<Ctx *>(ctx);
+    p->work.stream = s;
+    p->A = A;
+    p->B = B;
+    p->Cin = C_in;
+    p->ta = ta;
+    p->tb = tb;
+    p->eps = eps;
+    p->oa = make_opview(A, ta, p->arena, s);
+    p->ob = make_opview(B, tb, p->arena, s);
+    p->M = p->oa.nr;
+    p->N = p->ob.nc;
+    p->K = p->oa.nc;
+    p->C = new bst_matrix();
+    p->C->ctx = ctx;
+    p->C->owned_by_plan = true;
+    symbolic_phase(p, s, schedule);
+  } catch (...) {
+    if (p->C) {
+      p->C->owned_by_plan = false;
+      delete p->C;
+    }
+    delete p;
+    throw;
+  }
+  return p;
+}
+
+}  // namespace bst
 
 extern "C" {
 
@@ -282,54 +353,7 @@ bst_status bst_multiply_plan(bst_ctx *ctx, char transa, char transb, const bst_m
   API_BEGIN
   BST_REQUIRE(ctx && A && B && out, BST_ERR_INVALID_ARG, "NULL argument");
   *out = nullptr;
-  const bool ta = transa == 'T' || transa == 't', tb = transb == 'T' || transb == 't';
-  BST_REQUIRE(ta || transa == 'N' || transa == 'n', BST_ERR_INVALID_ARG, "transa must be N or T");
-  BST_REQUIRE(tb || transb == 'N' || transb == 'n', BST_ERR_INVALID_ARG, "transb must be N or T");
-  BST_REQUIRE(eps >= 0.0, BST_ERR_INVALID_ARG, "eps must be >= 0");
-  BST_REQUIRE(A->nblocks == 0 || A->data, BST_ERR_STATE, "A data not bound");
-  BST_REQUIRE(B->nblocks == 0 || B->data, BST_ERR_STATE, "B data not bound");
-  // shapes: block columns of op(A) == block rows of op(B), with equal sizes
-  const std::vector<int32_t> &a_rs = ta ? A->h_csz : A->h_rsz, &a_cs = ta ? A->h_rsz : A->h_csz;
-  const std::vector<int32_t> &b_rs = tb ? B->h_csz : B->h_rsz, &b_cs = tb ? B->h_rsz : B->h_csz;
-  BST_REQUIRE(a_cs == b_rs, BST_ERR_SHAPE_MISMATCH,
-              "inner block sizes of op(A) and op(B) differ");
-  if (C_in) {
-    BST_REQUIRE(C_in->h_rsz == a_rs && C_in->h_csz == b_cs, BST_ERR_SHAPE_MISMATCH,
-                "C_in block grid differs from op(A) rows x op(B) columns");
-  }
-  use_device(ctx);
-  cudaStream_t s = as_stream(stream);
-  auto *p = new bst_plan();
-  try {
-    p->ctx = ctx;
-    p->arena.ctx = static_cast<bst::Ctx *>(ctx);
-    p->arena.stream = s;
-    p->work.ctx = static_cast<bst::Ctx *>(ctx);
-    p->work.stream = s;
-    p->A = A;
-    p->B = B;
-    p->Cin = C_in;
-    p->ta = ta;
-    p->tb = tb;
-    p->eps = eps;
-    p->oa = bst::make_opview(A, ta, p->arena, s);
-    p->ob = bst::make_opview(B, tb, p->arena, s);
-    p->M = p->oa.nr;
-    p->N = p->ob.nc;
-    p->K = p->oa.nc;
-    p->C = new bst_matrix();
-    p->C->ctx = ctx;
-    p->C->owned_by_plan = true;
-    bst::symbolic_phase(p, s);
-  } catch (...) {
-    if (p->C) {
-      p->C->owned_by_plan = false;
-      delete p->C;
-    }
-    delete p;
-    throw;
-  }
-  *out = p;
+  *out = bst::make_plan(ctx, transa, transb, A, B, C_in, eps, as_stream(stream), true);
   API_END
 }
 

@@ -76,12 +76,20 @@ struct DevBuf {
   size_t bytes = 0;
 };
 
-// A set of device allocations released together (by a plan, a matrix, ...).
+// A set of device allocations released together (by a plan, a matrix, ...).  With a chunk
+// size, allocations of up to a quarter of it are cut from chunks: a plan takes about a
+// hundred small arrays, and each allocation and release costs the host a microsecond or two.
+constexpr size_t kScratchChunk = 1 << 20;  // freed when the call returns
+constexpr size_t kPlanChunk = 1 << 16;     // kept by a plan
 struct Arena {
   Ctx *ctx = nullptr;
   cudaStream_t stream = nullptr;
   std::vector<DevBuf> bufs;
+  size_t chunk = 0;
+  char *next = nullptr;  // the open chunk's free part
+  size_t left = 0;
   void *alloc(size_t bytes);
+  void *alloc_own(size_t bytes);  // an allocation of its own
   template <class T>
   T *alloc_n(size_t n) {
     return static_cast<T *>(alloc(sizeof(T) * (n ? n : 1)));
@@ -108,10 +116,12 @@ struct bst_ctx {
   void *up_host = nullptr;
   size_t up_cap = 0;
   std::mutex up_mutex;
-  // recorded after the copies of an Upload finished with done_async(); the next Upload
-  // waits for it before it writes the staging buffer again
+  // recorded after the copies of an Upload finished with done_async(); the next Upload on
+  // the same stream stages behind them and waits for it only when the buffer is full
   cudaEvent_t up_event = nullptr;
   bool up_pending = false;
+  cudaStream_t up_stream = nullptr;  // of the pending copies
+  size_t up_tail = 0;                // end of the part that they read
   // kernel choices (bst_tune_set): emulated-FP64 digit scaling per whole op row /
   // column (1) or per block row / column (0); per (m, n) C block class, the tile
   // orientation of the emulated kernel (1 = MMA rows run over the C block's columns);
@@ -244,11 +254,12 @@ struct Upload {
   }
   void flush();  // launch the copies staged so far and wait for them
   void done();   // flush() and release the staging buffer to other threads
-  // launch the copies without waiting (the next Upload waits before it reuses the
-  // buffer): only for data the same stream consumes, before a later synchronisation of
+  // launch the copies without waiting (a later Upload waits before it reuses their part of
+  // the buffer): only for data the same stream consumes, before a later synchronisation of
   // that stream hands the result to the caller
   void done_async();
   void launch();  // the copy kernels of the items staged so far
+  void wait_pending();
 };
 void gather_i32(const int32_t *src, const int32_t *idx, int32_t *dst, int64_t n, cudaStream_t s);
 
@@ -271,7 +282,7 @@ struct OpView {
   const int32_t *rowptr = nullptr;             // nr + 1
   const int32_t *col = nullptr;                // block column of op(X) per entry
   const int32_t *blk = nullptr;                // stored block id per entry (null = identity)
-  std::vector<int32_t> h_rs, h_cs;
+  const std::vector<int32_t> *h_rs = nullptr, *h_cs = nullptr;  // the stored matrix's
   bool trans = false;
 };
 OpView make_opview(const bst_matrix *m, bool trans, Arena &ar, cudaStream_t s);
@@ -361,8 +372,13 @@ struct bst_plan {
 
 namespace bst {
 
-// symbolic phase (symbolic.cu): fills everything in the plan from oa/ob/Cin
-void symbolic_phase(bst_plan *p, cudaStream_t s);
+// symbolic phase (symbolic.cu): fills everything in the plan from oa/ob/Cin, except the
+// numeric schedule when the caller builds that itself
+void symbolic_phase(bst_plan *p, cudaStream_t s, bool schedule);
+// a checked multiply plan (bst_api.cu)
+bst_plan *make_plan(bst_ctx *ctx, char transa, char transb, const bst_matrix *A,
+                    const bst_matrix *B, const bst_matrix *C_in, double eps, cudaStream_t s,
+                    bool schedule);
 
 // numeric phase (numeric_fp64.cu / numeric_emu.cu)
 struct NumArgs {

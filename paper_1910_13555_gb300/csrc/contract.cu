@@ -250,6 +250,31 @@ void szoffsets(const bst_tensor *T, int32_t *szoff) {
   }
 }
 
+// Block sizes of the folded dimension over `modes` (first listed most significant): the
+// products of the modes' block sizes, built up mode by mode.
+std::vector<int32_t> fold_sizes(const bst_tensor *T, const std::vector<int32_t> &modes) {
+  int64_t n = 1;
+  for (int32_t d : modes) n *= T->h_nblk[d];
+  BST_REQUIRE(n < INT32_MAX, BST_ERR_UNSUPPORTED, "a folded tensor dimension exceeds 2^31-1 blocks");
+  std::vector<int32_t> out(1, 1);
+  if (n == 0) out.clear();
+  for (size_t q = 0; q < modes.size() && n > 0; ++q) {
+    const std::vector<int32_t> &sz = T->h_sz[modes[q]];
+    std::vector<int32_t> next(out.size() * sz.size());
+    int64_t most = 0;
+    int32_t *o = next.data();
+    for (int64_t v : out)
+      for (int32_t x : sz) {
+        const int64_t w = v * x;
+        most = std::max(most, w);
+        *o++ = (int32_t)w;
+      }
+    BST_REQUIRE(most < INT32_MAX, BST_ERR_OVERFLOW, "folded block size exceeds 2^31-1");
+    out.swap(next);
+  }
+  return out;
+}
+
 // Build the matrix view of T with rows = fold of `rm`, columns = fold of `cm`.
 void build_view(bst_ctx *ctx, const bst_tensor *T, const std::vector<int32_t> &rm,
                 const std::vector<int32_t> &cm, View &V, Arena &ar, cudaStream_t s) {
@@ -262,30 +287,14 @@ void build_view(bst_ctx *ctx, const bst_tensor *T, const std::vector<int32_t> &r
   for (int d = 0; d < T->rank; ++d) ident &= order[d] == d;
   V.identity = ident;
   V.copy = !ident;
-  // folded grid and block sizes (computed from the per-mode sizes; never stored per
-  // tensor block row beyond the folded dimension itself)
-  auto fold_sizes = [&](const std::vector<int32_t> &modes, std::vector<int32_t> &out) {
-    int64_t n = 1;
-    for (int32_t d : modes) n *= T->h_nblk[d];
-    BST_REQUIRE(n < INT32_MAX, BST_ERR_UNSUPPORTED, "a folded tensor dimension exceeds 2^31-1 blocks");
-    out.assign((size_t)n, 1);
-    for (int64_t x = 0; x < n; ++x) {
-      int64_t rem = x, v = 1;
-      for (int q = (int)modes.size() - 1; q >= 0; --q) {
-        const int32_t d = modes[q];
-        v *= T->h_sz[d][rem % T->h_nblk[d]];
-        rem /= T->h_nblk[d];
-      }
-      BST_REQUIRE(v < INT32_MAX, BST_ERR_OVERFLOW, "folded block size exceeds 2^31-1");
-      out[(size_t)x] = (int32_t)v;
-    }
-  };
   auto *M = new bst_matrix();
   V.M = M;
   M->ctx = ctx;
   M->owned_by_plan = true;
-  fold_sizes(rm, M->h_rsz);
-  fold_sizes(cm, M->h_csz);
+  // folded grid and block sizes (computed from the per-mode sizes; never stored per
+  // tensor block row beyond the folded dimension itself)
+  M->h_rsz = fold_sizes(T, rm);
+  M->h_csz = fold_sizes(T, cm);
   M->nbr = (int32_t)M->h_rsz.size();
   M->nbc = (int32_t)M->h_csz.size();
   M->nblocks = T->nblocks;
@@ -294,7 +303,7 @@ void build_view(bst_ctx *ctx, const bst_tensor *T, const std::vector<int32_t> &r
     Upload up(ctx, s);
     M->rsz = up.add_vector(ar, M->h_rsz);
     M->csz = up.add_vector(ar, M->h_csz);
-    up.done();
+    up.done_async();  // read by this stream's kernels; the plan synchronises later
   }
   const int64_t n = T->nblocks;
   FoldArgs F{};
@@ -315,6 +324,7 @@ void build_view(bst_ctx *ctx, const bst_tensor *T, const std::vector<int32_t> &r
   Arena scratch;
   scratch.ctx = static_cast<Ctx *>(ctx);
   scratch.stream = s;
+  scratch.chunk = kScratchChunk;
   int32_t *frow = ar.alloc_n<int32_t>((size_t)n), *fcol = ar.alloc_n<int32_t>((size_t)n);
   uint64_t *key = ident ? nullptr : scratch.alloc_n<uint64_t>((size_t)n);
   F.row = frow;
@@ -367,7 +377,6 @@ void build_view(bst_ctx *ctx, const bst_tensor *T, const std::vector<int32_t> &r
   M->rowptr = ar.alloc_n<int32_t>((size_t)M->nbr + 1);
   k_i64_to_i32_n<<<nblk((int64_t)M->nbr + 1, 256), 256, 0, s>>>(rp64, M->rowptr, (int64_t)M->nbr + 1);
   BST_CHECK_LAUNCH();
-  BST_CUDA(cudaStreamSynchronize(s));
   scratch.release_all();
   M->data = ident ? T->data : V.buf;
 }
@@ -412,23 +421,24 @@ void setup_slab_read(bst_plan *p, const View &V, const std::vector<int32_t> &F1,
     if (id) j = q;
   }
   if (j < 0 || V.M->nblocks == 0) return;
-  // k_i of every k block (mixed radix over C1, first listed most significant)
+  // k_i of every k block size, k = (outer fold size) x (inner fold size), over the distinct
+  // sizes of the two folds (every pair of them occurs)
+  auto distinct = [&](size_t q0, size_t q1) {
+    std::vector<int32_t> v = fold_sizes(T, std::vector<int32_t>(C1.begin() + q0, C1.begin() + q1));
+    std::sort(v.begin(), v.end());
+    v.erase(std::unique(v.begin(), v.end()), v.end());
+    return v;
+  };
+  const std::vector<int32_t> outer = distinct(0, (size_t)j), inner = distinct((size_t)j, (size_t)nc);
   std::map<int32_t, int32_t> kin_of;
-  const int64_t nk = (int64_t)V.M->h_csz.size();
-  for (int64_t x = 0; x < nk; ++x) {
-    int64_t rem = x, ki = 1;
-    for (int q = nc - 1; q >= 0; --q) {
-      const int32_t d = C1[q];
-      if (q >= j) ki *= T->h_sz[d][rem % T->h_nblk[d]];
-      rem /= T->h_nblk[d];
+  for (int32_t o : outer)
+    for (int32_t ki : inner) {
+      auto it = kin_of.find(o * ki);
+      if (it == kin_of.end())
+        kin_of[o * ki] = ki;
+      else if (it->second != ki)
+        return;  // two slab widths for one k class
     }
-    const int32_t k = V.M->h_csz[(size_t)x];
-    auto it = kin_of.find(k);
-    if (it == kin_of.end())
-      kin_of[k] = (int32_t)ki;
-    else if (it->second != ki)
-      return;  // two slab widths for one k class
-  }
   std::vector<int32_t> kin(p->k_vals.size());
   for (size_t kc = 0; kc < kin.size(); ++kc) {
     auto it = kin_of.find(p->k_vals[kc]);
@@ -441,7 +451,6 @@ void setup_slab_read(bst_plan *p, const View &V, const std::vector<int32_t> &F1,
   p->a_slab_kin = kin;
   p->a_slab_toff = toff;
   p->a_slab_base = T->data;
-  build_f64_schedule(p, s);
 }
 
 void free_view(View &V) {
@@ -749,6 +758,7 @@ bst_status bst_contract_plan(bst_ctx *ctx, const bst_tensor *T1, const bst_tenso
   try {
     K->ar.ctx = static_cast<bst::Ctx *>(ctx);
     K->ar.stream = s;
+    K->ar.chunk = bst::kPlanChunk;
     std::vector<int32_t> F1(f1, f1 + nfree1), F2(f2, f2 + nfree2), C1(c1, c1 + ncontract),
         C2(c2, c2 + ncontract);
     auto is_ident = [](const std::vector<int32_t> &a, const std::vector<int32_t> &b) {
@@ -784,12 +794,12 @@ bst_status bst_contract_plan(bst_ctx *ctx, const bst_tensor *T1, const bst_tenso
     // the symbolic phase reads the operand norms: fill the permuted copies first
     bst::permute_view(K->A, T1->data, K->A.buf, true, s);
     bst::permute_view(K->B, T2->data, K->B.buf, true, s);
-    bst_status st = bst_multiply_plan(ctx, ta ? 'T' : 'N', tb ? 'T' : 'N', K->A.M, K->B.M,
-                                      R_in ? K->Ci.M : nullptr, eps, stream, &p);
-    if (st != BST_OK) throw Error{st, bst_last_error()};
+    p = bst::make_plan(ctx, ta ? 'T' : 'N', tb ? 'T' : 'N', K->A.M, K->B.M,
+                       R_in ? K->Ci.M : nullptr, eps, s, false);
     p->contract = K;
     if (!ta && K->A.copy && static_cast<bst::Ctx *>(ctx)->tune_contract_slab)
       bst::setup_slab_read(p, K->A, F1, C1, K->ar, s);
+    bst::build_f64_schedule(p, s);
     // result tensor: blocks of C unfolded into result-order tuples
     const bst_matrix *C = p->C;
     auto *R = new bst_tensor();
@@ -810,7 +820,7 @@ bst_status bst_contract_plan(bst_ctx *ctx, const bst_tensor *T1, const bst_tenso
     {
       bst::Upload up(ctx, s);
       R->sz = up.add_vector(K->ar, flat);
-      up.done();
+      up.done_async();  // read by this stream's kernels; the read-back below synchronises
     }
     bool rid = true;
     for (int r = 0; r < rr; ++r) rid &= ro[r] == r;
@@ -835,6 +845,7 @@ bst_status bst_contract_plan(bst_ctx *ctx, const bst_tensor *T1, const bst_tenso
     bst::Arena scratch;
     scratch.ctx = static_cast<bst::Ctx *>(ctx);
     scratch.stream = s;
+    scratch.chunk = bst::kScratchChunk;
     int32_t *cidx = scratch.alloc_n<int32_t>((size_t)nc * rr);
     uint64_t *key = rid ? nullptr : scratch.alloc_n<uint64_t>((size_t)nc);
     U.idx = cidx;

@@ -1102,7 +1102,7 @@ static void panel_build(bst_plan *p, PanelState &PS, cudaStream_t s) {
     if (v > 32) return;
   const int64_t na = p->A->nblocks, nbk = p->B->nblocks;
   const HostView va = host_view(p, p->oa, na, s), vb = host_view(p, p->ob, nbk, s);
-  const std::vector<int32_t> &ars = p->oa.h_rs, &acs = p->oa.h_cs, &bcs = p->ob.h_cs;
+  const std::vector<int32_t> &ars = *p->oa.h_rs, &acs = *p->oa.h_cs, &bcs = *p->ob.h_cs;
   const int32_t K = p->oa.nc;
   // A panels: op(A) blocks grouped by block column k, in block-row order
   std::vector<int64_t> kcnt((size_t)K + 1, 0);

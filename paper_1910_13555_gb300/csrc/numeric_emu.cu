@@ -1176,7 +1176,7 @@ void emu_index(bst_plan *p, EmuState &E, cudaStream_t s) {
     return h;
   };
   {
-    const std::vector<int64_t> ha = starts(p->oa.h_rs, E.nrows), hb = starts(p->ob.h_cs, E.ncols);
+    const std::vector<int64_t> ha = starts(*p->oa.h_rs, E.nrows), hb = starts(*p->ob.h_cs, E.ncols);
     Upload up(p->ctx, s);
     E.a_rowstart = up.add_vector(ar, ha);
     E.b_colstart = up.add_vector(ar, hb);

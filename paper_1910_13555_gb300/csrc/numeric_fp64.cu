@@ -820,7 +820,7 @@ struct SchedTabs {
 
 // panels of one product of inner size k at panel width w: whole panels, or with slab
 // width ki > 0 panels that never cross a slab (several whole slabs when w >= ki)
-__device__ __forceinline__ int panel_count(int k, int w, int ki) {
+__host__ __device__ __forceinline__ int panel_count(int k, int w, int ki) {
   if (ki <= 0) return (k + w - 1) / w;
   if (w >= ki) {
     const int ws = (w / ki) * ki;
@@ -868,14 +868,16 @@ __device__ __forceinline__ void f64_tiles_of(
     const int32_t *__restrict__ c_cin, const int64_t *__restrict__ tbeg,
     const int64_t *__restrict__ ebeg, const SchedTabs &S, int32_t *__restrict__ desc,
     int4 *__restrict__ ents, int32_t *__restrict__ key, const int32_t *__restrict__ cls_smax,
-    int tile_max, int slot_elems, long long &c1_sum, long long &saved_sum) {
+    const int32_t *__restrict__ t_start, int tile_max, int slot_elems, long long &c1_sum,
+    long long &saved_sum) {
   const int cls = c_cls[c];
   const int m = S.cls_m[cls], n = S.cls_n[cls], tr = S.tile_rows[cls];
   const int nt = (m + tr - 1) / tr;
   for (int t = 0; t < nt; ++t) {
-    const int64_t tile = tbeg[c] + t;
+    const int64_t tile = tbeg ? tbeg[c] + t : c;
     const int p0 = t * tr, mt = min(tr, m - p0);
-    int64_t q = ebeg[tile];
+    const int64_t q0 = ebeg ? ebeg[tile] : t_start[c];
+    int64_t q = q0;
     unsigned long long flops = 0;
     TailCost tc = tail_cost(mt * n, cls_smax[cls]);
     for (int kc = 0; kc < S.Dk; ++kc) {
@@ -923,8 +925,8 @@ __device__ __forceinline__ void f64_tiles_of(
     // the descriptor as two 16-byte stores (word 7, the split, once it is known)
     int32_t *d = desc + tile * kF64Desc;
     int4 *dv = reinterpret_cast<int4 *>(d);
-    dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)ebeg[tile],
-                      (int32_t)(q - ebeg[tile]), mt | (n << 12));
+    dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)q0, (int32_t)(q - q0),
+                      mt | (n << 12));
     key[tile] = __clzll(flops + 1ull);
     const long long w1 = tc.w1;  // the tile's inner elements
     // a short tile never splits (the test f64_split_of starts with), decided here
@@ -950,11 +952,13 @@ __global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
                             const int64_t *__restrict__ tbeg, const int64_t *__restrict__ ebeg,
                             SchedTabs S, int32_t *__restrict__ desc, int4 *__restrict__ ents,
                             int32_t *__restrict__ key, const int32_t *__restrict__ cls_smax,
-                            int tile_max, int slot_elems, unsigned long long *__restrict__ sums) {
+                            const int32_t *__restrict__ t_start, int tile_max, int slot_elems,
+                            unsigned long long *__restrict__ sums) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   long long c1_sum = 0, saved_sum = 0;
   if (c < nc) f64_tiles_of(c, c_cls, run_start, run_len, s_a, s_b, c_off, c_cin, tbeg, ebeg, S,
-                           desc, ents, key, cls_smax, tile_max, slot_elems, c1_sum, saved_sum);
+                           desc, ents, key, cls_smax, t_start, tile_max, slot_elems, c1_sum,
+                           saved_sum);
   for (int o = 16; o > 0; o >>= 1) {
     c1_sum += __shfl_down_sync(0xffffffffu, c1_sum, o);
     saved_sum += __shfl_down_sync(0xffffffffu, saved_sum, o);
@@ -1167,24 +1171,40 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   // slab reading of A: whole C blocks only (a slab holds all m rows), op(A) = A
   const bool slab = slab_wanted && !strided && !tiled;
   if (slab) strided = true;
-  int64_t slot = 1;
-  for (int32_t b = 0; b < p->nb_all; ++b) {
-    if (p->h_bucket_ptr[b + 1] == p->h_bucket_ptr[b]) continue;
-    const int32_t kc = b % Dk, ncl = (b / Dk) % p->Dn, mc = b / (Dk * p->Dn);
-    const int32_t cls = mc * p->Dn + ncl;
-    const int64_t n = p->n_vals[ncl], k = p->k_vals[kc], tr = tile_rows[(size_t)cls];
-    // panels of about equal width (a narrow last one would cost a whole job); of whole
-    // slabs when read in place
-    const int64_t wmax = slot_max / (tr + n), np = (k + wmax - 1) / wmax;
-    const int64_t w = k <= wmax ? k : slab ? wmax : (k + np - 1) / np;
-    wpanel[(size_t)cls * Dk + kc] = (int32_t)w;
-    if (w < k) strided = true;
-    slot = std::max(slot, (tr + n) * w);
+  // panel widths, slot size, and the tiles and entries of all C blocks (from the class and
+  // bucket counts)
+  int64_t slot = 1, ntiles = 0, nents = 0;
+  for (int32_t cls = 0, b = 0; cls < ncls; ++cls) {
+    if (p->h_class_ptr[cls + 1] == p->h_class_ptr[cls]) {
+      b += Dk;
+      continue;
+    }
+    const int64_t m = p->m_vals[cls / p->Dn], n = p->n_vals[cls % p->Dn], tr = tile_rows[(size_t)cls];
+    const int64_t wmax = slot_max / (tr + n), nt = (m + tr - 1) / tr;
+    ntiles += ((int64_t)p->h_class_ptr[cls + 1] - p->h_class_ptr[cls]) * nt;
+    for (int32_t kc = 0; kc < Dk; ++kc, ++b) {
+      const int64_t cnt = p->h_bucket_ptr[b + 1] - p->h_bucket_ptr[b];
+      if (cnt == 0) continue;
+      // panels of about equal width (a narrow last one would cost a whole job); of whole
+      // slabs when read in place
+      const int64_t k = p->k_vals[kc];
+      int64_t w = k, panels = 1;
+      if (k > wmax) {
+        const int64_t np = (k + wmax - 1) / wmax;
+        w = slab ? wmax : (k + np - 1) / np;
+        strided = true;
+      }
+      if (k > wmax || slab) panels = panel_count(k, w, slab ? p->a_slab_kin[kc] : 0);
+      wpanel[(size_t)b] = (int32_t)w;
+      slot = std::max(slot, (tr + n) * w);
+      nents += cnt * nt * panels;
+    }
   }
   Arena &ar = p->sched_ar;
   Arena scratch;
   scratch.ctx = static_cast<Ctx *>(p->ctx);
   scratch.stream = s;
+  scratch.chunk = kScratchChunk;
   int32_t *d_tr, *d_wp, *d_kin = nullptr, *d_smax;
   {
     Upload up(p->ctx, s);
@@ -1208,36 +1228,30 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   S.kin = d_kin;
   S.s_ab = p->s_ab;
   S.a_toff = p->a_slab_toff;
-  int32_t *tcnt = scratch.alloc_n<int32_t>((size_t)nc);
-  int64_t *tbeg = scratch.alloc_n<int64_t>((size_t)nc + 1);
-  k_f64_tile_count<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, S, tcnt);
-  BST_CHECK_LAUNCH();
-  exscan_i32_i64(tcnt, tbeg, nc, scratch, s);
-  int64_t ntiles = 0;
-  {
-    ReadBack rb(p->ctx, s);
-    rb.add(&ntiles, tbeg + nc, 8);
-    rb.done();
-  }
-  int32_t *ecnt = scratch.alloc_n<int32_t>((size_t)ntiles);
-  int64_t *ebeg = scratch.alloc_n<int64_t>((size_t)ntiles + 1);
-  k_f64_ent_count<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->run_len, tbeg, S, ecnt);
-  BST_CHECK_LAUNCH();
-  exscan_i32_i64(ecnt, ebeg, ntiles, scratch, s);
-  int64_t nents = 0;
-  {
-    ReadBack rb(p->ctx, s);
-    rb.add(&nents, ebeg + ntiles, 8);
-    rb.done();
-  }
   BST_REQUIRE(nents < INT32_MAX && ntiles < INT32_MAX, BST_ERR_OVERFLOW,
               "more than 2^31-1 staged tiles or entries");
+  // where a block's tiles and a tile's entries start: with one tile per C block and one
+  // entry per product, the block itself and its first product
+  int64_t *tbeg = nullptr, *ebeg = nullptr;
+  if (ntiles != nc || nents != p->T) {
+    int32_t *tcnt = scratch.alloc_n<int32_t>((size_t)nc);
+    tbeg = scratch.alloc_n<int64_t>((size_t)nc + 1);
+    k_f64_tile_count<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, S, tcnt);
+    BST_CHECK_LAUNCH();
+    exscan_i32_i64(tcnt, tbeg, nc, scratch, s);
+    int32_t *ecnt = scratch.alloc_n<int32_t>((size_t)ntiles);
+    ebeg = scratch.alloc_n<int64_t>((size_t)ntiles + 1);
+    k_f64_ent_count<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->run_len, tbeg, S, ecnt);
+    BST_CHECK_LAUNCH();
+    exscan_i32_i64(ecnt, ebeg, ntiles, scratch, s);
+  }
   p->fents = ar.alloc_n<int4>((size_t)nents);
   p->fdesc = ar.alloc_n<int32_t>((size_t)ntiles * kF64Desc);
   p->tkeys = ar.alloc_n<int32_t>((size_t)ntiles);
   k_f64_tiles<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->run_start, p->run_len, p->s_a,
                                             p->s_b, p->C->off, p->c_cin, tbeg, ebeg, S, p->fdesc,
-                                            p->fents, p->tkeys, d_smax, tile, (int)slot, d_sums);
+                                            p->fents, p->tkeys, d_smax, p->t_start, tile,
+                                            (int)slot, d_sums);
   BST_CHECK_LAUNCH();
   // tiles by decreasing cost
   int64_t *it0 = scratch.alloc_n<int64_t>((size_t)ntiles);

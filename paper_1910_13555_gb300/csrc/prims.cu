@@ -310,12 +310,27 @@ void ReadBack::finish() {
 Upload::Upload(bst_ctx *c, cudaStream_t st) : ctx(c), s(st) {
   ctx->up_mutex.lock();
   locked = true;
+  if (ctx->up_pending) {
+    if (ctx->up_stream == s)
+      used = ctx->up_tail;  // behind the copies in flight
+    else
+      wait_pending();  // no throw here: the lock is held
+  }
+}
+
+void Upload::wait_pending() {
+  if (!ctx->up_pending) return;
+  ctx->up_pending = false;
+  (void)cudaEventSynchronize(ctx->up_event);
 }
 
 Upload::~Upload() {
   if (locked) {
     // an exception left copies in flight: let them land before the buffer is reused
-    if (!items.empty() || used) (void)cudaStreamSynchronize(s);
+    if (!items.empty() || used) {
+      (void)cudaStreamSynchronize(s);
+      ctx->up_pending = false;
+    }
     ctx->up_mutex.unlock();
   }
 }
@@ -332,8 +347,12 @@ void Upload::done_async() {
   if (!items.empty()) {
     launch();
     if (!ctx->up_event) BST_CUDA(cudaEventCreateWithFlags(&ctx->up_event, cudaEventDisableTiming));
+    // the event covers the earlier copies too, whatever became of their stream
+    if (ctx->up_pending) BST_CUDA(cudaStreamWaitEvent(s, ctx->up_event, 0));
     BST_CUDA(cudaEventRecord(ctx->up_event, s));
     ctx->up_pending = true;
+    ctx->up_stream = s;
+    ctx->up_tail = used;
     items.clear();
     used = 0;
   }
@@ -345,16 +364,16 @@ void Upload::done_async() {
 
 void Upload::add(void *dev_dst, const void *host_src, size_t bytes) {
   if (bytes == 0) return;
-  if (ctx->up_pending) {  // an earlier Upload's copies may still read the buffer
-    BST_CUDA(cudaEventSynchronize(ctx->up_event));
-    ctx->up_pending = false;
-  }
   const size_t off = (used + 15) & ~(size_t)15;
   if (off + bytes > ctx->up_cap) {
+    // full: once the copies in flight and the items staged so far are out, start over, or
     // grow (geometrically, never shrinking: freeing pinned memory synchronises the whole
-    // device): the items staged so far are copied out first
+    // device)
+    wait_pending();
     flush();
-    const size_t cap = std::max<size_t>({(size_t)1 << 20, 2 * ctx->up_cap, 2 * (off + bytes)});
+    used = 0;
+    if (4 * bytes <= ctx->up_cap) return add(dev_dst, host_src, bytes);
+    const size_t cap = std::max<size_t>({(size_t)1 << 20, 2 * ctx->up_cap, 8 * bytes});
     if (ctx->up_host) BST_CUDA(cudaFreeHost(ctx->up_host));
     ctx->up_host = nullptr;
     ctx->up_cap = 0;
@@ -372,6 +391,7 @@ void Upload::flush() {
   launch();
   BST_CUDA(cudaStreamSynchronize(s));
   items.clear();
+  ctx->up_pending = false;  // on this stream, so it is over too
   used = 0;
 }
 

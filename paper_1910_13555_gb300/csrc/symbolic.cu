@@ -429,8 +429,8 @@ OpView make_opview(const bst_matrix *m, bool trans, Arena &ar, cudaStream_t s) {
   v.nc = trans ? m->nbr : m->nbc;
   v.rs = trans ? m->csz : m->rsz;
   v.cs = trans ? m->rsz : m->csz;
-  v.h_rs = trans ? m->h_csz : m->h_rsz;
-  v.h_cs = trans ? m->h_rsz : m->h_csz;
+  v.h_rs = trans ? &m->h_csz : &m->h_rsz;
+  v.h_cs = trans ? &m->h_rsz : &m->h_csz;
   if (!trans) {
     v.rowptr = m->rowptr;
     v.col = m->col;
@@ -450,34 +450,48 @@ OpView make_opview(const bst_matrix *m, bool trans, Arena &ar, cudaStream_t s) {
   return v;
 }
 
-static std::vector<int32_t> distinct_sorted(const std::vector<int32_t> &v) {
-  std::vector<int32_t> u(v);
-  std::sort(u.begin(), u.end());
-  u.erase(std::unique(u.begin(), u.end()), u.end());
-  return u;
+// Distinct values of v, ascending, and each element's place among them.  Block sizes are
+// small, so both come from a table over the values: sorting the 500 000 block sizes of a
+// folded dimension and searching each one took milliseconds.
+static std::vector<int32_t> size_classes(const std::vector<int32_t> &v,
+                                         std::vector<int32_t> &vals) {
+  int32_t most = 0;
+  for (int32_t x : v) most = std::max(most, x);
+  std::vector<int32_t> cls(v.size());
+  vals.clear();
+  if (most <= (1 << 16)) {
+    std::vector<int32_t> at((size_t)most + 1, -1);
+    for (int32_t x : v) at[(size_t)x] = 0;
+    for (int32_t x = 0; x <= most; ++x)
+      if (at[(size_t)x] == 0) {
+        at[(size_t)x] = (int32_t)vals.size();
+        vals.push_back(x);
+      }
+    for (size_t i = 0; i < v.size(); ++i) cls[i] = at[(size_t)v[i]];
+    return cls;
+  }
+  vals = v;
+  std::sort(vals.begin(), vals.end());
+  vals.erase(std::unique(vals.begin(), vals.end()), vals.end());
+  for (size_t i = 0; i < v.size(); ++i)
+    cls[i] = (int32_t)(std::lower_bound(vals.begin(), vals.end(), v[i]) - vals.begin());
+  return cls;
 }
 
-static int32_t *upload_classes(const std::vector<int32_t> &sizes, const std::vector<int32_t> &vals,
-                               Arena &ar, Upload &up) {
-  std::vector<int32_t> cls(sizes.size());
-  for (size_t i = 0; i < sizes.size(); ++i)
-    cls[i] = (int32_t)(std::lower_bound(vals.begin(), vals.end(), sizes[i]) - vals.begin());
-  return up.add_vector(ar, cls);
-}
-
-void symbolic_phase(bst_plan *p, cudaStream_t s) {
+void symbolic_phase(bst_plan *p, cudaStream_t s, bool schedule) {
   Arena &ar = p->arena;
   Arena scratch;
   scratch.ctx = static_cast<Ctx *>(p->ctx);
   scratch.stream = s;
+  scratch.chunk = kScratchChunk;
   const bst_matrix *A = p->A, *B = p->B, *Ci = p->Cin;
   const OpView &oa = p->oa, &ob = p->ob;
   const int32_t M = p->M, N = p->N;
 
   // size classes of C rows (m), C columns (n) and the inner dimension (k)
-  p->m_vals = distinct_sorted(oa.h_rs);
-  p->n_vals = distinct_sorted(ob.h_cs);
-  p->k_vals = distinct_sorted(oa.h_cs);
+  const std::vector<int32_t> m_cls = size_classes(*oa.h_rs, p->m_vals),
+                             n_cls = size_classes(*ob.h_cs, p->n_vals),
+                             k_cls = size_classes(*oa.h_cs, p->k_vals);
   p->Dm = std::max<int32_t>(1, (int32_t)p->m_vals.size());
   p->Dn = std::max<int32_t>(1, (int32_t)p->n_vals.size());
   p->Dk = std::max<int32_t>(1, (int32_t)p->k_vals.size());
@@ -486,9 +500,9 @@ void symbolic_phase(bst_plan *p, cudaStream_t s) {
   p->nb_all = (int32_t)nb_all;
   {
     Upload up(p->ctx, s);
-    p->m_cls = upload_classes(oa.h_rs, p->m_vals, ar, up);
-    p->n_cls = upload_classes(ob.h_cs, p->n_vals, ar, up);
-    p->k_cls = upload_classes(oa.h_cs, p->k_vals, ar, up);
+    p->m_cls = up.add_vector(ar, m_cls);
+    p->n_cls = up.add_vector(ar, n_cls);
+    p->k_cls = up.add_vector(ar, k_cls);
     std::vector<int32_t> cm((size_t)p->Dm * p->Dn), cn((size_t)p->Dm * p->Dn), kv(p->k_vals);
     for (int32_t a = 0; a < p->Dm; ++a)
       for (int32_t b = 0; b < p->Dn; ++b) {
@@ -567,8 +581,8 @@ void symbolic_phase(bst_plan *p, cudaStream_t s) {
   bst_matrix *C = p->C;
   C->nbr = M;
   C->nbc = N;
-  C->h_rsz = oa.h_rs;
-  C->h_csz = ob.h_cs;
+  C->h_rsz = *oa.h_rs;
+  C->h_csz = *ob.h_cs;
   C->nblocks = nnzC;
   C->rsz = const_cast<int32_t *>(oa.rs);
   C->csz = const_cast<int32_t *>(ob.cs);
@@ -711,13 +725,14 @@ void symbolic_phase(bst_plan *p, cudaStream_t s) {
   st.n_c_elements = nelemC;
   int32_t nbk = 0;
   double flops = 0.0;
-  for (int32_t b = 0; b < p->nb_all; ++b) {
-    const int64_t n = (int64_t)hb[b + 1] - hb[b];
-    if (n <= 0) continue;
-    ++nbk;
-    const int32_t kc = b % p->Dk, nc = (b / p->Dk) % p->Dn, mc = b / (p->Dk * p->Dn);
-    flops += 2.0 * p->m_vals[mc] * p->n_vals[nc] * p->k_vals[kc] * (double)n;
-  }
+  for (size_t mc = 0, b = 0; mc < p->m_vals.size(); ++mc)
+    for (size_t nc = 0; nc < p->n_vals.size(); ++nc)
+      for (size_t kc = 0; kc < p->k_vals.size(); ++kc, ++b) {
+        const int64_t n = (int64_t)hb[b + 1] - hb[b];
+        if (n <= 0) continue;
+        ++nbk;
+        flops += 2.0 * p->m_vals[mc] * p->n_vals[nc] * p->k_vals[kc] * (double)n;
+      }
   st.n_buckets = nbk;
   st.flops = flops;
   st.split_k = 1;
@@ -725,7 +740,7 @@ void symbolic_phase(bst_plan *p, cudaStream_t s) {
   // entry, 8 bytes per norm (C_in read is added at execute time when beta != 0)
   st.bytes = 8.0 * ((double)hrefel[0] + (double)hrefel[1] + (double)nelemC) + 12.0 * (double)T +
              8.0 * (double)(A->nblocks + B->nblocks);
-  build_f64_schedule(p, s);
+  if (schedule) build_f64_schedule(p, s);
 }
 
 }  // namespace bst
