@@ -63,8 +63,10 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // per block, and the group's 32 square roots run together.  Matrices with larger blocks
 // (a contraction's folded views, up to hundreds of thousands of elements a block): one
 // warp per block, a butterfly at the end (grouping them left a few hundred warps
-// streaming 32 large blocks each: 4.6 ms for the rank-4 operand against a few tens of
-// microseconds).
+// streaming 32 large blocks each: 4.6 ms for the rank-4 operand).  Both read HBM once and are
+// bound by the loads a warp has in flight, so they issue eight before the dependent FMAs
+// (a rank-4 contraction as a whole 10.20 -> 10.06 ms, the small-B product 3.34 -> 3.29); each
+// lane's sum keeps its order, e = lane, lane + 32, ..., and the norms their bits.
 constexpr int kNormGroup = 32;
 constexpr int kNormWarps = 4;
 constexpr int64_t kNormSmall = 1024;
@@ -80,9 +82,16 @@ __global__ void __launch_bounds__(32 * kNormWarps)
   const int64_t len = (int64_t)rsz[row[b]] * csz[col[b]];
   const double *x = data + off[b];
   double s = 0.0;
-  for (int64_t e = lane; e < len; e += 32) {
-    const double v = __ldg(x + e);
-    s = fma(v, v, s);
+  for (int64_t e0 = 0; e0 < len; e0 += 256) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int64_t e = e0 + 32 * u + lane;
+      v[u] = e < len ? __ldg(x + e) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (e0 + 32 * u < len) s = fma(v[u], v[u], s);
   }
   s = warp_sum_d(s);
   if (lane == 0) norms[b] = sqrt(s);
@@ -105,15 +114,28 @@ __global__ void __launch_bounds__(32 * kNormWarps)
     my_off = off[b0 + lane];
   }
   double(*P)[33] = part[wl];
-  for (int j = 0; j < nb; ++j) {
-    const int len = __shfl_sync(0xffffffffu, my_len, j);
-    const double *x = data + __shfl_sync(0xffffffffu, my_off, j);
-    double s = 0.0;
-    for (int e = lane; e < len; e += 32) {
-      const double v = __ldg(x + e);
-      s = fma(v, v, s);
+  for (int j0 = 0; j0 < nb; j0 += 4) {  // four blocks at a time, two loads of each ahead
+    double v[4][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int len = __shfl_sync(0xffffffffu, my_len, j0 + u);
+      const double *x = data + __shfl_sync(0xffffffffu, my_off, j0 + u);
+      v[u][0] = lane < len ? __ldg(x + lane) : 0.0;
+      v[u][1] = lane + 32 < len ? __ldg(x + lane + 32) : 0.0;
     }
-    P[j][lane] = s;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int len = __shfl_sync(0xffffffffu, my_len, j0 + u);
+      const double *x = data + __shfl_sync(0xffffffffu, my_off, j0 + u);
+      double s = fma(v[u][0], v[u][0], 0.0);
+      if (len > 32) s = fma(v[u][1], v[u][1], s);
+#pragma unroll 4
+      for (int e = lane + 64; e < len; e += 32) {
+        const double y = __ldg(x + e);
+        s = fma(y, y, s);
+      }
+      P[j0 + u][lane] = s;
+    }
   }
   __syncwarp();
   if (lane < nb) {
