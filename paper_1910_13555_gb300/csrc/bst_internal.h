@@ -210,14 +210,16 @@ void iota_i32(int32_t *p, int64_t n, cudaStream_t s);
 void fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t s);
 
 // Device -> host reads of a few values (sizes, bucket and class pointers) during plan
-// construction.  A kernel writes them into the context's mapped pinned buffer, so they
-// do not queue on the copy engine behind a large transfer of another stream; finish()
-// synchronises the stream and copies them to their host destinations.
+// construction.  finish() has a kernel write them into the context's mapped pinned buffer,
+// so they do not queue on the copy engine behind a large transfer of another stream,
+// synchronises the stream and copies them to their host destinations; the sources stay
+// allocated and unchanged until then.
 struct ReadBack {
   bst_ctx *ctx;
   cudaStream_t s;
   struct Item {
     void *dst;
+    const void *src;
     size_t off, bytes;
   };
   std::vector<Item> items;

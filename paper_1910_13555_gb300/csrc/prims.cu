@@ -104,10 +104,48 @@ __global__ void k_tile_scan(const TI *__restrict__ in, int64_t n, const TO *__re
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) out[n] = ex;
 }
 
+// the whole scan by one CTA: three launches on a few thousand elements are mostly latency
+constexpr int kOneThreads = 1024, kOneTile = kOneThreads * kScanItems;
+
+template <class TI, class TO>
+__global__ void __launch_bounds__(kOneThreads)
+    k_scan_one(const TI *__restrict__ in, int64_t n, TO *__restrict__ out) {
+  __shared__ TO sums[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t base = (int64_t)threadIdx.x * kScanItems;
+  TO v[kScanItems];
+  TO acc = 0;
+#pragma unroll
+  for (int r = 0; r < kScanItems; ++r) {
+    v[r] = base + r < n ? (TO)in[base + r] : TO(0);
+    acc += v[r];
+  }
+  const TO inc = warp_incl_scan(acc);
+  if (lane == 31) sums[wid] = inc;
+  __syncthreads();
+  if (wid == 0) {
+    const TO w = sums[lane];
+    sums[lane] = warp_incl_scan(w) - w;
+  }
+  __syncthreads();
+  TO ex = inc - acc + sums[wid];
+#pragma unroll
+  for (int r = 0; r < kScanItems; ++r) {
+    if (base + r < n) out[base + r] = ex;
+    ex += v[r];
+  }
+  if (threadIdx.x == kOneThreads - 1) out[n] = ex;
+}
+
 template <class TI, class TO>
 void exscan_impl(const TI *in, TO *out, int64_t n, Arena &ar, cudaStream_t s) {
   if (n == 0) {
     BST_CUDA(cudaMemsetAsync(out, 0, sizeof(TO), s));
+    return;
+  }
+  if (n <= kOneTile) {
+    k_scan_one<TI, TO><<<1, kOneThreads, 0, s>>>(in, n, out);
+    BST_CHECK_LAUNCH();
     return;
   }
   int64_t nt = (n + kScanTile - 1) / kScanTile;
@@ -234,21 +272,35 @@ void iota_i32(int32_t *p, int64_t n, cudaStream_t s) {
   k_iota<<<nblk(n, 256), 256, 0, s>>>(p, n);
   BST_CHECK_LAUNCH();
 }
-__global__ void k_copy_bytes(unsigned char *__restrict__ dst, const unsigned char *__restrict__ src,
-                             int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = src[i];
-}
+// The copies of a ReadBack or an Upload, up to kCopyItems per launch (one row of CTAs each;
+// a launch per item was a fifth of the launches of a small plan): 16-byte words where both
+// ends are 16-byte aligned, the rest byte by byte.
+constexpr int kCopyItems = 16;
+struct CopyItems {
+  unsigned char *dst[kCopyItems];
+  const unsigned char *src[kCopyItems];
+  int64_t n[kCopyItems];
+};
 
-// n bytes, both ends 16-byte aligned: 16-byte words, then the tail byte by byte
-__global__ void k_copy_aligned(unsigned char *__restrict__ dst, const unsigned char *__restrict__ src,
-                               int64_t n) {
-  const int64_t nw = n >> 4, stride = (int64_t)gridDim.x * blockDim.x;
+__global__ void k_copy_items(CopyItems C) {
+  unsigned char *dst = C.dst[blockIdx.y];
+  const unsigned char *src = C.src[blockIdx.y];
+  const int64_t n = C.n[blockIdx.y], stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool aligned = ((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0;
+  const int64_t nw = aligned ? n >> 4 : 0;
   for (int64_t i = i0; i < nw; i += stride)
     reinterpret_cast<uint4 *>(dst)[i] = reinterpret_cast<const uint4 *>(src)[i];
   for (int64_t i = (nw << 4) + i0; i < n; i += stride) dst[i] = src[i];
+}
+
+static void copy_items(const CopyItems &C, int count, cudaStream_t s) {
+  if (count == 0) return;
+  int64_t most = 0;
+  for (int i = 0; i < count; ++i) most = std::max(most, C.n[i]);
+  const int blocks = (int)std::min<int64_t>(512, (most + 4095) / 4096);
+  k_copy_items<<<dim3((unsigned)std::max(blocks, 1), (unsigned)count), 256, 0, s>>>(C);
+  BST_CHECK_LAUNCH();
 }
 
 ReadBack::ReadBack(bst_ctx *c, cudaStream_t st) : ctx(c), s(st) {
@@ -288,18 +340,25 @@ void ReadBack::add(void *host_dst, const void *dev_src, size_t bytes) {
     ctx->rb_cap = cap;
     return add(host_dst, dev_src, bytes);
   }
-  void *dev_view = nullptr;
-  BST_CUDA(cudaHostGetDevicePointer(&dev_view, ctx->rb_host, 0));
-  const int64_t n = (int64_t)bytes;
-  const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, 1024);
-  k_copy_bytes<<<blocks, 256, 0, s>>>(static_cast<unsigned char *>(dev_view) + off,
-                                      static_cast<const unsigned char *>(dev_src), n);
-  BST_CHECK_LAUNCH();
-  items.push_back({host_dst, off, bytes});
+  items.push_back({host_dst, dev_src, off, bytes});
   used = off + bytes;
 }
 
 void ReadBack::finish() {
+  void *dev_view = nullptr;
+  if (!items.empty()) BST_CUDA(cudaHostGetDevicePointer(&dev_view, ctx->rb_host, 0));
+  CopyItems C;
+  int count = 0;
+  for (const Item &it : items) {
+    C.dst[count] = static_cast<unsigned char *>(dev_view) + it.off;
+    C.src[count] = static_cast<const unsigned char *>(it.src);
+    C.n[count] = (int64_t)it.bytes;
+    if (++count == kCopyItems) {
+      copy_items(C, count, s);
+      count = 0;
+    }
+  }
+  copy_items(C, count, s);
   BST_CUDA(cudaStreamSynchronize(s));
   for (const Item &it : items)
     std::memcpy(it.dst, static_cast<const char *>(ctx->rb_host) + it.off, it.bytes);
@@ -398,19 +457,18 @@ void Upload::flush() {
 void Upload::launch() {
   void *dev_view = nullptr;
   BST_CUDA(cudaHostGetDevicePointer(&dev_view, ctx->up_host, 0));
+  CopyItems C;
+  int count = 0;
   for (const Item &it : items) {
-    const int64_t n = (int64_t)it.bytes;
-    unsigned char *dst = static_cast<unsigned char *>(it.dst);
-    const unsigned char *src = static_cast<const unsigned char *>(dev_view) + it.off;
-    if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
-      const unsigned blocks = (unsigned)std::min<int64_t>((n / 16 + 255) / 256 + 1, 1024);
-      k_copy_aligned<<<blocks, 256, 0, s>>>(dst, src, n);
-    } else {
-      const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, 1024);
-      k_copy_bytes<<<blocks, 256, 0, s>>>(dst, src, n);
+    C.dst[count] = static_cast<unsigned char *>(it.dst);
+    C.src[count] = static_cast<const unsigned char *>(dev_view) + it.off;
+    C.n[count] = (int64_t)it.bytes;
+    if (++count == kCopyItems) {
+      copy_items(C, count, s);
+      count = 0;
     }
-    BST_CHECK_LAUNCH();
   }
+  copy_items(C, count, s);
 }
 
 void fill_i32(int32_t *p, int32_t v, int64_t n, cudaStream_t s) {
