@@ -83,6 +83,7 @@ __device__ inline int f64_split_of(int32_t *__restrict__ d, const int4 *__restri
 // inner split.
 struct TailCost {
   int t[2];
+  unsigned inv[2];  // ceil(2^16 / t): n / t = n inv >> 16 for n < 4096 and t <= 16
   long long c[2], w1;
 };
 
@@ -92,14 +93,18 @@ __device__ __forceinline__ TailCost tail_cost(int mn, int smax) {
   C.t[0] = rem ? min(32 / rem, min(smax, kMaxSplit)) : 1;
   C.t[1] = (C.t[0] + 1) >> 1;
   C.w1 = 0;
-  for (int i = 0; i < 2; ++i) C.c[i] = 32 - __clz(C.t[i] - 1);  // ceil(log2 t)
+  for (int i = 0; i < 2; ++i) {
+    C.c[i] = 32 - __clz(C.t[i] - 1);  // ceil(log2 t)
+    C.inv[i] = (65535 + C.t[i]) / C.t[i];
+  }
   return C;
 }
 
 __device__ __forceinline__ void tail_add(TailCost &C, int w) {
   C.w1 += w;
-  C.c[0] += (w + C.t[0] - 1) / C.t[0];
-  C.c[1] += (w + C.t[1] - 1) / C.t[1];
+  // panels are at most a slot wide, w <= kWideSlot
+  C.c[0] += ((unsigned)(w + C.t[0] - 1) * C.inv[0]) >> 16;
+  C.c[1] += ((unsigned)(w + C.t[1] - 1) * C.inv[1]) >> 16;
 }
 
 // FP64 instructions of the unsplit tile
