@@ -388,17 +388,15 @@ __device__ __forceinline__ double i64_ldexp(long long v, int e2) {
   return __longlong_as_double(bits + ((long long)e2 << 52));
 }
 
-// FP32 -> FP64 from the binary32 / binary64 encodings (normal numbers and zero; FP32
-// subnormals flush to zero), integer operations only
+// FP32 -> FP64 from the binary32 / binary64 encodings (FP32 subnormals flush to zero),
+// integer operations only.  Infinities and NaN too: a hardware conversion for them alone was
+// executed for every element, and the FP64 pipe, 16 cycles a warp instruction, was the 3xTF32
+// kernel's busiest (54 %).
 __device__ __forceinline__ double f32_to_f64(float f) {
-  const unsigned b = __float_as_uint(f);
-  const unsigned ex = (b >> 23) & 0xffu;
-  if (ex == 0) return 0.0;
-  if (ex == 0xffu) return (double)f;
-  const unsigned long long bits = ((unsigned long long)(b >> 31) << 63) |
-                                  ((unsigned long long)(ex - 127 + 1023) << 52) |
-                                  ((unsigned long long)(b & 0x7fffffu) << 29);
-  return __longlong_as_double((long long)bits);
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  const unsigned bias = m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
+  if (m < 0x00800000u) return 0.0;
+  return __hiloint2double((int)(((m >> 3) + bias) | (b & 0x80000000u)), (int)(b << 29));
 }
 
 __device__ __forceinline__ long long round_shift(long long v, int sh) {
@@ -914,18 +912,16 @@ __global__ void __launch_bounds__(256, 2)
 // runs each in passes of 16 rows x 24 columns of the (possibly transposed) block, where one
 // 16-byte load gives a lane the high and low parts of a fragment.  There is one pass body of
 // runtime size: bodies per tile count filled the instruction cache (5.6 of 13 cycles per
-// instruction waited for it; 5.86 ms on the 2000 x 2000 banded product at 2 % against 3.58
-// now, and 7.74 with a warp per 16 x 16 tile walking the stacks); loading the next fragments
-// during the current MMAs costs spills (4.24 ms), three CTAs per SM measure the same (3.65).
-// The sums leave through shared memory, so that the FP64 adds,
-// 16 cycles a warp instruction, run on full warps and the stores are contiguous.  Per element
-// the MMAs and sums run in the order entry, chunk, {a_lo b_hi, a_hi b_lo, a_hi b_hi}
-// whatever the tile orientation.
+// instruction waited for it; 5.86 ms on the 2000 x 2000 banded product at 2 % against 3.22
+// now, and 7.74 with a warp per 16 x 16 tile walking the stacks).  Instructions are what to
+// save: operand rows past a pass's edge are read again instead of predicated, a block's first
+// product is its sum without a TwoSum.  Loading the next fragments during the current MMAs
+// costs spills (4.24 ms), staging them through shared memory instructions and warps (4.37),
+// three CTAs per SM spills again (3.42).  The sums leave through shared memory, so that the
+// FP64 adds, 16 cycles a warp instruction, run on full warps and the stores are contiguous.
+// Per element the MMAs and sums run in the order entry, chunk, {a_lo b_hi, a_hi b_lo,
+// a_hi b_hi} whatever the tile orientation.
 constexpr int kTfPitch = 8 * kTfCols + 1;  // float2 per row of the pass in shared memory
-
-__device__ __forceinline__ float4 ld16f(const float4 *p, bool ok) {
-  return ok ? __ldg(p) : make_float4(0.f, 0.f, 0.f, 0.f);
-}
 
 __device__ __forceinline__ void mma_tf32f(float (&d)[4], float a0, float a1, float a2, float a3,
                                           float b0, float b1) {
@@ -935,10 +931,6 @@ __device__ __forceinline__ void mma_tf32f(float (&d)[4], float a0, float a1, flo
 
 struct TfBlk {
   int off, eb, ne, cin, m, n, sw;
-};
-
-struct TfFrag {
-  float4 a0, a1, b[kTfCols];
 };
 
 // the pass from row r00, column c00 of the block (of its transpose when it runs swapped)
@@ -957,80 +949,68 @@ __device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, in
   for (int j = 0; j < kTfCols; ++j)
 #pragma unroll
     for (int h = 0; h < 4; ++h) hi[j][h] = lo[j][h] = acc[j][h] = 0.f;
-  const float4 *x0, *y0;
-  int rs = 0;  // float4 per operand row: 4 per chunk of 8
-  auto entry = [&](const int4 &e, int j) {
-    const unsigned ea = (unsigned)__shfl_sync(kFull, e.x, j);
-    const unsigned eb = (unsigned)__shfl_sync(kFull, e.y, j);
-    rs = 4 * __shfl_sync(kFull, e.z, j);
-    x0 = X + 4 * (size_t)(b.sw ? eb : ea) + ((int64_t)(r00 + g) * rs + t);
-    y0 = Y + 4 * (size_t)(b.sw ? ea : eb) + ((int64_t)(c00 + g) * rs + t);
-  };
-  auto load = [&](TfFrag &f, int ch) {
-    const float4 *x = x0 + 4 * ch, *y = y0 + 4 * ch;
-    f.a0 = ld16f(x, g < rows);
-    f.a1 = ld16f(x + 8 * (int64_t)rs, g + 8 < rows);
+  // the lane's operand rows and columns; past the pass's edge it reads the last one again
+  // (an output depends on its own row and column only, and those outputs are not stored)
+  const int ra0 = r00 + min(g, rows - 1), ra1 = r00 + min(g + 8, rows - 1);
+  int cb[kTfCols];
 #pragma unroll
-    for (int j = 0; j < kTfCols; ++j) {
-      f.b[j] = ld16f(y, g + 8 * j < cols);
-      y += 8 * (int64_t)rs;
-    }
-  };
-  if (b.ne > 0) {
-    int4 ent = ent0;
-    int left = b.ne, g0 = 0, j = 0, ch = 0;
-    entry(ent, 0);
-    int nch = rs >> 2;
-    TfFrag cur;
-    load(cur, 0);
+  for (int q = 0; q < kTfCols; ++q) cb[q] = c00 + min(g + 8 * q, cols - 1);
+  int4 ent = ent0;
+  for (int e = 0; e < b.ne; ++e) {
+    if (e > 0 && (e & 31) == 0)
+      ent = e + lane < b.ne ? P.ents[(int64_t)b.eb + e + lane] : make_int4(0, 0, 0, 0);
+    const unsigned ea = (unsigned)__shfl_sync(kFull, ent.x, e & 31);
+    const unsigned eb = (unsigned)__shfl_sync(kFull, ent.y, e & 31);
+    const int rs = 4 * __shfl_sync(kFull, ent.z, e & 31);  // float4 per row: 4 per chunk of 8
+    const float4 *x = X + 4 * (size_t)(b.sw ? eb : ea) + t, *y = Y + 4 * (size_t)(b.sw ? ea : eb) + t;
+    const float4 *x0 = x + (int64_t)ra0 * rs, *x1 = x + (int64_t)ra1 * rs;
+    const float4 *yq[kTfCols];
+#pragma unroll
+    for (int q = 0; q < kTfCols; ++q) yq[q] = y + (int64_t)cb[q] * rs;
 #pragma unroll 1
-    for (;;) {
-      const bool last = ch + 1 == nch;  // last chunk of this product
-      if (last) {
-        ch = 0;
-        if (--left > 0) {
-          if (++j == 32) {
-            g0 += 32;
-            j = 0;
-            ent = g0 + lane < b.ne ? P.ents[(int64_t)b.eb + g0 + lane] : make_int4(0, 0, 0, 0);
-          }
-          entry(ent, j);
-          nch = rs >> 2;
-        }
-      } else {
-        ++ch;
-      }
+    for (int o = 0; o < rs; o += 4) {
+      const float4 a0 = __ldg(x0 + o), a1 = __ldg(x1 + o);
+      float4 f[kTfCols];
+#pragma unroll
+      for (int q = 0; q < kTfCols; ++q)
+        if (8 * q < cols) f[q] = __ldg(yq[q] + o);
 #pragma unroll
       for (int q = 0; q < kTfCols; ++q) {
         if (8 * q >= cols) break;
-        const float4 &a0 = cur.a0, &a1 = cur.a1, &bb = cur.b[q];
         if (b.sw) {  // rows are op(B)'s: its high part times op(A)'s low part first
-          mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, bb.z, bb.w);
-          mma_tf32f(acc[q], a0.z, a1.z, a0.w, a1.w, bb.x, bb.y);
+          mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, f[q].z, f[q].w);
+          mma_tf32f(acc[q], a0.z, a1.z, a0.w, a1.w, f[q].x, f[q].y);
         } else {
-          mma_tf32f(acc[q], a0.z, a1.z, a0.w, a1.w, bb.x, bb.y);
-          mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, bb.z, bb.w);
+          mma_tf32f(acc[q], a0.z, a1.z, a0.w, a1.w, f[q].x, f[q].y);
+          mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, f[q].z, f[q].w);
         }
-        mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, bb.x, bb.y);
+        mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, f[q].x, f[q].y);
       }
-      if (last) {
+    }
+    if (e == 0) {  // 0 + v: the low part is 0 (NaN where v is not finite)
 #pragma unroll
-        for (int q = 0; q < kTfCols; ++q) {
-          if (8 * q >= cols) break;
+      for (int q = 0; q < kTfCols; ++q)
 #pragma unroll
-          for (int h = 0; h < 4; ++h) {
-            const float a = hi[q][h], v = acc[q][h];
-            const float sum = __fadd_rn(a, v);
-            const float bb = __fsub_rn(sum, a);
-            const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bb)), __fsub_rn(v, bb));
-            hi[q][h] = sum;
-            lo[q][h] = __fadd_rn(lo[q][h], err);
-            acc[q][h] = 0.f;
-          }
+        for (int h = 0; h < 4; ++h) {
+          hi[q][h] = __fadd_rn(0.f, acc[q][h]);
+          lo[q][h] = __fsub_rn(acc[q][h], acc[q][h]);
+          acc[q][h] = 0.f;
         }
+      continue;
+    }
+#pragma unroll
+    for (int q = 0; q < kTfCols; ++q) {
+      if (8 * q >= cols) break;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const float a = hi[q][h], v = acc[q][h];
+        const float sum = __fadd_rn(a, v);
+        const float bb = __fsub_rn(sum, a);
+        const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bb)), __fsub_rn(v, bb));
+        hi[q][h] = sum;
+        lo[q][h] = __fadd_rn(lo[q][h], err);
+        acc[q][h] = 0.f;
       }
-      if (left == 0) break;
-      load(cur, ch);
     }
   }
 #pragma unroll
@@ -1047,25 +1027,30 @@ __device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, in
   const int ni = b.sw ? rows : cols, total = rows * cols;
   const int so = b.sw ? 1 : kTfPitch, si = b.sw ? kTfPitch : 1;
   const int di = 32 % ni, dO = 32 / ni;
-  int y = lane / ni, x = lane - y * ni;
+  int x = lane % ni;
+  const float2 *from = sm + (lane / ni) * so + x * si;
+  int64_t at = c0 + (int64_t)(lane / ni) * b.n + x;
+  const int sstep = dO * so + di * si, swrap = so - ni * si;
+  const int64_t cstep = (int64_t)dO * b.n + di, cwrap = b.n - ni;
 #pragma unroll 1
   for (int o = lane; o - lane < total; o += 32) {
-    const float2 v2 = o < total ? sm[y * so + x * si] : make_float2(0.f, 0.f);
+    const float2 v2 = o < total ? *from : make_float2(0.f, 0.f);
     // the FP64 add only where some low part is not zero (a NaN is not): blocks of one
     // product have none
     double v = f32_to_f64(v2.x);
     if (__any_sync(kFull, v2.y != 0.f)) v += f32_to_f64(v2.y);
     if (o < total) {
-      const int64_t at = c0 + (int64_t)y * b.n + x;
       if (!P.alpha_one) v *= P.alpha;
       if (ci) v = fma(P.beta, ci[at], v);
       P.C[b.off + at] = v;
     }
-    y += dO;
+    from += sstep;
+    at += cstep;
     x += di;
     if (x >= ni) {
       x -= ni;
-      ++y;
+      from += swrap;
+      at += cwrap;
     }
   }
   __syncwarp();
