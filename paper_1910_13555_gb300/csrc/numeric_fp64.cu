@@ -1130,8 +1130,8 @@ void sort_items(const int64_t *items, const int32_t *keys, int64_t n, int64_t *o
 }
 
 // Tiles, entries, descriptors and slot size of the staged kernel; false (stage_elems
-// stays 0) when a block size does not fit the descriptor's 12 bits or a row of C (n
-// elements) exceeds one output tile.
+// stays 0) when a block size does not fit the descriptor's 12 bits, an inner size the
+// entries' 15, or a row of C (n elements) exceeds one output tile.
 static std::vector<int32_t> class_split_bounds(const bst_plan *p);
 static void apply_split_gate(bst_plan *p, const unsigned long long sums[2], cudaStream_t s);
 
@@ -1188,6 +1188,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
       // panels of about equal width (a narrow last one would cost a whole job); of whole
       // slabs when read in place
       const int64_t k = p->k_vals[kc];
+      if (k >= (1 << 15)) return false;  // an entry holds the stored row strides in 16 bits
       int64_t w = k, panels = 1;
       if (k > wmax) {
         const int64_t np = (k + wmax - 1) / wmax;
