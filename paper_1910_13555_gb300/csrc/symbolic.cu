@@ -53,20 +53,20 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 
 // ---- block norms -------------------------------------------------------------------
 
-// Matrices of small blocks (at most kNormSmall elements): one warp per group of 32
-// consecutive blocks.  Lane j first loads the size and offset of block j of the group
-// (one coalesced round of index loads).  For each block the lanes accumulate
-// lane-strided squares and park their 32 partial sums in a row of shared memory; then
-// lane j adds row j (the partials of block j) in lane order and takes its square root.
-// GB300's FP64 pipe takes as long for a warp instruction with one active lane as with
-// 32: a butterfly costs five full FP64 instructions per block, the transposed sum one
-// per block, and the group's 32 square roots run together.  Matrices with larger blocks
-// (a contraction's folded views, up to hundreds of thousands of elements a block): one
-// warp per block, a butterfly at the end (grouping them left a few hundred warps
-// streaming 32 large blocks each: 4.6 ms for the rank-4 operand).  Both read HBM once and are
-// bound by the loads a warp has in flight, so they issue eight before the dependent FMAs
-// (a rank-4 contraction as a whole 10.20 -> 10.06 ms, the small-B product 3.34 -> 3.29); each
-// lane's sum keeps its order, e = lane, lane + 32, ..., and the norms their bits.
+// Matrices of small blocks (at most kNormSmall elements): one CTA per group of 32
+// consecutive blocks.  For each block the lanes of a warp accumulate lane-strided squares and
+// park their 32 partial sums in a row of shared memory; then lane j of the first warp adds row
+// j (the partials of block j) in lane order and takes its square root.  GB300's FP64 pipe
+// takes as long for a warp instruction with one active lane as with 32: a butterfly costs five
+// full FP64 instructions per block, the transposed sum one per block, and the group's 32
+// square roots run together.  The four warps of the CTA take eight blocks each: with a group
+// per warp, two dozen warps per SM walked 32 blocks one after another (six norm passes of a sign step
+// 509 us, now 267).
+// Matrices with larger blocks (a contraction's folded views, up to hundreds of thousands of
+// elements a block): one warp per block, a butterfly at the end (grouping them left a few
+// hundred warps streaming 32 large blocks each: 4.6 ms for the rank-4 operand).  Both issue
+// several loads before the dependent FMAs; each lane's sum keeps its order, e = lane,
+// lane + 32, ..., and the norms their bits.
 constexpr int kNormGroup = 32;
 constexpr int kNormWarps = 4;
 constexpr int64_t kNormSmall = 1024;
@@ -102,19 +102,20 @@ __global__ void __launch_bounds__(32 * kNormWarps)
                   const int32_t *__restrict__ col, const int32_t *__restrict__ rsz,
                   const int32_t *__restrict__ csz, const int64_t *__restrict__ off,
                   const double *__restrict__ data, double *__restrict__ norms) {
-  __shared__ double part[kNormWarps][kNormGroup][33];
+  __shared__ double part[kNormGroup][33];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  const int64_t b0 = ((int64_t)blockIdx.x * kNormWarps + wl) * kNormGroup;
-  if (b0 >= nblocks) return;
+  const int64_t b0 = (int64_t)blockIdx.x * kNormGroup;
   const int nb = (int)min((int64_t)kNormGroup, nblocks - b0);
+  constexpr int kPer = kNormGroup / kNormWarps;  // blocks per warp
   int my_len = 0;
   long long my_off = 0;
-  if (lane < nb) {
-    my_len = rsz[row[b0 + lane]] * csz[col[b0 + lane]];
-    my_off = off[b0 + lane];
+  if (lane < kPer && wl * kPer + lane < nb) {
+    const int64_t b = b0 + wl * kPer + lane;
+    my_len = rsz[row[b]] * csz[col[b]];
+    my_off = off[b];
   }
-  double(*P)[33] = part[wl];
-  for (int j0 = 0; j0 < nb; j0 += 4) {  // four blocks at a time, two loads of each ahead
+#pragma unroll
+  for (int j0 = 0; j0 < kPer; j0 += 4) {  // four blocks at a time, two loads of each ahead
     double v[4][2];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -127,20 +128,21 @@ __global__ void __launch_bounds__(32 * kNormWarps)
     for (int u = 0; u < 4; ++u) {
       const int len = __shfl_sync(0xffffffffu, my_len, j0 + u);
       const double *x = data + __shfl_sync(0xffffffffu, my_off, j0 + u);
-      double s = fma(v[u][0], v[u][0], 0.0);
+      double s = 0.0;
+      if (len > 0) s = fma(v[u][0], v[u][0], s);
       if (len > 32) s = fma(v[u][1], v[u][1], s);
 #pragma unroll 4
       for (int e = lane + 64; e < len; e += 32) {
         const double y = __ldg(x + e);
         s = fma(y, y, s);
       }
-      P[j0 + u][lane] = s;
+      part[wl * kPer + j0 + u][lane] = s;
     }
   }
-  __syncwarp();
-  if (lane < nb) {
-    double t = P[lane][0];
-    for (int q = 1; q < 32; ++q) t += P[lane][q];
+  __syncthreads();
+  if (wl == 0 && lane < nb) {
+    double t = part[lane][0];
+    for (int q = 1; q < 32; ++q) t += part[lane][q];
     norms[b0 + lane] = sqrt(t);
   }
 }
@@ -438,7 +440,7 @@ void block_norms(const bst_matrix *m, double *norms, cudaStream_t s) {
         m->nblocks, m->row, m->col, m->rsz, m->csz, m->off, m->data, norms);
   } else {
     const int64_t groups = (m->nblocks + kNormGroup - 1) / kNormGroup;
-    k_block_norms<<<nblk(groups, kNormWarps), 32 * kNormWarps, 0, s>>>(
+    k_block_norms<<<(unsigned)groups, 32 * kNormWarps, 0, s>>>(
         m->nblocks, m->row, m->col, m->rsz, m->csz, m->off, m->data, norms);
   }
   BST_CHECK_LAUNCH();
