@@ -138,8 +138,13 @@ struct PermArgs {
 // One CTA per tensor block: its elements are visited in view order, which reads (or
 // writes) the tensor layout out of order; with one block in flight per CTA (a few per
 // SM) its lines stay in L1 / L2 until every element is used.  A warp per block, with
-// dozens of blocks of up to ~175 KB in flight per SM, re-fetched them from DRAM.
-__global__ void k_permute(PermArgs P) {
+// dozens of blocks of up to ~175 KB in flight per SM, re-fetched them from DRAM.  An element
+// costs a few instructions per mode, so the kernel is specialised for the rank (all eight
+// possible modes cost as much as the memory), and a thread has four loads in flight: the three
+// permutations of a rank-3 contraction with its gradients 1.89 -> 1.07 ms, those of a rank-4
+// contraction 1.45 -> 1.26.
+template <int RANK>
+__global__ void __launch_bounds__(kPermThreads) k_permute(PermArgs P) {
   const int64_t q = blockIdx.x;
   if (q >= P.nblocks) return;
   const int64_t tb = P.tblk ? P.tblk[q] : q;
@@ -159,13 +164,13 @@ __global__ void k_permute(PermArgs P) {
   // digits over the view's modes (slowest first): decoded once by division, then
   // advanced by the step's own digits with one carry per mode (an element costs a few
   // adds instead of one division per mode)
-  // (loops over all kMaxRank modes with the unused ones as size-1 modes, so that the
-  // digit arrays live in registers)
-  int32_t dig[kMaxRank], inc[kMaxRank], sv[kMaxRank], tv[kMaxRank];
+  // (loops over RANK modes with the unused ones as size-1 modes, so that the digit arrays
+  // live in registers)
+  int32_t dig[RANK], inc[RANK], sv[RANK], tv[RANK];
   {
-    int32_t rem = (int32_t)threadIdx.x, stp = (int32_t)blockDim.x;
+    int32_t rem = (int32_t)threadIdx.x, stp = kPermThreads;
 #pragma unroll
-    for (int j = kMaxRank - 1; j >= 0; --j) {
+    for (int j = RANK - 1; j >= 0; --j) {
       const bool used = j < P.rank;
       const int d = used ? P.ord[j] : 0;
       sv[j] = used ? s[d] : 1;
@@ -176,22 +181,48 @@ __global__ void k_permute(PermArgs P) {
       stp /= sv[j];
     }
   }
-  for (int32_t e = threadIdx.x; e < len; e += blockDim.x) {
-    int32_t src = 0;
+  // the element's place in the tensor block, and the digits of the thread's next element
+  auto next = [&]() -> int32_t {
+    int32_t src = 0, carry = 0;
 #pragma unroll
-    for (int j = 0; j < kMaxRank; ++j) src += dig[j] * tv[j];
-    if (P.to_view)
-      P.dst[vo + e] = P.src[to + src];
-    else
-      P.dst[to + src] = P.src[vo + e];
-    int32_t carry = 0;
+    for (int j = 0; j < RANK; ++j) src += dig[j] * tv[j];
 #pragma unroll
-    for (int j = kMaxRank - 1; j >= 0; --j) {
+    for (int j = RANK - 1; j >= 0; --j) {
       const int32_t v = dig[j] + inc[j] + carry;
       carry = v >= sv[j];
       dig[j] = carry ? v - sv[j] : v;
     }
+    return src;
+  };
+  const double *from = P.src + (P.to_view ? to : vo);
+  double *dst = P.dst + (P.to_view ? vo : to);
+  int32_t e = threadIdx.x;
+  for (; e + 3 * kPermThreads < len; e += 4 * kPermThreads) {
+    int32_t at[4];
+    double v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      at[u] = next();
+      v[u] = from[P.to_view ? at[u] : e + u * kPermThreads];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) dst[P.to_view ? e + u * kPermThreads : at[u]] = v[u];
   }
+  for (; e < len; e += kPermThreads) {
+    const int32_t at = next();
+    dst[P.to_view ? e : at] = from[P.to_view ? at : e];
+  }
+}
+
+void launch_permute(const PermArgs &P, cudaStream_t s) {
+  const unsigned n = (unsigned)P.nblocks;
+  if (P.rank <= 3)
+    k_permute<3><<<n, kPermThreads, 0, s>>>(P);
+  else if (P.rank == 4)
+    k_permute<4><<<n, kPermThreads, 0, s>>>(P);
+  else
+    k_permute<kMaxRank><<<n, kPermThreads, 0, s>>>(P);
+  BST_CHECK_LAUNCH();
 }
 
 // R tuple of every C block: decode folded row / column, reorder by result_order
@@ -396,8 +427,7 @@ void permute_view(const View &V, const double *src, double *dst, bool to_view, c
   P.src = src;
   P.dst = dst;
   P.to_view = to_view;
-  k_permute<<<(unsigned)P.nblocks, kPermThreads, 0, s>>>(P);
-  BST_CHECK_LAUNCH();
+  launch_permute(P, s);
 }
 
 // Slab reading of T1 (the second remap of a non-fold view).  When T1's modes are stored
@@ -524,8 +554,7 @@ void contract_finish(bst_plan *p, cudaStream_t s) {
   P.src = K.cbuf;
   P.dst = K.R->data;
   P.to_view = 0;
-  k_permute<<<(unsigned)P.nblocks, kPermThreads, 0, s>>>(P);
-  BST_CHECK_LAUNCH();
+  launch_permute(P, s);
 }
 
 // adjoint of a contraction: dR (tensor layout) -> dC, matrix adjoint, views -> tensors
@@ -548,8 +577,7 @@ void contract_adjoint(bst_plan *p, const double *dR, double *dT1, double *dT2, d
     P.src = dR;
     P.dst = K.dcbuf;
     P.to_view = 1;
-    k_permute<<<(unsigned)P.nblocks, kPermThreads, 0, s>>>(P);
-    BST_CHECK_LAUNCH();
+    launch_permute(P, s);
     dC = K.dcbuf;
   }
   // view-layout gradients: straight into the tensors when zero-copy, else through a
