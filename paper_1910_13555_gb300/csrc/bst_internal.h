@@ -191,6 +191,9 @@ namespace bst {
 
 // exclusive scan of n int32 counts into int64 (out has n + 1 entries, out[n] = total)
 void exscan_i32_i64(const int32_t *in, int64_t *out, int64_t n, Arena &ar, cudaStream_t s);
+// three of them of the same length
+void exscan3_i32_i64(const int32_t *const (&in)[3], int64_t *const (&out)[3], int64_t n, Arena &ar,
+                     cudaStream_t s);
 // exclusive scan int64 -> int64 (n + 1 outputs)
 void exscan_i64(const int64_t *in, int64_t *out, int64_t n, Arena &ar, cudaStream_t s);
 // exclusive scan int32 -> int32 (n + 1 outputs); caller guarantees no overflow

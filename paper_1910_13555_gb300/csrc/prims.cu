@@ -107,9 +107,13 @@ __global__ void k_tile_scan(const TI *__restrict__ in, int64_t n, const TO *__re
 // the whole scan by one CTA: three launches on a few thousand elements are mostly latency
 constexpr int kOneThreads = 1024, kOneTile = kOneThreads * kScanItems;
 
+// (one CTA per array: up to three of the same length at once)
 template <class TI, class TO>
 __global__ void __launch_bounds__(kOneThreads)
-    k_scan_one(const TI *__restrict__ in, int64_t n, TO *__restrict__ out) {
+    k_scan_one(const TI *__restrict__ in0, const TI *__restrict__ in1, const TI *__restrict__ in2,
+               int64_t n, TO *__restrict__ out0, TO *__restrict__ out1, TO *__restrict__ out2) {
+  const TI *in = blockIdx.x == 0 ? in0 : blockIdx.x == 1 ? in1 : in2;
+  TO *out = blockIdx.x == 0 ? out0 : blockIdx.x == 1 ? out1 : out2;
   __shared__ TO sums[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t base = (int64_t)threadIdx.x * kScanItems;
@@ -144,7 +148,7 @@ void exscan_impl(const TI *in, TO *out, int64_t n, Arena &ar, cudaStream_t s) {
     return;
   }
   if (n <= kOneTile) {
-    k_scan_one<TI, TO><<<1, kOneThreads, 0, s>>>(in, n, out);
+    k_scan_one<TI, TO><<<1, kOneThreads, 0, s>>>(in, in, in, n, out, out, out);
     BST_CHECK_LAUNCH();
     return;
   }
@@ -208,6 +212,60 @@ __global__ void k_part_scatter(const int32_t *__restrict__ keys, int64_t n, int6
   }
 }
 
+// The whole partition by one CTA, for short inputs: five launches otherwise.  Each of the 32
+// warps owns a segment; its key counts, scanned in (key, segment) order, become its write
+// cursors.
+constexpr int kOnePartKeys = 256, kOnePartItems = 8192;
+
+__global__ void __launch_bounds__(1024)
+    k_part_one(const int32_t *__restrict__ keys, int n, int nkeys, int32_t *__restrict__ perm,
+               int32_t *__restrict__ key_ptr) {
+  __shared__ int32_t cur[kOnePartKeys * 32];
+  __shared__ int32_t sums[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int cells = nkeys * 32;
+  for (int i = threadIdx.x; i < cells; i += 1024) cur[i] = 0;
+  __syncthreads();
+  const int L = (n + 31) / 32, p0 = min(w * L, n), p1 = min(p0 + L, n);
+  for (int p = p0 + lane; p < p1; p += 32) atomicAdd(&cur[keys[p] * 32 + w], 1);
+  __syncthreads();
+  // exclusive scan of the cells, cells / 1024 (at most 8) consecutive ones per thread
+  const int per = (cells + 1023) / 1024, c0 = threadIdx.x * per;
+  int acc = 0;
+  for (int i = c0; i < min(c0 + per, cells); ++i) acc += cur[i];
+  const int inc = warp_incl_scan(acc);
+  if (lane == 31) sums[w] = inc;
+  __syncthreads();
+  if (w == 0) {
+    const int v = sums[lane];
+    sums[lane] = warp_incl_scan(v) - v;
+  }
+  __syncthreads();
+  int ex = inc - acc + sums[w];
+  for (int i = c0; i < min(c0 + per, cells); ++i) {
+    const int v = cur[i];
+    cur[i] = ex;
+    if ((i & 31) == 0) key_ptr[i >> 5] = ex;
+    ex += v;
+  }
+  if (threadIdx.x == 0) key_ptr[nkeys] = n;
+  __syncthreads();
+  for (int b = p0; b < p1; b += 32) {
+    const int p = b + lane;
+    const unsigned act = __ballot_sync(0xffffffffu, p < p1);
+    int cell = 0;
+    unsigned peers = 0;
+    if (p < p1) {
+      cell = keys[p] * 32 + w;
+      peers = __match_any_sync(act, cell);
+      perm[cur[cell] + __popc(peers & ((1u << lane) - 1u))] = p;
+    }
+    __syncwarp();
+    if (p < p1 && (int)(__ffs(peers) - 1) == lane) cur[cell] += __popc(peers);
+    __syncwarp();
+  }
+}
+
 // digit of key[perm[i]] (perm null: key[i]): its `bits` low bits, or those above them
 __global__ void k_key_digit(const int32_t *__restrict__ keys, const int32_t *__restrict__ perm,
                             int64_t n, int bits, int high, int32_t *__restrict__ dig) {
@@ -259,6 +317,16 @@ inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 void exscan_i32_i64(const int32_t *in, int64_t *out, int64_t n, Arena &ar, cudaStream_t s) {
   exscan_impl<int32_t, int64_t>(in, out, n, ar, s);
+}
+void exscan3_i32_i64(const int32_t *const (&in)[3], int64_t *const (&out)[3], int64_t n, Arena &ar,
+                     cudaStream_t s) {
+  if (n == 0 || n > kOneTile) {
+    for (int i = 0; i < 3; ++i) exscan_i32_i64(in[i], out[i], n, ar, s);
+    return;
+  }
+  k_scan_one<int32_t, int64_t><<<3, kOneThreads, 0, s>>>(in[0], in[1], in[2], n, out[0], out[1],
+                                                         out[2]);
+  BST_CHECK_LAUNCH();
 }
 void exscan_i64(const int64_t *in, int64_t *out, int64_t n, Arena &ar, cudaStream_t s) {
   exscan_impl<int64_t, int64_t>(in, out, n, ar, s);
@@ -496,6 +564,11 @@ void stable_partition(const int32_t *keys, int64_t n, int32_t nkeys, int32_t *pe
   BST_REQUIRE(nkeys >= 1, BST_ERR_INVALID_ARG, "stable_partition: nkeys < 1");
   if (n == 0) {
     BST_CUDA(cudaMemsetAsync(key_ptr, 0, sizeof(int32_t) * ((size_t)nkeys + 1), s));
+    return;
+  }
+  if (n <= kOnePartItems && nkeys <= kOnePartKeys) {
+    k_part_one<<<1, 1024, 0, s>>>(keys, (int)n, nkeys, perm, key_ptr);
+    BST_CHECK_LAUNCH();
     return;
   }
   // segment length: at least 256 items per warp, and at most 2^24 histogram cells

@@ -354,14 +354,13 @@ __global__ void k_sym_fill(SymArgs S, FillOut O) {
   });
 }
 
-__global__ void k_i64_to_i32_one(const int64_t *__restrict__ in, int32_t *__restrict__ out) {
-  *out = (int32_t)*in;
-}
-
+// C's row pointer in 32 bits, and the product count at the end of t_start
 __global__ void k_rowptr_i64_to_i32(const int64_t *__restrict__ in, int32_t *__restrict__ out,
-                                    int64_t n) {
+                                    int64_t n, const int64_t *__restrict__ total,
+                                    int32_t *__restrict__ t_end) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i <= n) out[i] = (int32_t)in[i];
+  if (i == 0) *t_end = (int32_t)*total;
 }
 
 __global__ void k_c_sizes(int64_t nc, const int32_t *__restrict__ c_row,
@@ -396,8 +395,13 @@ struct EmitArgs {
   int32_t *refA, *refB;
 };
 
+// The stacks, and the run of every (C block, k class): a bucket lists its products by C block,
+// so a run is consecutive entries.  Its first entry sets the start and its last the length
+// (atomics per entry, on the start and on the length, took twice as long).
 __global__ void k_emit_stacks(EmitArgs E) {
   int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const unsigned act = __ballot_sync(0xffffffffu, q < E.T);
   if (q >= E.T) return;
   const int p = E.perm[q];
   const int a = E.t_a[p], b = E.t_b[p], c = E.t_c[p], k = E.t_k[p];
@@ -408,21 +412,44 @@ __global__ void k_emit_stacks(EmitArgs E) {
   E.s_k[q] = k;
   E.s_ab[q] = a;
   E.s_bb[q] = b;
-  const int64_t r = (int64_t)c * E.Dk + E.k_cls[k];
-  atomicMin(&E.run_start[r], (int32_t)q);
-  atomicAdd(&E.run_len[r], 1);
+  // runs are numbered below 2^31
+  auto run_of = [&](int64_t x) -> int {
+    const int px = E.perm[x];
+    return E.t_c[px] * E.Dk + E.k_cls[E.t_k[px]];
+  };
+  const int r = c * E.Dk + E.k_cls[k];
+  int before = __shfl_up_sync(act, r, 1), after = __shfl_down_sync(act, r, 1);
+  if (lane == 0) before = q > 0 ? run_of(q - 1) : -1;
+  if (q + 1 == E.T)
+    after = -1;
+  else if (lane == 31)
+    after = run_of(q + 1);
+  const bool first = before != r, last = after != r;
+  if (first) E.run_start[r] = (int32_t)q;
+  if (first && last)
+    E.run_len[r] = 1;
+  else if (first)
+    atomicAdd(&E.run_len[r], -(int32_t)q);
+  else if (last)
+    atomicAdd(&E.run_len[r], (int32_t)q + 1);
   E.refA[a] = 1;
   E.refB[b] = 1;
 }
 
-// referenced elements: sum over flagged blocks of their areas
-__global__ void k_ref_elems(int64_t nblocks, const int32_t *__restrict__ flag,
-                            const int32_t *__restrict__ row, const int32_t *__restrict__ col,
-                            const int32_t *__restrict__ rsz, const int32_t *__restrict__ csz,
-                            unsigned long long *__restrict__ out) {
+// referenced elements of both operands: sum over flagged blocks of their areas
+struct RefArgs {
+  int64_t nblocks[2];
+  const int32_t *flag[2], *row[2], *col[2], *rsz[2], *csz[2];
+  unsigned long long *out;
+};
+
+__global__ void k_ref_elems(RefArgs A) {
+  const int y = blockIdx.y;
+  const int32_t *row = A.row[y], *col = A.col[y], *rsz = A.rsz[y], *csz = A.csz[y];
+  unsigned long long *out = A.out + y;
   int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long v = 0;
-  if (b < nblocks && flag[b]) v = (unsigned long long)rsz[row[b]] * csz[col[b]];
+  if (b < A.nblocks[y] && A.flag[y][b]) v = (unsigned long long)rsz[row[b]] * csz[col[b]];
   for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(out, v);
 }
@@ -585,9 +612,7 @@ void symbolic_phase(bst_plan *p, cudaStream_t s, bool schedule) {
   int64_t *c_rowptr64 = scratch.alloc_n<int64_t>((size_t)M + 1);
   int64_t *t_rowptr = scratch.alloc_n<int64_t>((size_t)M + 1);
   int64_t *cand_ptr = scratch.alloc_n<int64_t>((size_t)M + 1);
-  exscan_i32_i64(c_rownnz, c_rowptr64, M, scratch, s);
-  exscan_i32_i64(t_rowcnt, t_rowptr, M, scratch, s);
-  exscan_i32_i64(cand_rowcnt, cand_ptr, M, scratch, s);
+  exscan3_i32_i64({c_rownnz, t_rowcnt, cand_rowcnt}, {c_rowptr64, t_rowptr, cand_ptr}, M, scratch, s);
   int64_t tot[3];
   {
     ReadBack rb(p->ctx, s);
@@ -614,11 +639,13 @@ void symbolic_phase(bst_plan *p, cudaStream_t s, bool schedule) {
   C->row = ar.alloc_n<int32_t>((size_t)nnzC);
   C->col = ar.alloc_n<int32_t>((size_t)nnzC);
   C->off = ar.alloc_n<int64_t>((size_t)nnzC + 1);
-  k_rowptr_i64_to_i32<<<nblk(M + 1, 256), 256, 0, s>>>(c_rowptr64, C->rowptr, M);
-  BST_CHECK_LAUNCH();
   p->c_cin = ar.alloc_n<int32_t>((size_t)nnzC);
   p->c_cls = ar.alloc_n<int32_t>((size_t)nnzC);
   p->t_start = ar.alloc_n<int32_t>((size_t)nnzC + 1);
+  // t_start[nnzC] = T, from the device's own count (no host round trip)
+  k_rowptr_i64_to_i32<<<nblk(M + 1, 256), 256, 0, s>>>(c_rowptr64, C->rowptr, M, t_rowptr + M,
+                                                       p->t_start + nnzC);
+  BST_CHECK_LAUNCH();
   int32_t *cnt = scratch.alloc_n<int32_t>((size_t)nnzC);
   int32_t *t_a = scratch.alloc_n<int32_t>((size_t)T);
   int32_t *t_b = scratch.alloc_n<int32_t>((size_t)T);
@@ -640,9 +667,6 @@ void symbolic_phase(bst_plan *p, cudaStream_t s, bool schedule) {
     k_sym_fill<<<nblk(M, wpc), 32 * wpc, smem_fill, s>>>(S, O);
     BST_CHECK_LAUNCH();
   }
-  // t_start[nnzC] = T, from the device's own count (no host round trip)
-  k_i64_to_i32_one<<<1, 1, 0, s>>>(t_rowptr + M, p->t_start + nnzC);
-  BST_CHECK_LAUNCH();
 
   // element offsets and (m,n) class of every C block
   int64_t *csize = scratch.alloc_n<int64_t>((size_t)nnzC);
@@ -685,12 +709,12 @@ void symbolic_phase(bst_plan *p, cudaStream_t s, bool schedule) {
   BST_REQUIRE(nruns < INT32_MAX, BST_ERR_UNSUPPORTED, "run table too large");
   p->run_start = ar.alloc_n<int32_t>((size_t)nruns);
   p->run_len = ar.alloc_n<int32_t>((size_t)nruns);
-  fill_i32(p->run_start, INT32_MAX, nruns, s);
   BST_CUDA(cudaMemsetAsync(p->run_len, 0, sizeof(int32_t) * (size_t)std::max<int64_t>(nruns, 1), s));
-  int32_t *refA = scratch.alloc_n<int32_t>((size_t)A->nblocks);
-  int32_t *refB = scratch.alloc_n<int32_t>((size_t)B->nblocks);
-  BST_CUDA(cudaMemsetAsync(refA, 0, sizeof(int32_t) * (size_t)std::max<int64_t>(A->nblocks, 1), s));
-  BST_CUDA(cudaMemsetAsync(refB, 0, sizeof(int32_t) * (size_t)std::max<int64_t>(B->nblocks, 1), s));
+  // flags of the referenced blocks of A and B and their element counts, cleared together
+  const size_t na = (size_t)A->nblocks, nb = (size_t)B->nblocks;
+  unsigned long long *refel = static_cast<unsigned long long *>(scratch.alloc(16 + 4 * (na + nb)));
+  int32_t *refA = reinterpret_cast<int32_t *>(refel + 2), *refB = refA + na;
+  BST_CUDA(cudaMemsetAsync(refel, 0, 16 + 4 * (na + nb), s));
   if (T > 0) {
     EmitArgs E;
     E.T = T;
@@ -719,16 +743,19 @@ void symbolic_phase(bst_plan *p, cudaStream_t s, bool schedule) {
     BST_CHECK_LAUNCH();
   }
   p->items_counter = ar.alloc_n<unsigned long long>(1);
-  unsigned long long *refel = scratch.alloc_n<unsigned long long>(2);
-  BST_CUDA(cudaMemsetAsync(refel, 0, 16, s));
-  if (A->nblocks > 0) {
-    k_ref_elems<<<nblk(A->nblocks, 256), 256, 0, s>>>(A->nblocks, refA, A->row, A->col, A->rsz,
-                                                      A->csz, refel);
-    BST_CHECK_LAUNCH();
-  }
-  if (B->nblocks > 0) {
-    k_ref_elems<<<nblk(B->nblocks, 256), 256, 0, s>>>(B->nblocks, refB, B->row, B->col, B->rsz,
-                                                      B->csz, refel + 1);
+  if (na + nb > 0) {
+    RefArgs ra;
+    for (int y = 0; y < 2; ++y) {
+      const bst_matrix *X = y ? B : A;
+      ra.nblocks[y] = X->nblocks;
+      ra.flag[y] = y ? refB : refA;
+      ra.row[y] = X->row;
+      ra.col[y] = X->col;
+      ra.rsz[y] = X->rsz;
+      ra.csz[y] = X->csz;
+    }
+    ra.out = refel;
+    k_ref_elems<<<dim3(nblk((int64_t)std::max(na, nb), 256), 2), 256, 0, s>>>(ra);
     BST_CHECK_LAUNCH();
   }
   unsigned long long hrefel[2];
