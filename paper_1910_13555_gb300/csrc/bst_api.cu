@@ -24,7 +24,7 @@ void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 void set_error(const std::string &msg) { g_last_error = msg; }
 
 void *Arena::alloc(size_t bytes) {
-  if (4 * bytes > chunk) return alloc_own(bytes);
+  if (chunk == 0 || 4 * bytes > chunk) return alloc_own(bytes);
   const size_t need = (std::max<size_t>(bytes, 8) + 255) & ~(size_t)255;
   if (left < need) {
     next = static_cast<char *>(alloc_own(chunk));
