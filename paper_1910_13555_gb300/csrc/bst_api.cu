@@ -388,7 +388,7 @@ bst_status bst_plan_split_histogram(const bst_plan *plan, int64_t *hist) {
     BST_CUDA(cudaMemcpy2D(w.data(), 4, plan->fdesc + 7, 4 * bst::kF64DescWords, 4,
                           (size_t)plan->n_tiles, cudaMemcpyDeviceToHost));
     // whole-tile split, else the split of the tile's last partial round
-    for (int32_t v : w) ++hist[std::min(std::max((v & 0xff) > 1 ? v & 0xff : v >> 8, 1), 16)];
+    for (int32_t v : w) ++hist[std::min(std::max((v & 0xff) > 1 ? v & 0xff : (v >> 8) & 0xff, 1), 16)];
   } else if (plan->C) {
     hist[0] = plan->C->nblocks;
   }

@@ -21,7 +21,18 @@ constexpr int kNarrowSlot = 896, kWideSlot = 1184;
 constexpr int kStageWarps = 4;    // warps per CTA
 constexpr int kF64Desc = kF64DescWords;
 
-__device__ __forceinline__ int f64_split_word(int s, int tail) { return s | (tail << 8); }
+__device__ __forceinline__ int f64_split_word(int s, int tail, int fresh = 0) {
+  return s | (tail << 8) | (fresh << 16);
+}
+
+// Whether a tile sums every panel by itself and adds it to the output once (split instances
+// only): long sums without a whole-tile split, over panels wide enough that the extra add
+// costs at most 1/16.  One chain over 300 inner elements rounds twice as far as the partial
+// sums of the whole-tile split that the tail split replaces (relative error of the rank-3
+// contraction with gradients 2.1e-15, so 0.8e-15, for 1 % of its time).
+__device__ __forceinline__ int f64_fresh(long long w1, int ne, int split, int tail) {
+  return split == 1 && tail > 1 && w1 >= 128 && w1 >= 16ll * ne;
+}
 
 // Inner split of every tile (descriptor word 7): the s <= smax of the tile's class that
 // needs the fewest FP64 warp instructions -- ceil(s mt n / 32) for each of the

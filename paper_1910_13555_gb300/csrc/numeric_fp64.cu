@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(256, 2)
 // elements).  Descriptor: 0 element offset of the tile in C, 1 first entry, 2 entry
 // count, 3 tile rows m | n << 12, 4 C_in block (-1: none), 5 element offset of the tile
 // inside the C_in block, 6 C block, 7 inner split s (>= 1) | tail split << 8 (>= 1, taken
-// when s = 1; see slot_tail).  In a schedule of rectangular tiles (the adjoint's, TILED
+// when s = 1; see slot_tail) | panels summed by themselves << 16 (f64_fresh).  In a schedule of rectangular tiles (the adjoint's, TILED
 // below) the entries are those of the whole output block, shared by its tiles: word 4 holds
 // the tile's first row and column p0 | q0 << 16, word 5 the row length of the output block.
 struct F64Blk {
@@ -429,9 +429,10 @@ __device__ __forceinline__ double lds(unsigned a) {
 // loop unrolled by 2 or 4, and two or four outputs at a time as independent FMA chains all
 // measured the same or slower (banded 4000 x 4000: 19.0 ms rolled with one chain or two,
 // 20.7 ms unrolled by four with two).
-template <int MR>
+// FRESH and fresh: the panel is summed by itself and added once (f64_fresh).
+template <int MR, bool FRESH>
 __device__ __forceinline__ void slot_product_rt(const NumParams &P, const double *As, int m, int n,
-                                                int k, int F, const LaneMap &L,
+                                                int k, int F, const LaneMap &L, bool fresh,
                                                 double (&acc)[MR]) {
   const int lane = threadIdx.x & 31, mn = m * n;
   const unsigned A0 = (unsigned)__cvta_generic_to_shared(As), B0 = A0 + 8 * m * k;
@@ -443,13 +444,14 @@ __device__ __forceinline__ void slot_product_rt(const NumParams &P, const double
     if (r >= F) break;
     if (lane + 32 * r < mn) {
       unsigned a = A0 + p * a_sp, b = B0 + q * b_sq;
-      double s = acc[r];
+      double s = FRESH && fresh ? 0.0 : acc[r];
 #pragma unroll 1
       for (int l = 0; l < k; ++l) {
         s = fma(lds(a), lds(b), s);
         a += a_sl;
         b += b_sl;
       }
+      if (FRESH && fresh) s += acc[r];
       acc[r] = s;
     }
     lane_step(L, n, p, q);
@@ -712,7 +714,7 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
 #pragma unroll
     for (int r = 0; r < MR; ++r) acc[r] = 0.0;
     const int bs = SPLIT ? b.s & 0xff : 1;  // whole-tile split, else the tail's
-    const int ts = bs > 1 ? 1 : b.s >> 8, mn = b.m * b.n;
+    const int ts = bs > 1 ? 1 : (b.s >> 8) & 0xff, mn = b.m * b.n;
     const int F = ts > 1 ? mn >> 5 : (mn + 31) >> 5;
     const LaneMap L = lane_map(b.n);
     const TailMap T = ts > 1 ? tail_map(mn, b.n, ts) : TailMap{0, 0, 0};
@@ -744,7 +746,7 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
       if (SPLIT && bs > 1) {
         slot_product_split(P, cur, b.m, b.n, k, bs, acc);
       } else {
-        slot_product_rt(P, cur, b.m, b.n, k, F, L, acc);
+        slot_product_rt<MR, SPLIT && !TILED>(P, cur, b.m, b.n, k, F, L, b.s >> 16, acc);
         if (ts > 1) acct = slot_tail(P, cur, b.m, b.n, k, ts, T, acct);
       }
       __syncwarp();
@@ -938,7 +940,9 @@ __device__ __forceinline__ void f64_tiles_of(
     int split = 1;
     if (w1 >= kSplitMinInner && smax >= 2)
       split = f64_split_of(d, ents, cls_smax[cls], tile_max, slot_elems, c1, saved);
-    dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, f64_split_word(split, tail_of(tc)));
+    const int tail = tail_of(tc);
+    dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c,
+                      f64_split_word(split, tail, f64_fresh(w1, (int)(q - q0), split, tail)));
     c1_sum += c1;
     saved_sum += saved;
   }
@@ -983,7 +987,9 @@ __global__ void k_f64_split(int64_t ntiles, const int4 *__restrict__ ents,
     TailCost tc = tail_cost(mn, smax);
     for (int e = 0; e < d[2]; ++e) tail_add(tc, ents[(int64_t)d[1] + e].z);
     c1 = tail_total(tc, mn);
-    d[7] = f64_split_word(f64_split_of(d, ents, smax, tile_max, slot_elems, c1, saved), tail_of(tc));
+    const int split = f64_split_of(d, ents, smax, tile_max, slot_elems, c1, saved);
+    const int tail = tail_of(tc);
+    d[7] = f64_split_word(split, tail, f64_fresh(tc.w1, d[2], split, tail));
   }
   for (int o = 16; o > 0; o >>= 1) {
     c1 += __shfl_down_sync(0xffffffffu, c1, o);
