@@ -96,21 +96,26 @@ __device__ __forceinline__ int exp_of(double x) {
   return ex == 0 ? kExpNone : ex - 1022;
 }
 
-struct SideArgs {
+// one operand's stored blocks as its op sees them
+struct SideView {
   int64_t nblocks;
   const int32_t *row, *col, *rsz, *csz;  // stored block index and sizes
   const int64_t *off;                    // element offset of stored block
   const double *data;
-  int trans;       // op(X) = X^T
-  int is_b;        // 0: exponents per op row (A side), 1: per op column (B side)
+  int trans;            // op(X) = X^T
+  int is_b;             // 0: outer index = op row (A side), 1: op column (B side)
+  const int64_t *doff;  // per block digit / tf32 offset
+  float *tf;            // 3xTF32 parts
+};
+
+// what the digit kernels need on top
+struct SideArgs : SideView {
   const int64_t *eoff;   // per block exponent offset
-  const int64_t *doff;   // per block digit / tf32 offset
   int32_t *bexp;         // per block exponents
   const int64_t *start;  // global start of each op row block (A) / op column block (B)
   int32_t *gexp;         // largest exponent of each whole op row (A) / op column (B)
   int row_scale;         // digits scaled by the whole op row / column (1) or the block's (0)
   __nv_bfloat16 *dig;
-  float *tf;
 };
 
 // The side kernels run one warp per stored block; in the digit kernels four lanes share one
@@ -123,10 +128,9 @@ struct SideBlock {
   const double *x;
   int Cc, nouter, ninner, nch;
   bool outer_major;
-  int64_t gbase;
 };
 
-__device__ __forceinline__ SideBlock side_block(const SideArgs &S, int64_t b) {
+__device__ __forceinline__ SideBlock side_block(const SideView &S, int64_t b) {
   SideBlock B;
   const int R = S.rsz[S.row[b]], Cc = S.csz[S.col[b]];
   B.x = S.data + S.off[b];
@@ -135,10 +139,13 @@ __device__ __forceinline__ SideBlock side_block(const SideArgs &S, int64_t b) {
   B.ninner = S.is_b ? (S.trans ? Cc : R) : (S.trans ? R : Cc);
   B.nch = (B.ninner + 15) >> 4;
   B.outer_major = S.is_b == S.trans;
-  // op block index along the exponent dimension (rows of op(A), columns of op(B))
-  const int obr = S.trans ? S.col[b] : S.row[b], obc = S.trans ? S.row[b] : S.col[b];
-  B.gbase = S.start[S.is_b ? obc : obr];
   return B;
+}
+
+// first place of block b among the exponents of whole op rows (columns): the op block index
+// along that dimension is op(A)'s block row, op(B)'s block column
+__device__ __forceinline__ int64_t side_gbase(const SideArgs &S, int64_t b) {
+  return S.start[(S.is_b != 0) == (S.trans != 0) ? S.row[b] : S.col[b]];
 }
 
 __device__ __forceinline__ double side_value(const SideBlock &B, int outer, int inner) {
@@ -157,6 +164,7 @@ __global__ void k_emu_exponents(SideArgs S) {
   const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (b >= S.nblocks) return;
   const SideBlock B = side_block(S, b);
+  const int64_t gbase = side_gbase(S, b);
   const int total = B.nouter * B.nch;
   for (int q0 = 0; q0 < total; q0 += 8) {  // uniform trip count: every lane shuffles
     const int q = q0 + (lane >> 2);
@@ -170,7 +178,7 @@ __global__ void k_emu_exponents(SideArgs S) {
     E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
     if (ok && t == 0 && E != kExpNone) {
       atomicMax(&S.bexp[S.eoff[b] + outer], E);
-      atomicMax(&S.gexp[B.gbase + outer], E);
+      atomicMax(&S.gexp[gbase + outer], E);
     }
   }
 }
@@ -184,11 +192,12 @@ __global__ void k_emu_digits(SideArgs S) {
   const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (b >= S.nblocks) return;
   const SideBlock B = side_block(S, b);
+  const int64_t gbase = side_gbase(S, b);
   __nv_bfloat16 *d = S.dig + S.doff[b];
   const int total = B.nouter * B.nch;
   for (int q = lane >> 2; q < total; q += 8) {
     const int outer = q / B.nch, ch = q - outer * B.nch;
-    const int E = S.row_scale ? S.gexp[B.gbase + outer] : S.bexp[S.eoff[b] + outer];
+    const int E = S.row_scale ? S.gexp[gbase + outer] : S.bexp[S.eoff[b] + outer];
     uint32_t w[kSlices][2];
 #pragma unroll
     for (int s = 0; s < kSlices; ++s) w[s][0] = w[s][1] = 0u;
@@ -232,7 +241,7 @@ __device__ __forceinline__ float to_tf32(float x) {
 // order the m16n8k8 fragments take them: lane t of four holds inner t and t + 4, so its 16
 // bytes are {high t, high t + 4, low t, low t + 4} and a fragment is one 16-byte load.  The
 // padding of the last chunk is written as zeros with it (no clearing pass).
-__global__ void k_tf32_split(SideArgs S) {
+__global__ void k_tf32_split(SideView S) {
   const int lane = threadIdx.x & 31, t = lane & 3;
   const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (b >= S.nblocks) return;
@@ -1482,7 +1491,7 @@ void execute_tf32x3(bst_plan *p, const NumArgs &a, cudaStream_t s) {
   for (int side = 0; side < 2; ++side) {
     const bst_matrix *X = side ? p->B : p->A;
     if (X->nblocks == 0) continue;
-    SideArgs S = side_args(X, side ? p->tb : p->ta, side == 1);
+    SideView S = side_args(X, side ? p->tb : p->ta, side == 1);
     S.data = side ? a.B : a.A;
     S.doff = side ? E.b_toff : E.a_toff;
     S.tf = side ? E.b_tf : E.a_tf;
