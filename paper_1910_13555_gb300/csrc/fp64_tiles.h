@@ -21,69 +21,30 @@ constexpr int kNarrowSlot = 896, kWideSlot = 1184;
 constexpr int kStageWarps = 4;    // warps per CTA
 constexpr int kF64Desc = kF64DescWords;
 
-__device__ __forceinline__ int f64_split_word(int s, int tail, int fresh = 0) {
-  return s | (tail << 8) | (fresh << 16);
+// descriptor word 7: whole-tile split, tail split, and whether every panel is summed by itself
+// and then added (full rounds, tail)
+__host__ __device__ __forceinline__ int f64_split_word(int s, int tail, int fresh = 0,
+                                                       int tail_fresh = 0) {
+  return s | (tail << 8) | (fresh << 16) | (tail_fresh << 17);
 }
 
-// Whether a tile sums every panel by itself and adds it to the output once (split instances
-// only): long sums without a whole-tile split, over panels wide enough that the extra add
-// costs at most 1/16.  One chain over 300 inner elements rounds twice as far as the partial
-// sums of the whole-tile split that the tail split replaces (relative error of the rank-3
-// contraction with gradients 2.1e-15, so 0.8e-15, for 1 % of its time).
-__device__ __forceinline__ int f64_fresh(long long w1, int ne, int split, int tail) {
-  return split == 1 && tail > 1 && w1 >= 128 && w1 >= 16ll * ne;
-}
-
-// Inner split of every tile (descriptor word 7): the s <= smax of the tile's class that
-// needs the fewest FP64 warp instructions -- ceil(s mt n / 32) for each of the
-// ceil(w / s) steps of a panel of width w, plus (s - 1) ceil(mt n / 32) adds for the
-// final sums -- when it saves anything on a tile with at least kSplitLongInner inner
-// elements in all, at least 1/8 of the unsplit count on one with kSplitMinInner or more,
-// else 1 (on short tiles the final sums cost more than the idle lanes).  The plan-wide
-// sums of the unsplit counts and of the savings decide whether the plan splits at all
-// (refresh_f64_split).
+// Inner split of a tile (descriptor word 7): the s <= smax of the tile's class that needs the
+// fewest FP64 warp instructions -- ceil(s mt n / 32) for each of the ceil(w / s) steps of a
+// panel of width w, plus (s - 1) ceil(mt n / 32) adds for the final sums -- when it saves
+// anything on a tile with at least kSplitLongInner inner elements in all, at least 1/8 of the
+// other count on one with kSplitMinInner or more, else 1 (on short tiles the final sums cost
+// more than the idle lanes).  choose_tile weighs it against the tail split.
 constexpr int kMaxSplit = 16;
 constexpr int kSplitMinInner = 48;
 constexpr int kSplitLongInner = 128;
 
 // FP64 instructions of a tile split s ways whose steps number W, and whether the best of
 // them (cb) is worth it against c1 unsplit ones on w1 inner elements
-__device__ __forceinline__ long long split_cost(int s, int mn, long long W) {
+__host__ __device__ __forceinline__ long long split_cost(int s, int mn, long long W) {
   return (long long)((s * mn + 31) / 32) * W + (s - 1) * ((mn + 31) / 32);
 }
-__device__ __forceinline__ bool split_pays(long long cb, long long c1, long long w1) {
+__host__ __device__ __forceinline__ bool split_pays(long long cb, long long c1, long long w1) {
   return w1 >= kSplitMinInner && (w1 >= kSplitLongInner ? cb < c1 : 8 * cb <= 7 * c1);
-}
-
-__device__ inline int f64_split_of(int32_t *__restrict__ d, const int4 *__restrict__ ents,
-                                   int smax, int tile, int slot_elems, long long c1,
-                                   long long &saved) {
-  const int mn = (d[3] & 0xfff) * ((d[3] >> 12) & 0xfff), ne = d[2];
-  // s m n partial sums fit the accumulators and, for the final sums, one slot
-  smax = min(min(smax, kMaxSplit), min(tile, slot_elems) / max(mn, 1));
-  int best = 1;
-  saved = 0;
-  // short tiles (most of a plan of small products) never split: one pass over the widths
-  long long w1 = 0;
-  for (int e = 0; e < ne; ++e) w1 += ents[(int64_t)d[1] + e].z;
-  if (w1 < kSplitMinInner || smax < 2) return 1;
-  long long W[kMaxSplit + 1];
-  for (int s = 1; s <= max(smax, 1); ++s) W[s] = 0;
-  for (int e = 0; e < ne; ++e) {
-    const int w = ents[(int64_t)d[1] + e].z;
-    for (int s = 1; s <= max(smax, 1); ++s) W[s] += (w + s - 1) / s;
-  }
-  long long cb = c1;
-  for (int s = 2; s <= smax; ++s) {
-    const long long c = split_cost(s, mn, W[s]);
-    if (c < cb) {
-      cb = c;
-      best = s;
-    }
-  }
-  if (!split_pays(cb, c1, W[1])) best = 1;
-  if (best > 1) saved = c1 - cb;
-  return best;
 }
 
 // Tail split of a tile (descriptor word 7, bits 8 and up): the t <= 32 / rem lane groups
@@ -98,34 +59,179 @@ struct TailCost {
   long long c[2], w1;
 };
 
-__device__ __forceinline__ TailCost tail_cost(int mn, int smax) {
+__host__ __device__ __forceinline__ TailCost tail_cost(int mn, int smax) {
   TailCost C;
   const int rem = mn & 31;
-  C.t[0] = rem ? min(32 / rem, min(smax, kMaxSplit)) : 1;
+  C.t[0] = 1;
+  if (rem) {
+    const int most = smax < kMaxSplit ? smax : kMaxSplit;
+    C.t[0] = 32 / rem < most ? 32 / rem : most;
+  }
   C.t[1] = (C.t[0] + 1) >> 1;
   C.w1 = 0;
   for (int i = 0; i < 2; ++i) {
-    C.c[i] = 32 - __clz(C.t[i] - 1);  // ceil(log2 t)
+    C.c[i] = (C.t[i] > 1) + (C.t[i] > 2) + (C.t[i] > 4) + (C.t[i] > 8);  // ceil(log2 t)
     C.inv[i] = (65535 + C.t[i]) / C.t[i];
   }
   return C;
 }
 
-__device__ __forceinline__ void tail_add(TailCost &C, int w) {
+__host__ __device__ __forceinline__ void tail_add(TailCost &C, int w) {
   C.w1 += w;
   // panels are at most a slot wide, w <= kWideSlot
   C.c[0] += ((unsigned)(w + C.t[0] - 1) * C.inv[0]) >> 16;
   C.c[1] += ((unsigned)(w + C.t[1] - 1) * C.inv[1]) >> 16;
 }
 
-// FP64 instructions of the unsplit tile
-__device__ __forceinline__ long long tail_total(const TailCost &C, int mn) {
-  return (mn >> 5) * C.w1 + ((mn & 31) ? min(C.w1, min(C.c[0], C.c[1])) : 0);
+// FP64 instructions of the tile without a whole-tile split
+__host__ __device__ __forceinline__ long long tail_total(const TailCost &C, int mn) {
+  const long long t = C.c[0] < C.c[1] ? C.c[0] : C.c[1];
+  return (mn >> 5) * C.w1 + ((mn & 31) ? (t < C.w1 ? t : C.w1) : 0);
 }
 
-__device__ __forceinline__ int tail_of(const TailCost &C) {
+__host__ __device__ __forceinline__ int tail_of(const TailCost &C) {
   const int i = C.c[1] < C.c[0] ? 1 : 0;
   return C.t[i] > 1 && C.c[i] < C.w1 ? C.t[i] : 1;
+}
+
+// What a whole-tile split's cost is formed from: steps[s] = sum of ceil(w / s) over the panels
+// (32 bits hold a tile's: its inner elements are elements of A, which 31 bits index)
+template <class T>
+struct SplitSteps {
+  T steps[kMaxSplit + 1] = {};
+  int wmax = 0;
+  __host__ __device__ __forceinline__ void add(int w, T times = 1) {
+#pragma unroll
+    for (int s = 2; s <= kMaxSplit; ++s) steps[s] += times * (T)((unsigned)(w + s - 1) / s);
+    wmax = w > wmax ? w : wmax;
+  }
+};
+
+// an add of a fresh panel waits for the panel's chain, with no other FMA of the warp behind it:
+// 4.7 % of the time of 10 x 10 and 5 x 13 blocks over panels of 35, 12 % over panels of 13,
+// where the added instructions are 2.7 % and 7.3 %
+constexpr int kFreshAdd = 2;
+
+struct TileChoice {
+  int split = 1, tail = 1, fresh = 0, tail_fresh = 0;
+  long long plain = 0;      // instructions with the tail split alone
+  long long cost = 0;       // of what was chosen
+  long long saved = 0;      // plain minus cost where a whole-tile split was chosen
+  long long unsplit = 0;    // without any split
+  long long reference = 0;  // what the reference split saves of that
+};
+
+// the largest whole-tile split whose partial sums fit `elems` accumulators and a slot
+__host__ __device__ __forceinline__ int split_bound(int smax, int mn, int elems, int slot) {
+  const int room = (elems < slot ? elems : slot) / (mn > 1 ? mn : 1);
+  const int most = smax < kMaxSplit ? smax : kMaxSplit;
+  return room < most ? room : most;
+}
+
+// Whether choose_tile may split a tile and reads `steps`.  A split saves at most the idle lanes,
+// so short tiles (which split for 1/8 of the instructions) need 1/8 of them idle: the 1.3 M tiles
+// of the 4000 x 4000 banded plan are mostly short, and going through their splits took 0.25 ms.
+__host__ __device__ __forceinline__ bool tile_may_split(long long w1, int smax, int mn, int slot) {
+  const int lanes = (mn + 31) & ~31, idle = lanes - mn;
+  return w1 >= kSplitMinInner && idle > 0 && (w1 >= kSplitLongInner || 8 * idle >= lanes) &&
+         split_bound(smax, mn, 32 * kWideR, slot) >= 2;
+}
+
+// How a tile of mn outputs, ne panels and C.w1 inner elements in all sums them (tile: elements
+// of the largest tile of the plan's shape; slot: doubles of its slots).
+//
+// An output of one chain over w1 elements rounds as sqrt(w1); the s partial sums of a whole-tile
+// split as sqrt(w1 / s + s), panels summed by themselves ("fresh") as sqrt(wmax + ne), at one add
+// per output and panel.  The tail split is often cheaper than a whole-tile split but leaves the
+// full rounds one chain: the relative error of 13 x 13 blocks with 60 products of 35 was 1.2e-15
+// that way, 4.4e-16 with the sums split in three.  So where a whole-tile split would pay (at
+// least 1/25 of the unsplit instructions, by the accumulators of the wide shape), it is the
+// reference: the tile takes the cheapest form whose chains are no longer than that split's.
+// Elsewhere one chain stays, except that long sums over wide panels beside a tail split are
+// fresh too (an add per 16 elements at most; the rank-3 contraction with gradients 2.1e-15, so
+// 0.8e-15, for 1 % of its time).
+template <class T>
+__host__ __device__ inline TileChoice choose_tile(const TailCost &C, const SplitSteps<T> &S, int mn,
+                                                  long long ne, int smax, int tile, int slot) {
+  TileChoice R;
+  const long long w1 = C.w1;
+  const unsigned inner = w1 < (1ll << 31) ? (unsigned)w1 : 1u << 31;  // for the chains' lengths
+  const int rounds = (mn + 31) >> 5;
+  R.tail = tail_of(C);
+  R.plain = R.cost = tail_total(C, mn);
+  R.unsplit = rounds * w1;
+  if (w1 < kSplitMinInner) return R;
+  const int full = R.tail > 1 ? mn >> 5 : rounds;
+  if (!tile_may_split(w1, smax, mn, slot)) {
+    R.fresh = R.tail > 1 && full > 0 && w1 >= kSplitLongInner && w1 >= 16 * ne;
+    R.cost += R.fresh ? kFreshAdd * full * ne : 0;
+    return R;
+  }
+  int s0 = 1;
+  long long c0 = R.unsplit;
+  const int most = split_bound(smax, mn, 32 * kWideR, slot), now = split_bound(smax, mn, tile, slot);
+#pragma unroll
+  for (int s = 2; s <= kMaxSplit; ++s) {
+    const long long c = split_cost(s, mn, S.steps[s]);
+    if (s <= most && c < c0) {
+      c0 = c;
+      s0 = s;
+    }
+  }
+  if (!split_pays(c0, R.unsplit, w1) || 25 * (R.unsplit - c0) < R.unsplit) s0 = 1;
+  R.reference = s0 > 1 ? R.unsplit - c0 : 0;
+  const long long limit = s0 > 1 ? inner / (unsigned)s0 + s0 : w1 + ne;
+  long long chain = 0;  // the longest without a whole-tile split
+  if (full > 0) {
+    R.fresh = s0 > 1 || (R.tail > 1 && w1 >= kSplitLongInner && w1 >= 16 * ne);
+    R.cost += R.fresh ? kFreshAdd * full * ne : 0;
+    chain = R.fresh ? S.wmax + ne : w1;
+  }
+  if (R.tail > 1) {
+    const long long one = inner / (unsigned)R.tail + R.tail;
+    R.tail_fresh = one > limit;
+    R.cost += R.tail_fresh ? kFreshAdd * ne : 0;
+    const long long t = R.tail_fresh ? (S.wmax + R.tail - 1) / R.tail + ne : one;
+    chain = chain > t ? chain : t;
+  }
+  int best = 1, shortest = 1;
+  long long cb = 0, least = chain;
+#pragma unroll
+  for (int s = 2; s <= kMaxSplit; ++s) {
+    const long long c = split_cost(s, mn, S.steps[s]), ch = inner / (unsigned)s + s;
+    if (s > now) continue;
+    if (ch < least) {
+      shortest = s;
+      least = ch;
+    }
+    if (ch <= limit && (best == 1 || c < cb)) {
+      best = s;
+      cb = c;
+    }
+  }
+  if (chain > limit) {
+    if (best == 1) best = shortest;
+  } else if (best > 1 && !split_pays(cb, R.cost, w1)) {
+    best = 1;
+  }
+  if (best > 1) {
+    R.split = best;
+    R.cost = 0;
+#pragma unroll
+    for (int s = 2; s <= kMaxSplit; ++s)
+      if (s == best) R.cost = split_cost(s, mn, S.steps[s]);
+    R.saved = R.plain > R.cost ? R.plain - R.cost : 0;
+  }
+  return R;
+}
+
+// Plan-wide sums that decide whether a plan's tiles split at all (apply_split_gate)
+struct SplitSums {
+  unsigned long long plain, saved, unsplit, reference, marked;
+};
+
+__host__ __device__ __forceinline__ int choice_word(const TileChoice &R) {
+  return f64_split_word(R.split, R.tail, R.fresh, R.tail_fresh);
 }
 
 }  // namespace

@@ -297,7 +297,8 @@ __global__ void __launch_bounds__(256, 2)
 // elements).  Descriptor: 0 element offset of the tile in C, 1 first entry, 2 entry
 // count, 3 tile rows m | n << 12, 4 C_in block (-1: none), 5 element offset of the tile
 // inside the C_in block, 6 C block, 7 inner split s (>= 1) | tail split << 8 (>= 1, taken
-// when s = 1; see slot_tail) | panels summed by themselves << 16 (f64_fresh).  In a schedule of rectangular tiles (the adjoint's, TILED
+// when s = 1; see slot_tail) | panels summed by themselves << 16 (full rounds) and << 17 (tail),
+// both for s = 1 (choose_tile).  In a schedule of rectangular tiles (the adjoint's, TILED
 // below) the entries are those of the whole output block, shared by its tiles: word 4 holds
 // the tile's first row and column p0 | q0 << 16, word 5 the row length of the output block.
 struct F64Blk {
@@ -429,7 +430,7 @@ __device__ __forceinline__ double lds(unsigned a) {
 // loop unrolled by 2 or 4, and two or four outputs at a time as independent FMA chains all
 // measured the same or slower (banded 4000 x 4000: 19.0 ms rolled with one chain or two,
 // 20.7 ms unrolled by four with two).
-// FRESH and fresh: the panel is summed by itself and added once (f64_fresh).
+// FRESH and fresh: the panel is summed by itself and added once (choose_tile).
 template <int MR, bool FRESH>
 __device__ __forceinline__ void slot_product_rt(const NumParams &P, const double *As, int m, int n,
                                                 int k, int F, const LaneMap &L, bool fresh,
@@ -746,8 +747,12 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
       if (SPLIT && bs > 1) {
         slot_product_split(P, cur, b.m, b.n, k, bs, acc);
       } else {
-        slot_product_rt<MR, SPLIT && !TILED>(P, cur, b.m, b.n, k, F, L, b.s >> 16, acc);
-        if (ts > 1) acct = slot_tail(P, cur, b.m, b.n, k, ts, T, acct);
+        slot_product_rt<MR, SPLIT && !TILED>(P, cur, b.m, b.n, k, F, L, b.s & (1 << 16), acc);
+        if (ts > 1) {
+          const bool alone = SPLIT && !TILED && (b.s & (1 << 17));
+          const double sum = slot_tail(P, cur, b.m, b.n, k, ts, T, alone ? 0.0 : acct);
+          acct = alone ? acct + sum : sum;
+        }
       }
       __syncwarp();
       slot ^= 1;
@@ -858,11 +863,47 @@ __global__ void k_f64_ent_count(int64_t nc, const int32_t *__restrict__ c_cls,
   for (int t = 0; t < nt; ++t) cnt[tbeg[c] + t] = s;
 }
 
-constexpr unsigned long long kSplitGate = 100;
+// a plan's counters, summed over a CTA's tiles (an atomic per warp and counter took 0.25 ms of
+// the 4000 x 4000 banded plan)
+__device__ __forceinline__ void add_sums(const SplitSums &v, SplitSums *__restrict__ sums) {
+  constexpr int kN = 5;
+  static_assert(sizeof(SplitSums) == kN * sizeof(unsigned long long), "kN counters");
+  __shared__ unsigned long long part[32][kN];
+  const unsigned long long *x = &v.plain;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int i = 0; i < kN; ++i) {
+    unsigned long long t = x[i];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) part[wid][i] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x < kN) {
+    unsigned long long t = 0;
+    for (int w = 0; w < nw; ++w) t += part[w][threadIdx.x];
+    if (t) atomicAdd(&sums->plain + threadIdx.x, t);
+  }
+}
+
+// word 7 of a tile whose entries are in place, its counts added to v
+__device__ __forceinline__ int split_word_of(const int4 *__restrict__ ents, int ne, int mn,
+                                             const TailCost &tc, int smax, int tile, int slot,
+                                             SplitSums &v) {
+  SplitSteps<unsigned> st;
+  if (tile_may_split(tc.w1, smax, mn, slot))
+    for (int e = 0; e < ne; ++e) st.add(ents[e].z);
+  const TileChoice R = choose_tile(tc, st, mn, ne, smax, tile, slot);
+  v.plain += R.plain;
+  v.saved += R.saved;
+  v.unsplit += R.unsplit;
+  v.reference += R.reference;
+  v.marked += R.split > 1 || R.fresh || R.tail_fresh;
+  return choice_word(R);
+}
 
 // descriptors and entries of every tile of C block c, each tile's cost key
 // (63 - floor(log2(flops)): a stable partition on it lists costly tiles first) and its
-// inner split, with its FP64 instruction counts added to c1_sum / saved_sum
+// inner split, with its FP64 instruction counts added to sums
 __device__ __forceinline__ void f64_tiles_of(
     int64_t c, const int32_t *__restrict__ c_cls, const int32_t *__restrict__ run_start,
     const int32_t *__restrict__ run_len, const int32_t *__restrict__ s_a,
@@ -870,8 +911,7 @@ __device__ __forceinline__ void f64_tiles_of(
     const int32_t *__restrict__ c_cin, const int64_t *__restrict__ tbeg,
     const int64_t *__restrict__ ebeg, const SchedTabs &S, int32_t *__restrict__ desc,
     int4 *__restrict__ ents, int32_t *__restrict__ key, const int32_t *__restrict__ cls_smax,
-    const int32_t *__restrict__ t_start, int tile_max, int slot_elems, long long &c1_sum,
-    long long &saved_sum) {
+    const int32_t *__restrict__ t_start, int tile_max, int slot_elems, SplitSums &sums) {
   const int cls = c_cls[c];
   const int m = S.cls_m[cls], n = S.cls_n[cls], tr = S.tile_rows[cls];
   const int nt = (m + tr - 1) / tr;
@@ -930,26 +970,15 @@ __device__ __forceinline__ void f64_tiles_of(
     dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)q0, (int32_t)(q - q0),
                       mt | (n << 12));
     key[tile] = __clzll(flops + 1ull);
-    const long long w1 = tc.w1;  // the tile's inner elements
-    // a short tile never splits (the test f64_split_of starts with), decided here
-    // without reading its entries back
-    const int mn = mt * n;
-    const int smax = min(min(cls_smax[cls], kMaxSplit), min(tile_max, slot_elems) / max(mn, 1));
-    const long long c1 = tail_total(tc, mn);
-    long long saved = 0;
-    int split = 1;
-    if (w1 >= kSplitMinInner && smax >= 2)
-      split = f64_split_of(d, ents, cls_smax[cls], tile_max, slot_elems, c1, saved);
-    const int tail = tail_of(tc);
-    dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c,
-                      f64_split_word(split, tail, f64_fresh(w1, (int)(q - q0), split, tail)));
-    c1_sum += c1;
-    saved_sum += saved;
+    const int word = split_word_of(ents + q0, (int)(q - q0), mt * n, tc, cls_smax[cls], tile_max,
+                                   slot_elems, sums);
+    dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, word);
   }
 }
 
-// all C blocks; sums[0] += unsplit FP64 instruction counts, sums[1] += split savings
-__global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
+// all C blocks
+__global__ void __launch_bounds__(256, 4)
+    k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
                             const int32_t *__restrict__ run_start, const int32_t *__restrict__ run_len,
                             const int32_t *__restrict__ s_a, const int32_t *__restrict__ s_b,
                             const int64_t *__restrict__ c_off, const int32_t *__restrict__ c_cin,
@@ -957,53 +986,36 @@ __global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
                             SchedTabs S, int32_t *__restrict__ desc, int4 *__restrict__ ents,
                             int32_t *__restrict__ key, const int32_t *__restrict__ cls_smax,
                             const int32_t *__restrict__ t_start, int tile_max, int slot_elems,
-                            unsigned long long *__restrict__ sums) {
+                            SplitSums *__restrict__ sums) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  long long c1_sum = 0, saved_sum = 0;
+  SplitSums v = {};
   if (c < nc) f64_tiles_of(c, c_cls, run_start, run_len, s_a, s_b, c_off, c_cin, tbeg, ebeg, S,
-                           desc, ents, key, cls_smax, t_start, tile_max, slot_elems, c1_sum,
-                           saved_sum);
-  for (int o = 16; o > 0; o >>= 1) {
-    c1_sum += __shfl_down_sync(0xffffffffu, c1_sum, o);
-    saved_sum += __shfl_down_sync(0xffffffffu, saved_sum, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&sums[0], (unsigned long long)c1_sum);
-    if (saved_sum) atomicAdd(&sums[1], (unsigned long long)saved_sum);
-  }
+                           desc, ents, key, cls_smax, t_start, tile_max, slot_elems, v);
+  add_sums(v, sums);
 }
 
-// sums[0] += unsplit FP64 instruction counts, sums[1] += savings of the chosen splits
+// word 7 of every tile for new bounds of the inner split
 __global__ void k_f64_split(int64_t ntiles, const int4 *__restrict__ ents,
                             const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_smax,
                             int tile_max, int slot_elems, int32_t *__restrict__ desc,
-                            unsigned long long *__restrict__ sums) {
+                            SplitSums *__restrict__ sums) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  long long c1 = 0, saved = 0;
+  SplitSums v = {};
   if (t < ntiles) {
     int32_t *d = desc + t * kF64Desc;
     const int smax = cls_smax[c_cls[d[6]]];
     const int mn = (d[3] & 0xfff) * ((d[3] >> 12) & 0xfff);
     TailCost tc = tail_cost(mn, smax);
     for (int e = 0; e < d[2]; ++e) tail_add(tc, ents[(int64_t)d[1] + e].z);
-    c1 = tail_total(tc, mn);
-    const int split = f64_split_of(d, ents, smax, tile_max, slot_elems, c1, saved);
-    const int tail = tail_of(tc);
-    d[7] = f64_split_word(split, tail, f64_fresh(tc.w1, d[2], split, tail));
+    d[7] = split_word_of(ents + d[1], d[2], mn, tc, smax, tile_max, slot_elems, v);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    c1 += __shfl_down_sync(0xffffffffu, c1, o);
-    saved += __shfl_down_sync(0xffffffffu, saved, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&sums[0], (unsigned long long)c1);
-    atomicAdd(&sums[1], (unsigned long long)saved);
-  }
+  add_sums(v, sums);
 }
 
+// tail splits only: the word that every kernel instance runs the same way
 __global__ void k_f64_nosplit(int64_t ntiles, int32_t *__restrict__ desc) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < ntiles) desc[t * kF64Desc + 7] = f64_split_word(1, desc[t * kF64Desc + 7] >> 8);
+  if (t < ntiles) desc[t * kF64Desc + 7] = f64_split_word(1, (desc[t * kF64Desc + 7] >> 8) & 0xff);
 }
 
 __global__ void k_plan_items(int64_t nc, int64_t base, int64_t *__restrict__ item) {
@@ -1139,7 +1151,7 @@ void sort_items(const int64_t *items, const int32_t *keys, int64_t n, int64_t *o
 // stays 0) when a block size does not fit the descriptor's 12 bits, an inner size the
 // entries' 15, or a row of C (n elements) exceeds one output tile.
 static std::vector<int32_t> class_split_bounds(const bst_plan *p);
-static void apply_split_gate(bst_plan *p, const unsigned long long sums[2], cudaStream_t s);
+static void apply_split_gate(bst_plan *p, const SplitSums &sums, cudaStream_t s);
 
 static bool build_staged(bst_plan *p, cudaStream_t s) {
   p->stage_elems = 0;
@@ -1221,8 +1233,8 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
     if (slab) d_kin = up.add_vector(scratch, p->a_slab_kin);
     up.done_async();  // read by this stream's kernels below; the plan synchronises later
   }
-  unsigned long long *d_sums = scratch.alloc_n<unsigned long long>(2);
-  BST_CUDA(cudaMemsetAsync(d_sums, 0, 2 * sizeof(unsigned long long), s));
+  SplitSums *d_sums = scratch.alloc_n<SplitSums>(1);
+  BST_CUDA(cudaMemsetAsync(d_sums, 0, sizeof(SplitSums), s));
   SchedTabs S;
   S.cls_m = p->cls_m;
   S.cls_n = p->cls_n;
@@ -1266,10 +1278,10 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   k_plan_items<<<nblk(ntiles, 256), 256, 0, s>>>(ntiles, 0, it0);
   BST_CHECK_LAUNCH();
   sort_items(it0, p->tkeys, ntiles, p->titems, scratch, s);
-  unsigned long long sums[2] = {0, 0};
+  SplitSums sums = {};
   {
     ReadBack rb(p->ctx, s);
-    rb.add(sums, d_sums, sizeof(sums));
+    rb.add(&sums, d_sums, sizeof(sums));
     rb.done();
   }
   scratch.release_all();
@@ -1294,12 +1306,18 @@ static std::vector<int32_t> class_split_bounds(const bst_plan *p) {
   return smax;
 }
 
-// The plan runs the split instance only when the chosen splits save at least 1 % of all
-// its FP64 instructions (a safeguard: a longer loop body once cost every tile a few per
-// cent); otherwise every tile is set back to s = 1.
-static void apply_split_gate(bst_plan *p, const unsigned long long sums[2], cudaStream_t s) {
-  p->stage_split = sums[1] > 0 && kSplitGate * sums[1] >= sums[0];
-  if (!p->stage_split && sums[1] > 0) {  // with no saving every tile already has s = 1
+// The plan runs the split instance when its whole-tile splits save at least 1 % of all its FP64
+// instructions (a safeguard: a longer loop body once cost every tile a few per cent), when the
+// reference splits (choose_tile), whose accuracy the tiles keep, would save 4 % of the unsplit
+// ones, and always in the wide shape, which has no other.  Otherwise every tile is set back to
+// its tail split: a word then means the same in every instance, so that a plan gives the same
+// bits alone and in a batch that runs another plan's splits.
+constexpr unsigned long long kSplitGate = 100, kReferenceGate = 25;
+
+static void apply_split_gate(bst_plan *p, const SplitSums &v, cudaStream_t s) {
+  p->stage_split = v.marked > 0 && (p->stage_wide || (v.saved > 0 && kSplitGate * v.saved >= v.plain) ||
+                                    (v.reference > 0 && kReferenceGate * v.reference >= v.unsplit));
+  if (!p->stage_split && v.marked > 0) {
     k_f64_nosplit<<<nblk(p->n_tiles, 256), 256, 0, s>>>(p->n_tiles, p->fdesc);
     BST_CHECK_LAUNCH();
   }
@@ -1325,16 +1343,16 @@ void refresh_f64_split(bst_plan *p, cudaStream_t s) {
     d_smax = up.add_vector(scratch, smax);
     up.done();
   }
-  unsigned long long *d_sums = scratch.alloc_n<unsigned long long>(2);
-  BST_CUDA(cudaMemsetAsync(d_sums, 0, 2 * sizeof(unsigned long long), s));
+  SplitSums *d_sums = scratch.alloc_n<SplitSums>(1);
+  BST_CUDA(cudaMemsetAsync(d_sums, 0, sizeof(SplitSums), s));
   k_f64_split<<<nblk(p->n_tiles, 128), 128, 0, s>>>(p->n_tiles, p->fents, p->c_cls, d_smax,
                                                    32 * (p->stage_wide ? kWideR : kNarrowR),
                                                    p->stage_elems, p->fdesc, d_sums);
   BST_CHECK_LAUNCH();
-  unsigned long long sums[2] = {0, 0};
+  SplitSums sums = {};
   {
     ReadBack rb(p->ctx, s);
-    rb.add(sums, d_sums, sizeof(sums));
+    rb.add(&sums, d_sums, sizeof(sums));
     rb.done();
   }
   apply_split_gate(p, sums, s);
