@@ -1151,7 +1151,93 @@ void sort_items(const int64_t *items, const int32_t *keys, int64_t n, int64_t *o
 // stays 0) when a block size does not fit the descriptor's 12 bits, an inner size the
 // entries' 15, or a row of C (n elements) exceeds one output tile.
 static std::vector<int32_t> class_split_bounds(const bst_plan *p);
+static bool split_opens(const SplitSums &v, bool wide);
 static void apply_split_gate(bst_plan *p, const SplitSums &sums, cudaStream_t s);
+
+// FP64 instructions of the plan's tiles in one shape, as choose_tile counts them for tiles with
+// their class's average number of products
+static double shape_cost(const bst_plan *p, const std::vector<int32_t> &smax, bool wide) {
+  const int tile = 32 * (wide ? kWideR : kNarrowR), slot_max = wide ? kWideSlot : kNarrowSlot;
+  const int32_t ncls = p->Dm * p->Dn, Dk = p->Dk;
+  auto rows = [&](int64_t m, int64_t n) { return m * n <= tile ? m : tile / n; };
+  int64_t slot = 1;
+  for (int pass = 0; pass < 2; ++pass) {  // the slot size, then the counts
+    SplitSums v = {};
+    double split = 0.0, plain = 0.0;
+    for (int32_t cls = 0; cls < ncls; ++cls) {
+      const int64_t nblk = (int64_t)p->h_class_ptr[cls + 1] - p->h_class_ptr[cls];
+      if (nblk == 0) continue;
+      const int64_t m = p->m_vals[cls / p->Dn], n = p->n_vals[cls % p->Dn], tr = rows(m, n);
+      SplitSteps<long long> sum;
+      int64_t w1 = 0, ne = 0;
+      TailCost tc[2] = {tail_cost((int)(tr * n), smax[cls]), tail_cost((int)(m % tr * n), smax[cls])};
+      long long tc_sum[2][2] = {};
+      for (int32_t kc = 0; kc < Dk; ++kc) {
+        const int32_t b = cls * Dk + kc;
+        const int64_t cnt = (int64_t)p->h_bucket_ptr[b + 1] - p->h_bucket_ptr[b];
+        if (cnt == 0) continue;
+        const int64_t k = p->k_vals[kc], np = (k + slot_max / (tr + n) - 1) / (slot_max / (tr + n));
+        const int64_t w = (k + np - 1) / np;
+        if (pass == 0) {
+          slot = std::max(slot, (tr + n) * w);
+          continue;
+        }
+        for (int64_t l0 = 0; l0 < k; l0 += w) {
+          const int wl = (int)std::min(w, k - l0);
+          sum.add(wl, cnt);
+          for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j) tc_sum[i][j] += cnt * ((wl + tc[i].t[j] - 1) / tc[i].t[j]);
+        }
+        w1 += cnt * k;
+        ne += cnt * np;
+      }
+      if (pass == 0) continue;
+      for (long long &x : sum.steps) x /= nblk;
+      for (int i = 0; i < 2; ++i) {  // whole tiles, and the last rows
+        const int mn = (int)((i ? m % tr : tr) * n);
+        if (mn == 0) continue;
+        tc[i].w1 = w1 / nblk;
+        for (int j = 0; j < 2; ++j) tc[i].c[j] += tc_sum[i][j] / nblk;
+        const TileChoice R = choose_tile(tc[i], sum, mn, ne / nblk, smax[cls], tile, (int)slot);
+        const unsigned long long times = (unsigned long long)(nblk * (i ? 1 : m / tr));
+        v.plain += times * R.plain;
+        v.saved += times * R.saved;
+        v.unsplit += times * R.unsplit;
+        v.reference += times * R.reference;
+        v.marked += R.split > 1 || R.fresh || R.tail_fresh;
+        split += (double)times * R.cost;
+        plain += (double)times * R.plain;
+      }
+    }
+    if (pass == 1) return split_opens(v, wide) ? split : plain;
+  }
+  return 0.0;
+}
+
+// Whether the wide shape runs a plan that the narrow one could: where its whole-tile splits (544
+// accumulators instead of 320) and wider panels save more instructions than the fourth CTA is
+// worth: with 60 products of 35, counted 1.04 times as many in the narrow shape, 10 x 10 blocks
+// take 9.33 ms narrow and 9.29 wide; 1.03, 5 x 13 blocks 6.28 and 6.35; 1.12, 5 x 23 blocks 12.1
+// and 10.7; at equal counts the wide shape takes 1.05 to 1.1 times as long.  Only long sums over small blocks can gain, and only bases of few sizes are counted (a
+// pass over classes and inner sizes on the host).
+constexpr double kWideGain = 1.06;
+constexpr int32_t kShapeBuckets = 1024;
+
+static bool wide_saves(const bst_plan *p, const std::vector<int32_t> &smax) {
+  if (p->nb_all > kShapeBuckets) return false;
+  bool may = false;
+  for (int32_t cls = 0; cls < p->Dm * p->Dn && !may; ++cls) {
+    const int64_t nblk = (int64_t)p->h_class_ptr[cls + 1] - p->h_class_ptr[cls];
+    if (nblk == 0 || (int64_t)p->m_vals[cls / p->Dn] * p->n_vals[cls % p->Dn] > 16 * kWideR) continue;
+    int64_t w1 = 0;
+    for (int32_t kc = 0; kc < p->Dk; ++kc) {
+      const int32_t b = cls * p->Dk + kc;
+      w1 += ((int64_t)p->h_bucket_ptr[b + 1] - p->h_bucket_ptr[b]) * p->k_vals[kc];
+    }
+    may = w1 >= kSplitMinInner * nblk;
+  }
+  return may && shape_cost(p, smax, false) >= kWideGain * shape_cost(p, smax, true);
+}
 
 static bool build_staged(bst_plan *p, cudaStream_t s) {
   p->stage_elems = 0;
@@ -1173,6 +1259,8 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
     wide = wide || n > 32 * kNarrowR ||
            (slab_wanted && m * n > 32 * kNarrowR && m * n <= 32 * kWideR);
   }
+  const std::vector<int32_t> smax = class_split_bounds(p);
+  wide = wide || (!slab_wanted && wide_saves(p, smax));
   const int tile = 32 * (wide ? kWideR : kNarrowR), slot_max = wide ? kWideSlot : kNarrowSlot;
   for (int32_t c = 0; c < ncls; ++c) {
     if (p->h_class_ptr[c + 1] == p->h_class_ptr[c]) continue;
@@ -1229,7 +1317,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
     Upload up(p->ctx, s);
     d_tr = up.add_vector(scratch, tile_rows);
     d_wp = up.add_vector(scratch, wpanel);
-    d_smax = up.add_vector(scratch, class_split_bounds(p));
+    d_smax = up.add_vector(scratch, smax);
     if (slab) d_kin = up.add_vector(scratch, p->a_slab_kin);
     up.done_async();  // read by this stream's kernels below; the plan synchronises later
   }
@@ -1314,9 +1402,13 @@ static std::vector<int32_t> class_split_bounds(const bst_plan *p) {
 // bits alone and in a batch that runs another plan's splits.
 constexpr unsigned long long kSplitGate = 100, kReferenceGate = 25;
 
+static bool split_opens(const SplitSums &v, bool wide) {
+  return v.marked > 0 && (wide || (v.saved > 0 && kSplitGate * v.saved >= v.plain) ||
+                          (v.reference > 0 && kReferenceGate * v.reference >= v.unsplit));
+}
+
 static void apply_split_gate(bst_plan *p, const SplitSums &v, cudaStream_t s) {
-  p->stage_split = v.marked > 0 && (p->stage_wide || (v.saved > 0 && kSplitGate * v.saved >= v.plain) ||
-                                    (v.reference > 0 && kReferenceGate * v.reference >= v.unsplit));
+  p->stage_split = split_opens(v, p->stage_wide);
   if (!p->stage_split && v.marked > 0) {
     k_f64_nosplit<<<nblk(p->n_tiles, 256), 256, 0, s>>>(p->n_tiles, p->fdesc);
     BST_CHECK_LAUNCH();

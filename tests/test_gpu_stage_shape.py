@@ -1,0 +1,47 @@
+"""Which shape of the staged native-FP64 kernel a plan takes, seen in the inner splits that only the
+wide one has room for (544 partial sums a tile against 320), and its results against the oracle.
+
+Tolerance: every output is an FP64 sum of at most 2100 products in some order, error below
+K 2^-53 relative to sum |a||b|; 1e-12 relative Frobenius leaves ample room."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import rel_fro, require_gpu, run_multiply
+from paper_1910_13555_gb300.workloads import Problem, make_matrix
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+def _dense(rng, m, n, k, nb, kb):
+    size = lambda v, c: np.full(c, v, np.int32)
+    grid = lambda r, c: [x.ravel().astype(np.int32) for x in np.meshgrid(range(r), range(c), indexing="ij")]
+    return Problem(make_matrix(rng, size(m, nb), size(k, kb), *grid(nb, kb)),
+                   make_matrix(rng, size(k, kb), size(n, nb), *grid(kb, nb)), None)
+
+
+# (m, n, k, products per block): split of every tile in the wide shape
+@pytest.mark.parametrize("m,n,k,kb,split", [(9, 9, 35, 60, 5), (7, 7, 35, 60, 7), (5, 23, 35, 60, 3),
+                                            (23, 5, 35, 60, 3), (13, 13, 35, 60, 3)])
+def test_long_sums_of_small_blocks_take_the_wide_shape(m, n, k, kb, split):
+    p = _dense(np.random.default_rng(m + n), m, n, k, 9, kb)
+    out = run_multiply(p, stacks=False)
+    assert out["plan"].split_histogram()[split] == 81
+    ref = oracle.multiply(p.A, p.B, None, 1.0, 0.0, 0.0)
+    assert rel_fro(out["data"], ref["data"]) <= 1e-12
+
+
+# equal counts in both shapes, or a tail split that the narrow shape runs with a fourth CTA
+@pytest.mark.parametrize("m,n,k,kb,split", [(5, 5, 35, 60, 5), (5, 13, 35, 60, 16), (9, 9, 13, 60, 1),
+                                            (5, 13, 35, 2, 4)])
+def test_others_stay_narrow(m, n, k, kb, split):
+    p = _dense(np.random.default_rng(m + n), m, n, k, 9, kb)
+    out = run_multiply(p, stacks=False)
+    assert out["plan"].split_histogram()[split] == 81
+    ref = oracle.multiply(p.A, p.B, None, 1.0, 0.0, 0.0)
+    assert rel_fro(out["data"], ref["data"]) <= 1e-12
