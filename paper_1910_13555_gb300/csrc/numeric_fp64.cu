@@ -1250,17 +1250,21 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   if (nc == 0 || p->T == 0) return false;
   const int32_t ncls = p->Dm * p->Dn, Dk = p->Dk;
   std::vector<int32_t> tile_rows((size_t)ncls, 1), wpanel((size_t)ncls * Dk, 1);
-  // the wide shape: rows of C, or whole C blocks of a slab-read operand, above a narrow tile
+  // the wide shape: rows of C, or whole C blocks of a slab-read operand, above a narrow tile (a
+  // block above a wide tile too rules the slab reading out)
   const bool slab_wanted = !p->a_slab_kin.empty() && !p->ta && p->a_slab_toff;
   bool wide = false;
+  int64_t largest = 0;
   for (int32_t c = 0; c < ncls; ++c) {
     if (p->h_class_ptr[c + 1] == p->h_class_ptr[c]) continue;
     const int64_t m = p->m_vals[c / p->Dn], n = p->n_vals[c % p->Dn];
-    wide = wide || n > 32 * kNarrowR ||
-           (slab_wanted && m * n > 32 * kNarrowR && m * n <= 32 * kWideR);
+    wide = wide || n > 32 * kNarrowR;
+    largest = std::max(largest, m * n);
   }
+  const bool slab_fits = slab_wanted && largest <= 32 * kWideR;
+  wide = wide || (slab_fits && largest > 32 * kNarrowR);
   const std::vector<int32_t> smax = class_split_bounds(p);
-  wide = wide || (!slab_wanted && wide_saves(p, smax));
+  wide = wide || (!slab_fits && wide_saves(p, smax));
   const int tile = 32 * (wide ? kWideR : kNarrowR), slot_max = wide ? kWideSlot : kNarrowSlot;
   for (int32_t c = 0; c < ncls; ++c) {
     if (p->h_class_ptr[c + 1] == p->h_class_ptr[c]) continue;
@@ -1275,7 +1279,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
     if (p->h_class_ptr[c + 1] > p->h_class_ptr[c] && tile_rows[(size_t)c] < p->m_vals[c / p->Dn])
       (p->ta ? strided : tiled) = true;
   // slab reading of A: whole C blocks only (a slab holds all m rows), op(A) = A
-  const bool slab = slab_wanted && !strided && !tiled;
+  const bool slab = slab_fits && !strided && !tiled;
   if (slab) strided = true;
   // panel widths, slot size, and the tiles and entries of all C blocks (from the class and
   // bucket counts)

@@ -45,3 +45,24 @@ def test_others_stay_narrow(m, n, k, kb, split):
     assert out["plan"].split_histogram()[split] == 81
     ref = oracle.multiply(p.A, p.B, None, 1.0, 0.0, 0.0)
     assert rel_fro(out["data"], ref["data"]) <= 1e-12
+
+
+def test_slab_reading_that_a_block_rules_out_keeps_the_narrow_shape():
+    import torch
+    from paper_1910_13555_gb300 import bst
+    from paper_1910_13555_gb300.workloads import _tensor
+    rng = np.random.default_rng(3)
+    P, nu = np.full(6, 3, np.int32), np.full(5, 7, np.int32)
+    mu = np.array([20, 24, 20, 24], np.int32)  # C blocks of 400 to 576 elements
+    every = lambda *n: np.stack([x.ravel() for x in np.meshgrid(*map(range, n), indexing="ij")], 1)
+    T, U = _tensor(rng, [P, mu, nu], every(6, 4, 5)), _tensor(rng, [P, nu, mu], every(6, 5, 4))
+    lib = lambda t: bst.Tensor.from_host(t.block_sizes, t.index, t.data)
+    keep = lib(T), lib(U)
+    plan = bst.contract_plan(*keep, [0, 2], [0, 1], [1], [2], None, None, 0.0)
+    plan.alloc_result()
+    assert not plan.schedule_info()["slab"]
+    assert plan.split_histogram().sum() == 2 * 16  # tiles of at most 320 elements
+    plan.execute(1.0, 0.0)
+    torch.cuda.synchronize()
+    ref = oracle.contract(T, U, [0, 2], [0, 1], [1], [2])
+    assert rel_fro(plan.result.data[:plan.result.info[2]].cpu().numpy(), ref["data"]) <= 1e-12
