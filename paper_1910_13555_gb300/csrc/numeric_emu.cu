@@ -30,8 +30,8 @@
 // runs one warp per C block (its 16 x 8 tiles one after another; no two warps write the
 // same element), taking consecutive C blocks in chunks from a counter; the tile rows may
 // run over the C block's columns instead (C^T = op(B)^T op(A)^T on the same slices),
-// chosen per (m, n) class by the autotuner.  The 3xTF32 kernel runs one warp per 16 x 16
-// tile.  The operand slices are staged once per execute in a padded, permuted layout that
+// chosen per (m, n) class by the autotuner.  The 3xTF32 kernel runs one warp per pass
+// of 16 x 24 (or 16 x 8) outputs.  The operand slices are staged once per execute in a padded, permuted layout that
 // makes every fragment a single 8-byte load at a fixed offset (inner dimension padded
 // with zeros to the MMA K, a chunk's slices side by side, and permuted inside each chunk
 // so a thread's four values are adjacent).
@@ -51,6 +51,8 @@ constexpr int kSegChunks = 2;  // 16-wide K chunks per exact FP32 segment (32 el
 constexpr int kExpNone = -4000;
 constexpr int kDescWords = 8;  // int32 words per C block descriptor of the BF16 kernel
 
+constexpr int kTfCols = 3;  // 16 x 8 tiles side by side in a pass of the 3xTF32 kernel, at most
+
 struct EmuState {
   Arena ar;
   bool index_ready = false;
@@ -69,9 +71,11 @@ struct EmuState {
   float *a_tf = nullptr, *b_tf = nullptr;
   int32_t *a_exp = nullptr, *b_exp = nullptr;
   bool dig_alloc = false, tf_alloc = false, tf_lists = false;
-  // 3xTF32: C-major entries and C block descriptors (k_tf32_ents, k_tf32_desc)
+  // 3xTF32: C-major entries and the passes' descriptors (k_tf32_ents, k_tf32_units)
   int4 *tents = nullptr;
   int32_t *tdesc = nullptr;
+  int tf_cols = kTfCols;
+  int64_t nunits = 0;
   // C-major stack entries of the BF16 kernel (int4 each) and where each C block's start
   int4 *ents = nullptr;
   int64_t *ebeg = nullptr;
@@ -308,31 +312,62 @@ __global__ void k_emu_ents(int64_t nc, int32_t Dk, const int32_t *__restrict__ r
   }
 }
 
-constexpr int kTfCols = 3;  // 16 x 8 tiles side by side in a pass of the 3xTF32 kernel
+// passes of an m x n C block (cols tiles each); swap: their rows run over the C block's columns
+// when that takes fewer passes, or as many of fewer 16 x 8 tiles
+__host__ __device__ inline int64_t tf32_passes(int m, int n, int cols, bool &swap) {
+  auto cost = [&](int64_t r, int64_t c, int64_t &passes) {
+    const int64_t mt = (r + 15) / 16, nt = (c + 7) / 8;
+    passes = mt * ((nt + cols - 1) / cols);
+    return mt * nt;
+  };
+  int64_t p, ps;
+  const int64_t t = cost(m, n, p), ts = cost(n, m, ps);
+  swap = ps < p || (ps == p && ts < t);
+  return swap ? ps : p;
+}
+
+// passes of every C block
+__global__ void k_tf32_passes(int64_t nc, const int32_t *__restrict__ c_cls,
+                              const int32_t *__restrict__ cls_m, const int32_t *__restrict__ cls_n,
+                              int cols, int64_t *__restrict__ cnt) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= nc) return;
+  bool sw;
+  cnt[c] = tf32_passes(cls_m[c_cls[c]], cls_n[c_cls[c]], cols, sw);
+}
+
+// 3xTF32 work units, a pass each (a C block's start at ubeg[c]; null: one pass per block): 0
+// element offset, 1 first entry, 2 entry count, 3 C_in block (-1: none), 4 m, 5 n, 6 swap | row
+// pass << 1, 7 column pass.  A warp per C block writes them.
+__global__ void k_tf32_units(int64_t nc, const int64_t *__restrict__ ebeg,
+                             const int64_t *__restrict__ ubeg, const int64_t *__restrict__ c_off,
+                             const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_m,
+                             const int32_t *__restrict__ cls_n, const int32_t *__restrict__ c_cin,
+                             int cols, int32_t *__restrict__ desc) {
+  const int lane = threadIdx.x & 31;
+  const int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (c >= nc) return;
+  const int m = cls_m[c_cls[c]], n = cls_n[c_cls[c]];
+  bool sw;
+  const int64_t np = tf32_passes(m, n, cols, sw), u0 = ubeg ? ubeg[c] : c;
+  const int across = ((sw ? m : n) + 8 * cols - 1) / (8 * cols);
+  for (int64_t u = lane; u < np; u += 32) {
+    int4 *d = reinterpret_cast<int4 *>(desc + (u0 + u) * kDescWords);
+    d[0] = make_int4((int)c_off[c], (int)ebeg[c], (int)(ebeg[c + 1] - ebeg[c]), c_cin[c]);
+    d[1] = make_int4(m, n, (int)sw | (int)(u / across) << 1, (int)(u % across));
+  }
+}
 
 // 3xTF32: the C-major entry list (at ebeg[c] too), {A and B offsets / 16 floats, 8-wide
-// chunks of the inner size, 0}, and the C block descriptors: 0 element offset, 1 first
-// entry, 2 entry count, 3 C_in block (-1: none), 4 m, 5 n, 6 swap (tile rows run over the
-// C block's columns when that takes fewer passes, or as many of fewer 16 x 8 tiles)
+// chunks of the inner size, 0}
 __global__ void k_tf32_ents(int64_t nc, int32_t Dk, const int32_t *__restrict__ run_start,
                             const int32_t *__restrict__ run_len, const int32_t *__restrict__ kval,
                             const int32_t *__restrict__ s_ab, const int32_t *__restrict__ s_bb,
                             const int64_t *__restrict__ a_toff, const int64_t *__restrict__ b_toff,
-                            const int64_t *__restrict__ ebeg, const int64_t *__restrict__ c_off,
-                            const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_m,
-                            const int32_t *__restrict__ cls_n, const int32_t *__restrict__ c_cin,
-                            int4 *__restrict__ ents, int32_t *__restrict__ desc) {
+                            const int64_t *__restrict__ ebeg, int4 *__restrict__ ents) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nc) return;
   int64_t q = ebeg[c];
-  int4 *d = reinterpret_cast<int4 *>(desc + c * kDescWords);
-  const int m = cls_m[c_cls[c]], n = cls_n[c_cls[c]];
-  auto cost = [](int r, int c) {
-    const int64_t mt = (r + 15) / 16, nt = (c + 7) / 8;
-    return (mt * ((nt + kTfCols - 1) / kTfCols) << 32) + mt * nt;
-  };
-  d[0] = make_int4((int)c_off[c], (int)q, (int)(ebeg[c + 1] - q), c_cin[c]);
-  d[1] = make_int4(m, n, cost(n, m) < cost(m, n), 0);
   for (int kc = 0; kc < Dk; ++kc) {
     const int len = run_len[c * Dk + kc];
     if (len == 0) continue;
@@ -430,7 +465,7 @@ struct EmuParams {
   const int32_t *c_row, *c_col, *c_cin, *c_cls;
   const int64_t *c_off, *cin_off;
   const int32_t *run_start, *run_len, *s_ab, *s_bb;
-  const int32_t *desc;  // C block descriptors (kDescWords each)
+  const int32_t *desc;  // C block (3xTF32: pass) descriptors (kDescWords each)
   const int4 *ents;     // C-major entries
   const int64_t *a_doff, *b_doff, *a_eoff, *b_eoff;
   const __nv_bfloat16 *a_dig, *b_dig;
@@ -913,16 +948,19 @@ __global__ void __launch_bounds__(256, 2)
       [](const EmuParams &Q, int w) { emu_block<ROWS>(Q, emu_blk(w)); });
 }
 
-// ---- the 3xTF32 kernel: one warp per C block ----------------------------------------
+// ---- the 3xTF32 kernel: one warp per pass over a C block ----------------------------
 //
 // Its products are short (about two per C block, two or three 8-wide chunks each), so it is
 // bound by instruction issue and by the chain of dependent index reads in front of the
-// operand loads, not by the tensor pipe.  A warp takes whole C blocks from the counter and
-// runs each in passes of 16 rows x 24 columns of the (possibly transposed) block, where one
-// 16-byte load gives a lane the high and low parts of a fragment.  There is one pass body of
-// runtime size: bodies per tile count filled the instruction cache (5.6 of 13 cycles per
-// instruction waited for it; 5.86 ms on the 2000 x 2000 banded product at 2 % against 3.22
-// now, and 7.74 with a warp per 16 x 16 tile walking the stacks).  Instructions are what to
+// operand loads, not by the tensor pipe.  A warp takes passes of 16 rows x 24 columns of the
+// (possibly transposed) block from the counter, where one 16-byte load gives a lane the high and
+// low parts of a fragment.  A whole C block per warp was no faster on small blocks (3.22 ms on
+// the banded product below, 3.16 now) and left large or few ones to few warps: 16 blocks of
+// 512 x 512 84 ms against 7.3, 1600 blocks of 5, 13 and 23 with 60 products each 0.31 against
+// 0.15 (passes of one tile, which have registers for four chunks in flight).  There is one pass
+// body of runtime size: bodies per tile count filled the instruction cache (5.6 of 13 cycles per
+// instruction waited for it; 5.86 ms on the 2000 x 2000 banded product at 2 % against 3.22,
+// and 7.74 with a warp per 16 x 16 tile walking the stacks).  Instructions are what to
 // save: operand rows past a pass's edge are read again instead of predicated, a block's first
 // product is its sum without a TwoSum.  Loading the next fragments during the current MMAs
 // costs spills (4.24 ms), staging them through shared memory instructions and warps (4.37),
@@ -930,7 +968,8 @@ __global__ void __launch_bounds__(256, 2)
 // FP64 adds, 16 cycles a warp instruction, run on full warps and the stores are contiguous.
 // Per element the MMAs and sums run in the order entry, chunk, {a_lo b_hi, a_hi b_lo,
 // a_hi b_hi} whatever the tile orientation.
-constexpr int kTfPitch = 8 * kTfCols + 1;  // float2 per row of the pass in shared memory
+// float2 per row of a pass of COLS tiles in shared memory
+constexpr int tf32_pitch(int cols) { return 8 * cols + 1; }
 
 __device__ __forceinline__ void mma_tf32f(float (&d)[4], float a0, float a1, float a2, float a3,
                                           float b0, float b1) {
@@ -939,31 +978,32 @@ __device__ __forceinline__ void mma_tf32f(float (&d)[4], float a0, float a1, flo
 }
 
 struct TfBlk {
-  int off, eb, ne, cin, m, n, sw;
+  int off, eb, ne, cin, m, n, sw, r00, c00;
 };
 
-// the pass from row r00, column c00 of the block (of its transpose when it runs swapped)
-__device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, int r00, int c00,
-                                          const int4 &ent0, float2 *__restrict__ sm) {
+// the pass from row b.r00, column b.c00 of the block (of its transpose when it runs swapped)
+template <int COLS>
+__device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, const int4 &ent0,
+                                          float2 *__restrict__ sm) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int RM = b.sw ? b.n : b.m, RN = b.sw ? b.m : b.n;
-  const int rows = min(16, RM - r00), cols = min(8 * kTfCols, RN - c00);
+  const int RM = b.sw ? b.n : b.m, RN = b.sw ? b.m : b.n, r00 = b.r00, c00 = b.c00;
+  const int rows = min(16, RM - r00), cols = min(8 * COLS, RN - c00);
   const float4 *X = reinterpret_cast<const float4 *>(b.sw ? P.b_tf : P.a_tf);
   const float4 *Y = reinterpret_cast<const float4 *>(b.sw ? P.a_tf : P.b_tf);
   // running sum over the block products as an unevaluated FP32 pair (hi + lo), each
   // product added with an error-free TwoSum, so the sum over many products keeps about
   // twice FP32's precision
-  float hi[kTfCols][4], lo[kTfCols][4], acc[kTfCols][4];
+  float hi[COLS][4], lo[COLS][4], acc[COLS][4];
 #pragma unroll
-  for (int j = 0; j < kTfCols; ++j)
+  for (int j = 0; j < COLS; ++j)
 #pragma unroll
     for (int h = 0; h < 4; ++h) hi[j][h] = lo[j][h] = acc[j][h] = 0.f;
   // the lane's operand rows and columns; past the pass's edge it reads the last one again
   // (an output depends on its own row and column only, and those outputs are not stored)
   const int ra0 = r00 + min(g, rows - 1), ra1 = r00 + min(g + 8, rows - 1);
-  int cb[kTfCols];
+  int cb[COLS];
 #pragma unroll
-  for (int q = 0; q < kTfCols; ++q) cb[q] = c00 + min(g + 8 * q, cols - 1);
+  for (int q = 0; q < COLS; ++q) cb[q] = c00 + min(g + 8 * q, cols - 1);
   int4 ent = ent0;
   for (int e = 0; e < b.ne; ++e) {
     if (e > 0 && (e & 31) == 0)
@@ -973,18 +1013,18 @@ __device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, in
     const int rs = 4 * __shfl_sync(kFull, ent.z, e & 31);  // float4 per row: 4 per chunk of 8
     const float4 *x = X + 4 * (size_t)(b.sw ? eb : ea) + t, *y = Y + 4 * (size_t)(b.sw ? ea : eb) + t;
     const float4 *x0 = x + (int64_t)ra0 * rs, *x1 = x + (int64_t)ra1 * rs;
-    const float4 *yq[kTfCols];
+    const float4 *yq[COLS];
 #pragma unroll
-    for (int q = 0; q < kTfCols; ++q) yq[q] = y + (int64_t)cb[q] * rs;
-#pragma unroll 1
+    for (int q = 0; q < COLS; ++q) yq[q] = y + (int64_t)cb[q] * rs;
+#pragma unroll(COLS == 1 ? 4 : 1)
     for (int o = 0; o < rs; o += 4) {
       const float4 a0 = __ldg(x0 + o), a1 = __ldg(x1 + o);
-      float4 f[kTfCols];
+      float4 f[COLS];
 #pragma unroll
-      for (int q = 0; q < kTfCols; ++q)
+      for (int q = 0; q < COLS; ++q)
         if (8 * q < cols) f[q] = __ldg(yq[q] + o);
 #pragma unroll
-      for (int q = 0; q < kTfCols; ++q) {
+      for (int q = 0; q < COLS; ++q) {
         if (8 * q >= cols) break;
         if (b.sw) {  // rows are op(B)'s: its high part times op(A)'s low part first
           mma_tf32f(acc[q], a0.x, a1.x, a0.y, a1.y, f[q].z, f[q].w);
@@ -998,7 +1038,7 @@ __device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, in
     }
     if (e == 0) {  // 0 + v: the low part is 0 (NaN where v is not finite)
 #pragma unroll
-      for (int q = 0; q < kTfCols; ++q)
+      for (int q = 0; q < COLS; ++q)
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
           hi[q][h] = __fadd_rn(0.f, acc[q][h]);
@@ -1008,7 +1048,7 @@ __device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, in
       continue;
     }
 #pragma unroll
-    for (int q = 0; q < kTfCols; ++q) {
+    for (int q = 0; q < COLS; ++q) {
       if (8 * q >= cols) break;
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
@@ -1023,18 +1063,18 @@ __device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, in
     }
   }
 #pragma unroll
-  for (int q = 0; q < kTfCols; ++q) {
+  for (int q = 0; q < COLS; ++q) {
     if (8 * q >= cols) break;
 #pragma unroll
     for (int h = 0; h < 4; ++h)
-      sm[(g + 8 * (h >> 1)) * kTfPitch + 8 * q + 2 * t + (h & 1)] = make_float2(hi[q][h], lo[q][h]);
+      sm[(g + 8 * (h >> 1)) * tf32_pitch(COLS) + 8 * q + 2 * t + (h & 1)] = make_float2(hi[q][h], lo[q][h]);
   }
   __syncwarp();
   // outputs in C order: (outer, inner) = (row, column) of the pass, or swapped
   const double *ci = (P.has_beta && b.cin >= 0) ? P.Cin + P.cin_off[b.cin] : nullptr;
   const int64_t c0 = b.sw ? (int64_t)c00 * b.n + r00 : (int64_t)r00 * b.n + c00;
   const int ni = b.sw ? rows : cols, total = rows * cols;
-  const int so = b.sw ? 1 : kTfPitch, si = b.sw ? kTfPitch : 1;
+  const int so = b.sw ? 1 : tf32_pitch(COLS), si = b.sw ? tf32_pitch(COLS) : 1;
   const int di = 32 % ni, dO = 32 / ni;
   int x = lane % ni;
   const float2 *from = sm + (lane / ni) * so + x * si;
@@ -1065,7 +1105,8 @@ __device__ __forceinline__ void tf32_pass(const EmuParams &P, const TfBlk &b, in
   __syncwarp();
 }
 
-__device__ __forceinline__ void tf32_block(const EmuParams &P, int dw, float2 *sm) {
+template <int COLS>
+__device__ __forceinline__ void tf32_unit(const EmuParams &P, int dw, float2 *sm) {
   const int lane = threadIdx.x & 31;
   TfBlk b;
   b.off = __shfl_sync(kFull, dw, 0);
@@ -1074,22 +1115,22 @@ __device__ __forceinline__ void tf32_block(const EmuParams &P, int dw, float2 *s
   b.cin = __shfl_sync(kFull, dw, 3);
   b.m = __shfl_sync(kFull, dw, 4);
   b.n = __shfl_sync(kFull, dw, 5);
-  b.sw = __shfl_sync(kFull, dw, 6);
+  const int r = __shfl_sync(kFull, dw, 6);
+  b.sw = r & 1;
+  b.r00 = (int)((unsigned)r >> 1) * 16;
+  b.c00 = __shfl_sync(kFull, dw, 7) * 8 * COLS;
   const int4 ent0 = lane < b.ne ? P.ents[(int64_t)b.eb + lane] : make_int4(0, 0, 0, 0);
-  const int RM = b.sw ? b.n : b.m, RN = b.sw ? b.m : b.n;
-#pragma unroll 1
-  for (int r = 0; r < RM; r += 16)
-#pragma unroll 1
-    for (int c = 0; c < RN; c += 8 * kTfCols) tf32_pass(P, b, r, c, ent0, sm);
+  tf32_pass<COLS>(P, b, ent0, sm);
 }
 
+template <int COLS>
 __global__ void __launch_bounds__(256, 2)
     k_num_tf32x3(EmuParams P, int64_t nitems, unsigned long long *counter, int take) {
-  __shared__ float2 sums[8][16 * kTfPitch];
+  __shared__ float2 sums[8][16 * tf32_pitch(COLS)];
   float2 *sm = sums[threadIdx.x >> 5];
   emu_persist(
       nullptr, nitems, counter, [&](int64_t) -> const EmuParams & { return P; },
-      [&](const EmuParams &Q, int w) { tf32_block(Q, w, sm); }, take);
+      [&](const EmuParams &Q, int w) { tf32_unit<COLS>(Q, w, sm); }, take);
 }
 
 SideArgs side_args(const bst_matrix *X, bool trans, bool is_b) {
@@ -1460,6 +1501,32 @@ void emu_costs(bst_plan *p, cudaStream_t s, double *tensor_flops, double *bytes,
            16.0 * (double)p->T + 4.0 * kDescWords * (double)p->C->nblocks;
 }
 
+// CTAs of 8 warps that the device holds at once
+static int64_t tf32_ctas(int cols, int num_sms) {
+  auto kernel = cols == 1 ? k_num_tf32x3<1> : k_num_tf32x3<kTfCols>;
+  int per = 0;
+  BST_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, 256, 0));
+  return (int64_t)std::max(per, 1) * num_sms;
+}
+
+// Passes of three tiles while they fill the device's warps: with 40 x 40 C blocks of 23 (3200
+// passes for 2432 warps) three tiles take 0.199 ms and one tile 0.240, with blocks of 5, 13 and 23
+// (1804) 0.193 and 0.150.
+static void tf32_choose(const bst_plan *p, EmuState &E) {
+  const int64_t warps = 8 * tf32_ctas(kTfCols, p->ctx->num_sms);
+  for (int cols : {kTfCols, 1}) {
+    E.tf_cols = cols;
+    E.nunits = 0;
+    for (int32_t c = 0; c < p->Dm * p->Dn; ++c) {
+      const int64_t cnt = (int64_t)p->h_class_ptr[c + 1] - p->h_class_ptr[c];
+      bool sw;
+      if (cnt > 0)
+        E.nunits += cnt * tf32_passes(p->m_vals[c / p->Dn], p->n_vals[c % p->Dn], cols, sw);
+    }
+    if (E.nunits >= warps) return;
+  }
+}
+
 void execute_tf32x3(bst_plan *p, const NumArgs &a, cudaStream_t s) {
   if (p->C->nblocks == 0) return;
   EmuState &E = emu_state(p, s);
@@ -1468,15 +1535,28 @@ void execute_tf32x3(bst_plan *p, const NumArgs &a, cudaStream_t s) {
     E.a_tf = E.ar.alloc_n<float>((size_t)E.a_tsize);
     E.b_tf = E.ar.alloc_n<float>((size_t)E.b_tsize);
     E.tents = E.ar.alloc_n<int4>((size_t)std::max<int64_t>(p->T, 1));
-    E.tdesc = E.ar.alloc_n<int32_t>((size_t)nc * kDescWords);
+    tf32_choose(p, E);
+    E.tdesc = E.ar.alloc_n<int32_t>((size_t)E.nunits * kDescWords);
     if (!E.counter) E.counter = E.ar.alloc_n<unsigned long long>(1);
     E.tf_alloc = true;
   }
   if (!E.tf_lists) {
     k_tf32_ents<<<nblk(nc, 256), 256, 0, s>>>(nc, p->Dk, p->run_start, p->run_len, p->kval, p->s_ab,
-                                              p->s_bb, E.a_toff, E.b_toff, E.ebeg, p->C->off,
-                                              p->c_cls, p->cls_m, p->cls_n, p->c_cin, E.tents,
-                                              E.tdesc);
+                                              p->s_bb, E.a_toff, E.b_toff, E.ebeg, E.tents);
+    BST_CHECK_LAUNCH();
+    Arena scratch;
+    scratch.ctx = static_cast<Ctx *>(p->ctx);
+    scratch.stream = s;
+    int64_t *ubeg = nullptr;
+    if (E.nunits != nc) {
+      int64_t *cnt = scratch.alloc_n<int64_t>((size_t)nc);
+      ubeg = scratch.alloc_n<int64_t>((size_t)nc + 1);
+      k_tf32_passes<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->cls_m, p->cls_n, E.tf_cols, cnt);
+      BST_CHECK_LAUNCH();
+      exscan_i64(cnt, ubeg, nc, scratch, s);
+    }
+    k_tf32_units<<<nblk(nc, 8), 256, 0, s>>>(nc, E.ebeg, ubeg, p->C->off, p->c_cls, p->cls_m,
+                                             p->cls_n, p->c_cin, E.tf_cols, E.tdesc);
     BST_CHECK_LAUNCH();
     // the lists serve later executes on any stream; an execute captured before they are
     // built builds them in its graph, on every replay
@@ -1501,14 +1581,15 @@ void execute_tf32x3(bst_plan *p, const NumArgs &a, cudaStream_t s) {
   EmuParams P = emu_params(p, E, a);
   P.desc = E.tdesc;
   P.ents = E.tents;
-  int per = 0;
-  BST_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_num_tf32x3, 32 * wpb, 0));
-  const int64_t full = (int64_t)std::max(per, 1) * p->ctx->num_sms;
-  // few C blocks: one at a time, so that every warp gets some
-  const int take = nc >= 4 * kChunk * wpb * full ? kChunk : 1;
-  const int g = (int)std::min<int64_t>(full, (nc + wpb * take - 1) / (wpb * take));
+  const int64_t full = tf32_ctas(E.tf_cols, p->ctx->num_sms), nu = E.nunits;
+  // few passes: one at a time, so that every warp gets some
+  const int take = nu >= 4 * kChunk * wpb * full ? kChunk : 1;
+  const int g = (int)std::min<int64_t>(full, (nu + wpb * take - 1) / (wpb * take));
   BST_CUDA(cudaMemsetAsync(E.counter, 0, sizeof(unsigned long long), s));
-  k_num_tf32x3<<<g, 32 * wpb, 0, s>>>(P, nc, E.counter, take);
+  if (E.tf_cols == 1)
+    k_num_tf32x3<1><<<g, 32 * wpb, 0, s>>>(P, nu, E.counter, take);
+  else
+    k_num_tf32x3<kTfCols><<<g, 32 * wpb, 0, s>>>(P, nu, E.counter, take);
   BST_CHECK_LAUNCH();
 }
 
