@@ -131,14 +131,27 @@ __host__ __device__ __forceinline__ int split_bound(int smax, int mn, int elems,
 // Whether choose_tile may split a tile and reads `steps`.  A split saves at most the idle lanes,
 // so short tiles (which split for 1/8 of the instructions) need 1/8 of them idle: the 1.3 M tiles
 // of the 4000 x 4000 banded plan are mostly short, and going through their splits took 0.25 ms.
-__host__ __device__ __forceinline__ bool tile_may_split(long long w1, int smax, int mn, int slot) {
+__host__ __device__ __forceinline__ bool tile_may_split(long long w1, int smax, int mn, int tile,
+                                                        int slot, bool whole) {
   const int lanes = (mn + 31) & ~31, idle = lanes - mn;
   return w1 >= kSplitMinInner && idle > 0 && (w1 >= kSplitLongInner || 8 * idle >= lanes) &&
-         split_bound(smax, mn, 32 * kWideR, slot) >= 2;
+         split_bound(smax, mn, whole ? 32 * kWideR : tile, slot) >= 2;
+}
+
+// the choice for a tile that tile_may_split turns down (see below)
+__host__ __device__ __forceinline__ TileChoice choose_tile(const TailCost &C, int mn, long long ne) {
+  TileChoice R;
+  R.tail = tail_of(C);
+  R.plain = R.cost = tail_total(C, mn);
+  R.unsplit = ((mn + 31) >> 5) * C.w1;
+  R.fresh = R.tail > 1 && mn >= 32 && C.w1 >= kSplitLongInner && C.w1 >= 16 * ne;
+  R.cost += R.fresh ? kFreshAdd * (mn >> 5) * ne : 0;
+  return R;
 }
 
 // How a tile of mn outputs, ne panels and C.w1 inner elements in all sums them (tile: elements
-// of the largest tile of the plan's shape; slot: doubles of its slots).
+// of the largest tile of the plan's shape; slot: doubles of its slots; whole: the tile is a whole
+// block).
 //
 // An output of one chain over w1 elements rounds as sqrt(w1); the s partial sums of a whole-tile
 // split as sqrt(w1 / s + s), panels summed by themselves ("fresh") as sqrt(wmax + ne), at one add
@@ -146,30 +159,25 @@ __host__ __device__ __forceinline__ bool tile_may_split(long long w1, int smax, 
 // full rounds one chain: the relative error of 13 x 13 blocks with 60 products of 35 was 1.2e-15
 // that way, 4.4e-16 with the sums split in three.  So where a whole-tile split would pay (at
 // least 1/25 of the unsplit instructions, by the accumulators of the wide shape), it is the
-// reference: the tile takes the cheapest form whose chains are no longer than that split's.
+// reference: the tile takes the cheapest form whose chains are no longer than that split's.  Parts
+// of blocks have none (in the wide shape they would be larger), nor have panels that the slot cuts
+// to four elements, whose adds cost a third of the time (200 x 200 blocks 64 -> 84 ms).
 // Elsewhere one chain stays, except that long sums over wide panels beside a tail split are
 // fresh too (an add per 16 elements at most; the rank-3 contraction with gradients 2.1e-15, so
 // 0.8e-15, for 1 % of its time).
 template <class T>
 __host__ __device__ inline TileChoice choose_tile(const TailCost &C, const SplitSteps<T> &S, int mn,
-                                                  long long ne, int smax, int tile, int slot) {
-  TileChoice R;
+                                                  long long ne, int smax, int tile, int slot,
+                                                  bool whole) {
+  TileChoice R = choose_tile(C, mn, ne);
   const long long w1 = C.w1;
+  if (!tile_may_split(w1, smax, mn, tile, slot, whole)) return R;
   const unsigned inner = w1 < (1ll << 31) ? (unsigned)w1 : 1u << 31;  // for the chains' lengths
-  const int rounds = (mn + 31) >> 5;
-  R.tail = tail_of(C);
-  R.plain = R.cost = tail_total(C, mn);
-  R.unsplit = rounds * w1;
-  if (w1 < kSplitMinInner) return R;
-  const int full = R.tail > 1 ? mn >> 5 : rounds;
-  if (!tile_may_split(w1, smax, mn, slot)) {
-    R.fresh = R.tail > 1 && full > 0 && w1 >= kSplitLongInner && w1 >= 16 * ne;
-    R.cost += R.fresh ? kFreshAdd * full * ne : 0;
-    return R;
-  }
+  const int full = R.tail > 1 ? mn >> 5 : (mn + 31) >> 5;
   int s0 = 1;
   long long c0 = R.unsplit;
-  const int most = split_bound(smax, mn, 32 * kWideR, slot), now = split_bound(smax, mn, tile, slot);
+  const int now = split_bound(smax, mn, tile, slot);
+  const int most = whole && w1 > 4 * ne ? split_bound(smax, mn, 32 * kWideR, slot) : 1;
 #pragma unroll
   for (int s = 2; s <= kMaxSplit; ++s) {
     const long long c = split_cost(s, mn, S.steps[s]);
@@ -183,8 +191,10 @@ __host__ __device__ inline TileChoice choose_tile(const TailCost &C, const Split
   const long long limit = s0 > 1 ? inner / (unsigned)s0 + s0 : w1 + ne;
   long long chain = 0;  // the longest without a whole-tile split
   if (full > 0) {
-    R.fresh = s0 > 1 || (R.tail > 1 && w1 >= kSplitLongInner && w1 >= 16 * ne);
-    R.cost += R.fresh ? kFreshAdd * full * ne : 0;
+    if (s0 > 1 && !R.fresh) {
+      R.fresh = 1;
+      R.cost += kFreshAdd * full * ne;
+    }
     chain = R.fresh ? S.wmax + ne : w1;
   }
   if (R.tail > 1) {

@@ -885,14 +885,7 @@ __device__ __forceinline__ void add_sums(const SplitSums &v, SplitSums *__restri
   }
 }
 
-// word 7 of a tile whose entries are in place, its counts added to v
-__device__ __forceinline__ int split_word_of(const int4 *__restrict__ ents, int ne, int mn,
-                                             const TailCost &tc, int smax, int tile, int slot,
-                                             SplitSums &v) {
-  SplitSteps<unsigned> st;
-  if (tile_may_split(tc.w1, smax, mn, slot))
-    for (int e = 0; e < ne; ++e) st.add(ents[e].z);
-  const TileChoice R = choose_tile(tc, st, mn, ne, smax, tile, slot);
+__device__ __forceinline__ int count_choice(const TileChoice &R, SplitSums &v) {
   v.plain += R.plain;
   v.saved += R.saved;
   v.unsplit += R.unsplit;
@@ -900,6 +893,9 @@ __device__ __forceinline__ int split_word_of(const int4 *__restrict__ ents, int 
   v.marked += R.split > 1 || R.fresh || R.tail_fresh;
   return choice_word(R);
 }
+
+// word 7 of a tile whose split k_f64_split chooses
+constexpr int kSplitLater = -1;
 
 // descriptors and entries of every tile of C block c, each tile's cost key
 // (63 - floor(log2(flops)): a stable partition on it lists costly tiles first) and its
@@ -970,15 +966,17 @@ __device__ __forceinline__ void f64_tiles_of(
     dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)q0, (int32_t)(q - q0),
                       mt | (n << 12));
     key[tile] = __clzll(flops + 1ull);
-    const int word = split_word_of(ents + q0, (int)(q - q0), mt * n, tc, cls_smax[cls], tile_max,
-                                   slot_elems, sums);
+    // another pass over the entries costs registers that this kernel has not (plans of long row
+    // tiles 38 -> 47 ms)
+    const bool later = tile_may_split(tc.w1, cls_smax[cls], mt * n, tile_max, slot_elems, nt == 1);
+    const int word =
+        later ? kSplitLater : count_choice(choose_tile(tc, mt * n, (int)(q - q0)), sums);
     dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, word);
   }
 }
 
 // all C blocks
-__global__ void __launch_bounds__(256, 4)
-    k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
+__global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
                             const int32_t *__restrict__ run_start, const int32_t *__restrict__ run_len,
                             const int32_t *__restrict__ s_a, const int32_t *__restrict__ s_b,
                             const int64_t *__restrict__ c_off, const int32_t *__restrict__ c_cin,
@@ -994,20 +992,30 @@ __global__ void __launch_bounds__(256, 4)
   add_sums(v, sums);
 }
 
-// word 7 of every tile for new bounds of the inner split
+// word 7 of every tile for new bounds of the inner split; with `item`, only of the tiles that
+// k_f64_tiles left, and the work items 0 .. ntiles - 1
 __global__ void k_f64_split(int64_t ntiles, const int4 *__restrict__ ents,
-                            const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_smax,
-                            int tile_max, int slot_elems, int32_t *__restrict__ desc,
-                            SplitSums *__restrict__ sums) {
+                            const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_m,
+                            const int32_t *__restrict__ cls_smax, int tile_max, int slot_elems,
+                            int32_t *__restrict__ desc, SplitSums *__restrict__ sums,
+                            int64_t *__restrict__ item) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   SplitSums v = {};
   if (t < ntiles) {
     int32_t *d = desc + t * kF64Desc;
-    const int smax = cls_smax[c_cls[d[6]]];
-    const int mn = (d[3] & 0xfff) * ((d[3] >> 12) & 0xfff);
-    TailCost tc = tail_cost(mn, smax);
-    for (int e = 0; e < d[2]; ++e) tail_add(tc, ents[(int64_t)d[1] + e].z);
-    d[7] = split_word_of(ents + d[1], d[2], mn, tc, smax, tile_max, slot_elems, v);
+    if (item) item[t] = t;
+    if (!item || d[7] == kSplitLater) {
+      const int cls = c_cls[d[6]], smax = cls_smax[cls], ne = d[2];
+      const int m = d[3] & 0xfff, mn = m * ((d[3] >> 12) & 0xfff);
+      TailCost tc = tail_cost(mn, smax);
+      SplitSteps<unsigned> st;
+      for (int e = 0; e < ne; ++e) {
+        const int w = ents[(int64_t)d[1] + e].z;
+        tail_add(tc, w);
+        st.add(w);
+      }
+      d[7] = count_choice(choose_tile(tc, st, mn, ne, smax, tile_max, slot_elems, m == cls_m[cls]), v);
+    }
   }
   add_sums(v, sums);
 }
@@ -1198,7 +1206,7 @@ static double shape_cost(const bst_plan *p, const std::vector<int32_t> &smax, bo
         if (mn == 0) continue;
         tc[i].w1 = w1 / nblk;
         for (int j = 0; j < 2; ++j) tc[i].c[j] += tc_sum[i][j] / nblk;
-        const TileChoice R = choose_tile(tc[i], sum, mn, ne / nblk, smax[cls], tile, (int)slot);
+        const TileChoice R = choose_tile(tc[i], sum, mn, ne / nblk, smax[cls], tile, (int)slot, tr == m);
         const unsigned long long times = (unsigned long long)(nblk * (i ? 1 : m / tr));
         v.plain += times * R.plain;
         v.saved += times * R.saved;
@@ -1367,7 +1375,8 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   // tiles by decreasing cost
   int64_t *it0 = scratch.alloc_n<int64_t>((size_t)ntiles);
   p->titems = ar.alloc_n<int64_t>((size_t)ntiles);
-  k_plan_items<<<nblk(ntiles, 256), 256, 0, s>>>(ntiles, 0, it0);
+  k_f64_split<<<nblk(ntiles, 128), 128, 0, s>>>(ntiles, p->fents, p->c_cls, p->cls_m, d_smax, tile,
+                                                (int)slot, p->fdesc, d_sums, it0);
   BST_CHECK_LAUNCH();
   sort_items(it0, p->tkeys, ntiles, p->titems, scratch, s);
   SplitSums sums = {};
@@ -1441,9 +1450,9 @@ void refresh_f64_split(bst_plan *p, cudaStream_t s) {
   }
   SplitSums *d_sums = scratch.alloc_n<SplitSums>(1);
   BST_CUDA(cudaMemsetAsync(d_sums, 0, sizeof(SplitSums), s));
-  k_f64_split<<<nblk(p->n_tiles, 128), 128, 0, s>>>(p->n_tiles, p->fents, p->c_cls, d_smax,
+  k_f64_split<<<nblk(p->n_tiles, 128), 128, 0, s>>>(p->n_tiles, p->fents, p->c_cls, p->cls_m, d_smax,
                                                    32 * (p->stage_wide ? kWideR : kNarrowR),
-                                                   p->stage_elems, p->fdesc, d_sums);
+                                                   p->stage_elems, p->fdesc, d_sums, nullptr);
   BST_CHECK_LAUNCH();
   SplitSums sums = {};
   {

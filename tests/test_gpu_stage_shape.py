@@ -47,6 +47,17 @@ def test_others_stay_narrow(m, n, k, kb, split):
     assert rel_fro(out["data"], ref["data"]) <= 1e-12
 
 
+# rows of one tile each, whose slots hold panels of four elements: no split, no sum per panel (which
+# the wide instance alone would add: "split" tells)
+@pytest.mark.parametrize("m,n,k,kb", [(9, 200, 60, 6), (3, 200, 40, 6), (2, 199, 40, 6)])
+def test_narrow_panels_of_row_tiles_keep_one_chain(m, n, k, kb):
+    p = _dense(np.random.default_rng(n), m, n, k, 3, kb)
+    out = run_multiply(p, stacks=False)
+    assert not out["plan"].schedule_info()["split"]
+    ref = oracle.multiply(p.A, p.B, None, 1.0, 0.0, 0.0)
+    assert rel_fro(out["data"], ref["data"]) <= 1e-12
+
+
 def test_slab_reading_that_a_block_rules_out_keeps_the_narrow_shape():
     import torch
     from paper_1910_13555_gb300 import bst
