@@ -850,7 +850,8 @@ __global__ void k_f64_tile_count(int64_t nc, const int32_t *__restrict__ c_cls, 
 // entries of every tile of block c: sum over its products of the panel count
 __global__ void k_f64_ent_count(int64_t nc, const int32_t *__restrict__ c_cls,
                                 const int32_t *__restrict__ run_len, const int64_t *__restrict__ tbeg,
-                                SchedTabs S, int32_t *__restrict__ cnt) {
+                                SchedTabs S, int32_t *__restrict__ cnt,
+                                int32_t *__restrict__ tile_c) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nc) return;
   const int cls = c_cls[c];
@@ -860,7 +861,10 @@ __global__ void k_f64_ent_count(int64_t nc, const int32_t *__restrict__ c_cls,
     s += run_len[c * S.Dk + kc] * panel_count(k, w, S.kin ? S.kin[kc] : 0);
   }
   const int nt = ntiles_of(S, cls);
-  for (int t = 0; t < nt; ++t) cnt[tbeg[c] + t] = s;
+  for (int t = 0; t < nt; ++t) {
+    cnt[tbeg[c] + t] = s;
+    tile_c[tbeg[c] + t] = (int32_t)c;
+  }
 }
 
 // a plan's counters, summed over a CTA's tiles (an atomic per warp and counter took 0.25 ms of
@@ -897,11 +901,11 @@ __device__ __forceinline__ int count_choice(const TileChoice &R, SplitSums &v) {
 // word 7 of a tile whose split k_f64_split chooses
 constexpr int kSplitLater = -1;
 
-// descriptors and entries of every tile of C block c, each tile's cost key
-// (63 - floor(log2(flops)): a stable partition on it lists costly tiles first) and its
-// inner split, with its FP64 instruction counts added to sums
-__device__ __forceinline__ void f64_tiles_of(
-    int64_t c, const int32_t *__restrict__ c_cls, const int32_t *__restrict__ run_start,
+// descriptor and entries of a tile of C block c, its cost key (63 - floor(log2(flops)): a
+// stable partition on it lists costly tiles first) and its inner split, with its FP64 instruction
+// counts added to sums
+__device__ __forceinline__ void f64_tile_of(
+    int64_t tile, int64_t c, const int32_t *__restrict__ c_cls, const int32_t *__restrict__ run_start,
     const int32_t *__restrict__ run_len, const int32_t *__restrict__ s_a,
     const int32_t *__restrict__ s_b, const int64_t *__restrict__ c_off,
     const int32_t *__restrict__ c_cin, const int64_t *__restrict__ tbeg,
@@ -910,73 +914,71 @@ __device__ __forceinline__ void f64_tiles_of(
     const int32_t *__restrict__ t_start, int tile_max, int slot_elems, SplitSums &sums) {
   const int cls = c_cls[c];
   const int m = S.cls_m[cls], n = S.cls_n[cls], tr = S.tile_rows[cls];
-  const int nt = (m + tr - 1) / tr;
-  for (int t = 0; t < nt; ++t) {
-    const int64_t tile = tbeg ? tbeg[c] + t : c;
-    const int p0 = t * tr, mt = min(tr, m - p0);
-    const int64_t q0 = ebeg ? ebeg[tile] : t_start[c];
-    int64_t q = q0;
-    unsigned long long flops = 0;
-    TailCost tc = tail_cost(mt * n, cls_smax[cls]);
-    for (int kc = 0; kc < S.Dk; ++kc) {
-      const int len = run_len[c * S.Dk + kc];
-      if (len == 0) continue;
-      const int e0 = run_start[c * S.Dk + kc];
-      const int k = S.kval[kc], w = S.wpanel[cls * S.Dk + kc];
-      // stored row strides of the panels: A is m x k (k x m when transposed), B is k x n
-      // (n x k when transposed)
-      const int strides = (S.ta ? m : k) | ((S.tb ? k : n) << 16);
-      const int ki = S.kin ? S.kin[kc] : 0;
-      for (int e = e0; e < e0 + len; ++e) {
-        if (ki > 0) {
-          // slabs of the tensor block (whole blocks only: p0 == 0): stored row stride ki
-          const int64_t ab = S.a_toff[S.s_ab[e]];
-          const int st = ki | ((S.tb ? k : n) << 16);
-          if (w >= ki) {
-            const int ws = (w / ki) * ki;
-            for (int l0 = 0; l0 < k; l0 += ws) {
-              const int b = s_b[e] + (S.tb ? l0 : l0 * n);
-              ents[q++] = make_int4((int)(ab + (int64_t)(l0 / ki) * m * ki), b, min(ws, k - l0), st);
-              tail_add(tc, min(ws, k - l0));
-            }
-          } else {
-            for (int l0 = 0; l0 < k; l0 += ki)
-              for (int c0 = 0; c0 < ki; c0 += w) {
-                const int b = s_b[e] + (S.tb ? l0 + c0 : (l0 + c0) * n);
-                ents[q++] = make_int4((int)(ab + (int64_t)(l0 / ki) * m * ki + c0), b,
-                                      min(w, ki - c0), st);
-                tail_add(tc, min(w, ki - c0));
-              }
+  const int p0 = (tbeg ? (int)(tile - tbeg[c]) : 0) * tr, mt = min(tr, m - p0);
+  const int64_t q0 = ebeg ? ebeg[tile] : t_start[c];
+  int64_t q = q0;
+  unsigned long long flops = 0;
+  TailCost tc = tail_cost(mt * n, cls_smax[cls]);
+  for (int kc = 0; kc < S.Dk; ++kc) {
+    const int len = run_len[c * S.Dk + kc];
+    if (len == 0) continue;
+    const int e0 = run_start[c * S.Dk + kc];
+    const int k = S.kval[kc], w = S.wpanel[cls * S.Dk + kc];
+    // stored row strides of the panels: A is m x k (k x m when transposed), B is k x n
+    // (n x k when transposed)
+    const int strides = (S.ta ? m : k) | ((S.tb ? k : n) << 16);
+    const int ki = S.kin ? S.kin[kc] : 0;
+    for (int e = e0; e < e0 + len; ++e) {
+      if (ki > 0) {
+        // slabs of the tensor block (whole blocks only: p0 == 0): stored row stride ki
+        const int64_t ab = S.a_toff[S.s_ab[e]];
+        const int st = ki | ((S.tb ? k : n) << 16);
+        if (w >= ki) {
+          const int ws = (w / ki) * ki;
+          for (int l0 = 0; l0 < k; l0 += ws) {
+            const int b = s_b[e] + (S.tb ? l0 : l0 * n);
+            ents[q++] = make_int4((int)(ab + (int64_t)(l0 / ki) * m * ki), b, min(ws, k - l0), st);
+            tail_add(tc, min(ws, k - l0));
           }
-          continue;
+        } else {
+          for (int l0 = 0; l0 < k; l0 += ki)
+            for (int c0 = 0; c0 < ki; c0 += w) {
+              const int b = s_b[e] + (S.tb ? l0 + c0 : (l0 + c0) * n);
+              ents[q++] = make_int4((int)(ab + (int64_t)(l0 / ki) * m * ki + c0), b,
+                                    min(w, ki - c0), st);
+              tail_add(tc, min(w, ki - c0));
+            }
         }
-        for (int l0 = 0; l0 < k; l0 += w) {
-          const int wl = min(w, k - l0);
-          const int a = s_a[e] + (S.ta ? l0 * m + p0 : p0 * k + l0);
-          const int b = s_b[e] + (S.tb ? l0 : l0 * n);
-          ents[q++] = make_int4(a, b, wl, strides);
-          tail_add(tc, wl);
-        }
+        continue;
       }
-      flops += (unsigned long long)len * mt * n * k;
+      for (int l0 = 0; l0 < k; l0 += w) {
+        const int wl = min(w, k - l0);
+        const int a = s_a[e] + (S.ta ? l0 * m + p0 : p0 * k + l0);
+        const int b = s_b[e] + (S.tb ? l0 : l0 * n);
+        ents[q++] = make_int4(a, b, wl, strides);
+        tail_add(tc, wl);
+      }
     }
-    // the descriptor as two 16-byte stores (word 7, the split, once it is known)
-    int32_t *d = desc + tile * kF64Desc;
-    int4 *dv = reinterpret_cast<int4 *>(d);
-    dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)q0, (int32_t)(q - q0),
-                      mt | (n << 12));
-    key[tile] = __clzll(flops + 1ull);
-    // another pass over the entries costs registers that this kernel has not (plans of long row
-    // tiles 38 -> 47 ms)
-    const bool later = tile_may_split(tc.w1, cls_smax[cls], mt * n, tile_max, slot_elems, nt == 1);
-    const int word =
-        later ? kSplitLater : count_choice(choose_tile(tc, mt * n, (int)(q - q0)), sums);
-    dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, word);
+    flops += (unsigned long long)len * mt * n * k;
   }
+  // the descriptor as two 16-byte stores (word 7, the split, once it is known)
+  int32_t *d = desc + tile * kF64Desc;
+  int4 *dv = reinterpret_cast<int4 *>(d);
+  dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)q0, (int32_t)(q - q0),
+                    mt | (n << 12));
+  key[tile] = __clzll(flops + 1ull);
+  // another pass over the entries costs registers that this kernel has not (plans of long row
+  // tiles 38 -> 47 ms)
+  const bool later = tile_may_split(tc.w1, cls_smax[cls], mt * n, tile_max, slot_elems, tr >= m);
+  const int word =
+      later ? kSplitLater : count_choice(choose_tile(tc, mt * n, (int)(q - q0)), sums);
+  dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, word);
 }
 
-// all C blocks
-__global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
+// all tiles, a thread each (tile_c: the C block of every tile; null: the tile itself).  A thread per
+// C block walked the tiles of large blocks one after another: plans of 200 x 200 blocks 6.5 ms
+__global__ void k_f64_tiles(int64_t ntiles, const int32_t *__restrict__ tile_c,
+                            const int32_t *__restrict__ c_cls,
                             const int32_t *__restrict__ run_start, const int32_t *__restrict__ run_len,
                             const int32_t *__restrict__ s_a, const int32_t *__restrict__ s_b,
                             const int64_t *__restrict__ c_off, const int32_t *__restrict__ c_cin,
@@ -985,10 +987,11 @@ __global__ void k_f64_tiles(int64_t nc, const int32_t *__restrict__ c_cls,
                             int32_t *__restrict__ key, const int32_t *__restrict__ cls_smax,
                             const int32_t *__restrict__ t_start, int tile_max, int slot_elems,
                             SplitSums *__restrict__ sums) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   SplitSums v = {};
-  if (c < nc) f64_tiles_of(c, c_cls, run_start, run_len, s_a, s_b, c_off, c_cin, tbeg, ebeg, S,
-                           desc, ents, key, cls_smax, t_start, tile_max, slot_elems, v);
+  if (t < ntiles)
+    f64_tile_of(t, tile_c ? tile_c[t] : t, c_cls, run_start, run_len, s_a, s_b, c_off, c_cin, tbeg,
+                ebeg, S, desc, ents, key, cls_smax, t_start, tile_max, slot_elems, v);
   add_sums(v, sums);
 }
 
@@ -1352,6 +1355,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   // where a block's tiles and a tile's entries start: with one tile per C block and one
   // entry per product, the block itself and its first product
   int64_t *tbeg = nullptr, *ebeg = nullptr;
+  int32_t *tile_c = nullptr;
   if (ntiles != nc || nents != p->T) {
     int32_t *tcnt = scratch.alloc_n<int32_t>((size_t)nc);
     tbeg = scratch.alloc_n<int64_t>((size_t)nc + 1);
@@ -1359,15 +1363,16 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
     BST_CHECK_LAUNCH();
     exscan_i32_i64(tcnt, tbeg, nc, scratch, s);
     int32_t *ecnt = scratch.alloc_n<int32_t>((size_t)ntiles);
+    tile_c = scratch.alloc_n<int32_t>((size_t)ntiles);
     ebeg = scratch.alloc_n<int64_t>((size_t)ntiles + 1);
-    k_f64_ent_count<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->run_len, tbeg, S, ecnt);
+    k_f64_ent_count<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->run_len, tbeg, S, ecnt, tile_c);
     BST_CHECK_LAUNCH();
     exscan_i32_i64(ecnt, ebeg, ntiles, scratch, s);
   }
   p->fents = ar.alloc_n<int4>((size_t)nents);
   p->fdesc = ar.alloc_n<int32_t>((size_t)ntiles * kF64Desc);
   p->tkeys = ar.alloc_n<int32_t>((size_t)ntiles);
-  k_f64_tiles<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->run_start, p->run_len, p->s_a,
+  k_f64_tiles<<<nblk(ntiles, 256), 256, 0, s>>>(ntiles, tile_c, p->c_cls, p->run_start, p->run_len, p->s_a,
                                             p->s_b, p->C->off, p->c_cin, tbeg, ebeg, S, p->fdesc,
                                             p->fents, p->tkeys, d_smax, p->t_start, tile,
                                             (int)slot, d_sums);
