@@ -8,6 +8,7 @@
 #include <cstring>
 
 #include "bst_internal.h"
+#include "partition.h"
 
 namespace bst {
 
@@ -266,27 +267,40 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-// digit of key[perm[i]] (perm null: key[i]): its `bits` low bits, or those above them
+// digit of key[perm[i]] (perm null: key[i]): the bits of mask from `shift` on
 __global__ void k_key_digit(const int32_t *__restrict__ keys, const int32_t *__restrict__ perm,
-                            int64_t n, int bits, int high, int32_t *__restrict__ dig) {
+                            int64_t n, int shift, int32_t mask, int32_t *__restrict__ dig) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int32_t k = keys[perm ? perm[i] : i];
-  dig[i] = high ? k >> bits : k & ((1 << bits) - 1);
+  dig[i] = (keys[perm ? perm[i] : i] >> shift) & mask;
 }
 
-// perm[i] = p1[p2[i]], and where the sorted keys start: item i opens every key after its
-// predecessor's up to its own
-__global__ void k_compose_keyptr(const int32_t *__restrict__ keys, const int32_t *__restrict__ p1,
-                                 const int32_t *__restrict__ p2, int64_t n, int32_t nkeys,
-                                 int32_t *__restrict__ perm, int32_t *__restrict__ key_ptr) {
+// perm[i] = p1[p2[i]], and the key there
+__global__ void k_compose_sorted(const int32_t *__restrict__ keys, const int32_t *__restrict__ p1,
+                                 const int32_t *__restrict__ p2, int64_t n,
+                                 int32_t *__restrict__ perm, int32_t *__restrict__ sorted) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const int32_t p = p1[p2[i]], k = keys[p];
+  const int32_t p = p1[p2[i]];
   perm[i] = p;
-  for (int32_t q = i ? keys[p1[p2[i - 1]]] + 1 : 0; q <= k; ++q) key_ptr[q] = (int32_t)i;
-  if (i == n - 1)
-    for (int32_t q = k + 1; q <= nkeys; ++q) key_ptr[q] = (int32_t)n;
+  sorted[i] = keys[p];
+}
+
+// where every key starts among the sorted ones: a search per key (an item filling the gap before
+// its key left one thread with all the keys of a sparse range)
+__global__ void k_key_starts(const int32_t *__restrict__ sorted, int64_t n, int32_t nkeys,
+                             int32_t *__restrict__ key_ptr) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q > nkeys) return;
+  int64_t lo = 0, hi = n;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (sorted[mid] < q)
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  key_ptr[q] = (int32_t)lo;
 }
 
 __global__ void k_iota(int32_t *p, int64_t n) {
@@ -554,11 +568,6 @@ void gather_i32(const int32_t *src, const int32_t *idx, int32_t *dst, int64_t n,
 static void partition_pass(const int32_t *keys, int64_t n, int32_t nkeys, int64_t L, int32_t *perm,
                            int32_t *key_ptr, Arena &ar, cudaStream_t s);
 
-// Segment length from which two passes are faster than one: grouping the 3.2 M products of the
-// 2000 x 2000 banded plan by 80 000 blocks took 0.95 ms in one pass of segments of 16 384
-// (two passes: 0.3 ms), the ragged product by 64 000 size buckets 0.37 ms.
-constexpr int64_t kTwoPassSegment = 1024;
-
 void stable_partition(const int32_t *keys, int64_t n, int32_t nkeys, int32_t *perm,
                       int32_t *key_ptr, Arena &ar, cudaStream_t s) {
   BST_REQUIRE(nkeys >= 1, BST_ERR_INVALID_ARG, "stable_partition: nkeys < 1");
@@ -571,30 +580,30 @@ void stable_partition(const int32_t *keys, int64_t n, int32_t nkeys, int32_t *pe
     BST_CHECK_LAUNCH();
     return;
   }
-  // segment length: at least 256 items per warp, and at most 2^24 histogram cells
-  int64_t L = 256;
-  const int64_t max_cells = int64_t(1) << 24;
-  while ((int64_t)nkeys * ((n + L - 1) / L) > max_cells) L *= 2;
-  if (L >= kTwoPassSegment) {
-    // so many keys that a warp would walk thousands of items one batch after another: two
-    // stable passes over the halves of the key instead
-    int bits = 1;
-    while ((1 << (2 * bits)) < nkeys) ++bits;
-    int32_t *dig = ar.alloc_n<int32_t>((size_t)n), *p1 = ar.alloc_n<int32_t>((size_t)n),
-            *p2 = ar.alloc_n<int32_t>((size_t)n);
-    const int32_t lo = 1 << bits, hi = ((nkeys - 1) >> bits) + 1;
-    int32_t *kp = ar.alloc_n<int32_t>((size_t)std::max(lo, hi) + 1);
-    k_key_digit<<<nblk(n, 256), 256, 0, s>>>(keys, nullptr, n, bits, 0, dig);
-    BST_CHECK_LAUNCH();
-    partition_pass(dig, n, lo, 1024, p1, kp, ar, s);
-    k_key_digit<<<nblk(n, 256), 256, 0, s>>>(keys, p1, n, bits, 1, dig);
-    BST_CHECK_LAUNCH();
-    partition_pass(dig, n, hi, 1024, p2, kp, ar, s);
-    k_compose_keyptr<<<nblk(n, 256), 256, 0, s>>>(keys, p1, p2, n, nkeys, perm, key_ptr);
-    BST_CHECK_LAUNCH();
+  const PartitionPlan P = partition_plan(n, nkeys);
+  if (P.passes == 1) {
+    partition_pass(keys, n, nkeys, P.segment[0], perm, key_ptr, ar, s);
     return;
   }
-  partition_pass(keys, n, nkeys, L, perm, key_ptr, ar, s);
+  // so many keys that a warp would walk thousands of items one batch after another: stable passes
+  // over the digits of the key instead
+  int32_t *dig = ar.alloc_n<int32_t>((size_t)n), *order = ar.alloc_n<int32_t>((size_t)n),
+          *p2 = ar.alloc_n<int32_t>((size_t)n);
+  const int64_t most = std::max({P.keys[0], P.keys[1], P.keys[2]});
+  int32_t *kp = ar.alloc_n<int32_t>((size_t)most + 1);
+  const int32_t mask = (int32_t)((int64_t(1) << P.bits) - 1);
+  for (int i = 0; i < P.passes; ++i) {
+    k_key_digit<<<nblk(n, 256), 256, 0, s>>>(keys, i ? order : nullptr, n, i * P.bits, mask, dig);
+    BST_CHECK_LAUNCH();
+    partition_pass(dig, n, (int32_t)P.keys[i], P.segment[i], i ? p2 : order, kp, ar, s);
+    if (i == 0) continue;
+    int32_t *out = i + 1 == P.passes ? perm : ar.alloc_n<int32_t>((size_t)n);
+    k_compose_sorted<<<nblk(n, 256), 256, 0, s>>>(keys, order, p2, n, out, dig);
+    BST_CHECK_LAUNCH();
+    order = out;
+  }
+  k_key_starts<<<nblk((int64_t)nkeys + 1, 256), 256, 0, s>>>(dig, n, nkeys, key_ptr);
+  BST_CHECK_LAUNCH();
 }
 
 static void partition_pass(const int32_t *keys, int64_t n, int32_t nkeys, int64_t L, int32_t *perm,
