@@ -19,6 +19,7 @@
 //   per pass, and read dC and the other operand from L1/L2.  It needs no schedule: it runs
 //   small plans, plans of large blocks and blocks with a dimension of 2^15 or more.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "bst_internal.h"
@@ -33,14 +34,15 @@ struct AdjSide {
   TileLaunch t;
 };
 
-// work counters of adjoint launches captured into a graph (other launches allocate theirs)
+// work counters of the first launches of a plan that are captured into graphs (other launches
+// allocate theirs)
 constexpr int kAdjCounters = 64;
 
 struct AdjState {
   Arena ar;
   AdjSide a, b;
   unsigned long long *counters = nullptr;
-  int next_counter = 0;
+  std::atomic<int> next_counter{0};
 };
 
 namespace {
@@ -567,18 +569,24 @@ static void adj_build(bst_plan *p, AdjState &S, cudaStream_t s) {
 // one side's gradient: out = alpha X Y by the staged schedule
 static void side_staged(bst_plan *p, const AdjSide &D, const double *X, const double *Y, double *out,
                         double alpha, cudaStream_t s) {
-  // adjoints of one plan may overlap on several streams, so each launch has its own work
-  // counter: from the stream's pool, or (a captured launch must not allocate) in turn from
-  // the plan's
+  // Adjoints of one plan may overlap on several streams, so each launch has its own work
+  // counter: from the stream's pool, or (a captured launch must not allocate) one of the plan's.
+  // Graphs keep theirs, and replays of different graphs may overlap too, so none is handed out
+  // twice; once they are used up, a captured launch deals its tiles out in turn (banded_backward
+  // 29.5 -> 30.6 ms).
   AdjState &S = *p->adj;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   BST_CUDA(cudaStreamIsCapturing(s, &cap));
   Arena scratch;
   scratch.ctx = static_cast<Ctx *>(p->ctx);
   scratch.stream = s;
-  unsigned long long *counter = cap == cudaStreamCaptureStatusNone
-                                    ? scratch.alloc_n<unsigned long long>(1)
-                                    : S.counters + S.next_counter++ % kAdjCounters;
+  unsigned long long *counter = nullptr;
+  if (cap == cudaStreamCaptureStatusNone) {
+    counter = scratch.alloc_n<unsigned long long>(1);
+  } else if (S.next_counter.load() < kAdjCounters) {
+    const int i = S.next_counter.fetch_add(1);
+    if (i < kAdjCounters) counter = S.counters + i;
+  }
   launch_fp64_tiles(D.t, X, Y, out, alpha, p->ctx->num_sms, counter, s);
   scratch.release_all();
 }

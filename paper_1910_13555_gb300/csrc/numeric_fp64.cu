@@ -653,16 +653,17 @@ __device__ __forceinline__ void staged_loop(const int64_t *__restrict__ items, i
   };
   // item positions [pos, end) left of the current chunk.  Chunks w and W + w are the
   // warp's own; on opening a chunk lane 0 requests the next one from the counter
-  // (`ticket`, chunk 2 W + ticket), whose value is first read when that chunk opens.
+  // (`ticket`, chunk 2 W + ticket), whose value is first read when that chunk opens.  Without a
+  // counter chunks w, W + w, 2 W + w, ... are the warp's own.
   int64_t pos = gw * chunk, end = pos + chunk;
   bool second = true;
-  unsigned long long ticket = 0;
+  unsigned long long ticket = (unsigned long long)(gw - nw);
   auto next_pos = [&]() -> int64_t {
     if (pos == end) {
       int64_t c = nw + gw;
       if (!second) c = 2 * nw + (int64_t)__shfl_sync(0xffffffffu, ticket, 0);
       second = false;
-      if (lane == 0) ticket = atomicAdd(counter, 1ull);
+      if (lane == 0) ticket = counter ? atomicAdd(counter, 1ull) : ticket + nw;
       pos = c * chunk;
       end = pos + chunk;
     }
@@ -1518,12 +1519,12 @@ static int staged_ctas_per_sm(K kernel, bool &attr_set, int max_slot, int slot_e
 // one launch of a staged kernel instance: as many CTAs as fit (all resident), at most
 // one warp per chunk of work items.  Chunks hold about 1/64 of a warp's share of the
 // items (1 .. 32 items): one counter request per chunk, fine enough that the last
-// chunks are small.  The counter is cleared on the launch's stream.
+// chunks are small.  The counter is cleared on the launch's stream; without one the chunks
+// are dealt out in turn.
 template <class K, class Arg>
 static void staged_launch(K kernel, bool &attr_set, int max_slot, Arg params, const int64_t *items,
                           int64_t nitems, int slot_elems, int num_sms,
                           unsigned long long *counter, cudaStream_t s, int ksplit = 1) {
-  BST_REQUIRE(counter, BST_ERR_STATE, "staged kernel without a work counter");
   size_t smem = 0;
   const int per = staged_ctas_per_sm(kernel, attr_set, max_slot, slot_elems, smem);
   const int64_t full = (int64_t)per * num_sms * kStageWarps;
@@ -1531,7 +1532,7 @@ static void staged_launch(K kernel, bool &attr_set, int max_slot, Arg params, co
   const int64_t nchunks = (nitems + chunk - 1) / chunk;
   const int g = (int)std::min<int64_t>((int64_t)per * num_sms,
                                        (nchunks + kStageWarps - 1) / kStageWarps);
-  BST_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s));
+  if (counter) BST_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s));
   kernel<<<g, 32 * kStageWarps, smem, s>>>(params, items, nitems, slot_elems, counter, chunk,
                                            ksplit);
   BST_CHECK_LAUNCH();
