@@ -1160,8 +1160,8 @@ void sort_items(const int64_t *items, const int32_t *keys, int64_t n, int64_t *o
 }
 
 // Tiles, entries, descriptors and slot size of the staged kernel; false (stage_elems
-// stays 0) when a block size does not fit the descriptor's 12 bits, an inner size the
-// entries' 15, or a row of C (n elements) exceeds one output tile.
+// stays 0) when a block size does not fit the descriptor's 12 bits, a stored row length the
+// entries' strides, or a row of C (n elements) exceeds one output tile.
 static std::vector<int32_t> class_split_bounds(const bst_plan *p);
 static bool split_opens(const SplitSums &v, bool wide);
 static void apply_split_gate(bst_plan *p, const SplitSums &sums, cudaStream_t s);
@@ -1310,7 +1310,10 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
       // panels of about equal width (a narrow last one would cost a whole job); of whole
       // slabs when read in place
       const int64_t k = p->k_vals[kc];
-      if (k >= (1 << 15)) return false;  // an entry holds the stored row strides in 16 bits
+      // an entry holds A's stored row length in 16 bits and B's in 15: op(A)'s rows are k long
+      // where A is not transposed (a slab's k_i), op(B)^T's where B is
+      const int64_t row_a = p->ta ? m : slab ? p->a_slab_kin[(size_t)kc] : k, row_b = p->tb ? k : n;
+      if (row_a >= (1 << 16) || row_b >= (1 << 15)) return false;
       int64_t w = k, panels = 1;
       if (k > wmax) {
         const int64_t np = (k + wmax - 1) / wmax;
