@@ -1592,13 +1592,14 @@ void launch_fp64_persist(const void *params, const int64_t *items, int64_t nitem
 int choose_split(const bst_plan *p, int num_sms) {
   const int64_t nc = p->C->nblocks;
   if (nc <= 0 || p->T <= 0) return 1;
-  // enough work units to fill every SM: the staged kernel's 12 resident warps eight
-  // items each (its tiles; on a 40 x 40-block C of 1600 tiles, parts 1, 2, 4, 8 ran
-  // 611, 748, 803, 930 GFLOP/s), else the direct-load kernel's 32 resident warps (its C
-  // blocks); never more parts than the average number of products per unit
+  // enough work units to fill every SM: the staged kernel's resident warps (16, or 12 in the wide
+  // shape) eight items each (its tiles; counting 16 instead of 12, 40 x 40 C blocks of 23 with 200
+  // products run in 7 parts instead of 5, 6.66 instead of 6.84 ms, of 5, 13 and 23 in 12 instead
+  // of 9, 1.44 instead of 1.49 ms; one part takes 7.65 and 1.90), else the direct-load kernel's 32
+  // resident warps (its C blocks); never more parts than the average number of products per unit
   const bool staged = p->stage_elems > 0;
   const int64_t units = staged ? std::max<int64_t>(p->n_tiles, 1) : nc;
-  const int64_t per_sm = staged ? (int64_t)kStageWarps * 3 * 8 : 32;
+  const int64_t per_sm = staged ? (int64_t)kStageWarps * (p->stage_wide ? 3 : 4) * 8 : 32;
   const int64_t want = ((int64_t)num_sms * per_sm + units - 1) / units;
   const int64_t avg = p->T / units;
   int64_t s = std::min<int64_t>(want, std::max<int64_t>(1, avg));

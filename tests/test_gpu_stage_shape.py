@@ -77,3 +77,16 @@ def test_slab_reading_that_a_block_rules_out_keeps_the_narrow_shape():
     torch.cuda.synchronize()
     ref = oracle.contract(T, U, [0, 2], [0, 1], [1], [2])
     assert rel_fro(plan.result.data[:plan.result.info[2]].cpu().numpy(), ref["data"]) <= 1e-12
+
+
+@pytest.mark.parametrize("m,n,k,kb,warps", [(23, 23, 23, 60, 16), (9, 9, 35, 60, 12), (5, 13, 13, 60, 16)])
+def test_automatic_k_split_counts_the_shape_s_warps(m, n, k, kb, warps):
+    import torch
+    p = _dense(np.random.default_rng(7), m, n, k, 40, kb)
+    out = run_multiply(p, stacks=False, split_k=0)
+    tiles = int(out["plan"].split_histogram().sum())
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    want = -(-sms * warps * 8 // tiles)
+    assert out["stats"]["split_k"] == max(1, min(want, 1600 * kb // tiles, 16))
+    ref = oracle.multiply(p.A, p.B, None, 1.0, 0.0, 0.0)
+    assert rel_fro(out["data"], ref["data"]) <= 1e-12
