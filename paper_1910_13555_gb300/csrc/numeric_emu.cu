@@ -455,19 +455,15 @@ struct EmuParams {
   const double *Cin;
   double *C;
   double alpha, beta;
-  int32_t Dk;
   int32_t alpha_one, has_beta;  // alpha == 1, beta != 0 (set on the host: FP64 compares
                                 // would occupy GB300's slow FP64 pipe in every tile)
   int32_t row_scale;  // 1: digits scaled per whole op row / column (shared by all products)
-  const int64_t *a_rowstart, *b_colstart;
   const int32_t *row_exp, *col_exp;
-  const int32_t *cls_m, *cls_n, *kval;
-  const int32_t *c_row, *c_col, *c_cin, *c_cls;
-  const int64_t *c_off, *cin_off;
-  const int32_t *run_start, *run_len, *s_ab, *s_bb;
+  const int64_t *cin_off;
+  const int32_t *s_ab, *s_bb;
   const int32_t *desc;  // C block (3xTF32: pass) descriptors (kDescWords each)
   const int4 *ents;     // C-major entries
-  const int64_t *a_doff, *b_doff, *a_eoff, *b_eoff;
+  const int64_t *a_eoff, *b_eoff;
   const __nv_bfloat16 *a_dig, *b_dig;
   const float *a_tf, *b_tf;
   const int32_t *a_exp, *b_exp;
@@ -1240,22 +1236,9 @@ EmuParams emu_params(bst_plan *p, const EmuState &E, const NumArgs &a) {
   P.alpha_one = a.alpha == 1.0;
   P.has_beta = a.beta != 0.0;
   P.beta = a.beta;
-  P.Dk = p->Dk;
-  P.a_rowstart = E.a_rowstart;
-  P.b_colstart = E.b_colstart;
   P.row_exp = E.row_exp;
   P.col_exp = E.col_exp;
-  P.cls_m = p->cls_m;
-  P.cls_n = p->cls_n;
-  P.kval = p->kval;
-  P.c_row = p->C->row;
-  P.c_cls = p->c_cls;
-  P.c_col = p->C->col;
-  P.c_cin = p->c_cin;
-  P.c_off = p->C->off;
   P.cin_off = p->Cin ? p->Cin->off : nullptr;
-  P.run_start = p->run_start;
-  P.run_len = p->run_len;
   P.s_ab = p->s_ab;
   P.s_bb = p->s_bb;
   P.desc = E.desc;
@@ -1318,8 +1301,6 @@ static void emu_prepare(bst_plan *p, EmuState &E, const NumArgs &a, cudaStream_t
 
 static EmuParams bf16_params(bst_plan *p, const EmuState &E, const NumArgs &a) {
   EmuParams P = emu_params(p, E, a);
-  P.a_doff = E.a_doff;
-  P.b_doff = E.b_doff;
   P.row_scale = p->ctx->tune_emu_row_scale;
   return P;
 }
