@@ -273,12 +273,22 @@ size_t bst_static_scratch_doubles(void);
  *   dop(B)_kj = alpha sum_{i kept} op(A)_ik^T dC_ij on pattern(B),
  *   dC_in = beta dC on pattern(C_in)  (dC_in may be NULL),
  * written (overwritten) in the stored layout of A, B, C_in.  dC is packed like
- * C_out.  For a contraction plan the buffers are the tensors' packings.  FP64. */
+ * C_out.  For a contraction plan the buffers are the tensors' packings.  FP64.
+ * The plan's first adjoint builds the schedule of every later one and synchronises: per side
+ * either 4 bytes per kept product and stored block, or, where the staged kernel saves time, about
+ * 16 bytes per kept product (per panel of its inner size) and 40 per tile of at most 320 gradient
+ * elements.  Later ones allocate 8 bytes per staged side while they run. */
 bst_status bst_plan_adjoint(bst_plan *plan, const double *dC, double *dA, double *dB,
                             double *dC_in, double alpha, double beta, void *stream);
 /* The same without a C_in gradient: bst_plan_adjoint(plan, dC, dA, dB, NULL, alpha, 0). */
 bst_status bst_multiply_adjoint(bst_plan *plan, const double *dC, double *dA, double *dB,
                                 double alpha, void *stream);
+
+/* How the adjoint of a plan runs (for tests and tuning): info[0] = 1 when the staged kernel
+ * computes dA (0: the direct kernel, or no adjoint of the plan has run yet), info[1] = 1 when its
+ * tiles are parts of gradient blocks or its entries parts of products; info[2], info[3] the same
+ * for dB. */
+bst_status bst_plan_adjoint_info(const bst_plan *plan, int32_t *info);
 
 bst_status bst_plan_destroy(bst_plan *plan);
 

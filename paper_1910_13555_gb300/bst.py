@@ -74,6 +74,7 @@ _SIGS = {
     "bst_plan_get_stacks": ([_VP, _VP, _VP, _VP, _VP, _VP], C.c_int32),
     "bst_plan_split_histogram": ([_VP, _VP], C.c_int32),
     "bst_plan_schedule_info": ([_VP, _VP], C.c_int32),
+    "bst_plan_adjoint_info": ([_VP, _VP], C.c_int32),
     "bst_plan_emu_costs": ([_VP, _VP], C.c_int32),
     "bst_multiply_execute": ([_VP, C.c_double, C.c_double, C.c_int32, C.c_int32, _VP], C.c_int32),
     "bst_multiply_execute_static": ([_VP, C.c_double, C.c_double, C.c_int32, _VP], C.c_int32),
@@ -258,6 +259,14 @@ def bst_plan_schedule_info(plan) -> dict:
     v = np.zeros(4, np.int32)
     _check(load().bst_plan_schedule_info(plan, _ptr(v)), "bst_plan_schedule_info")
     return dict(staged=bool(v[0]), strided=bool(v[1]), split=bool(v[2]), slab=bool(v[3]))
+
+
+def bst_plan_adjoint_info(plan) -> dict:
+    """Which kernel computes the plan's gradients (after its first adjoint): the staged one, and
+    whether over parts of blocks or products, for each operand."""
+    v = np.zeros(4, np.int32)
+    _check(load().bst_plan_adjoint_info(plan, _ptr(v)), "bst_plan_adjoint_info")
+    return dict(a_staged=bool(v[0]), a_tiled=bool(v[1]), b_staged=bool(v[2]), b_tiled=bool(v[3]))
 
 
 def bst_plan_emu_costs(plan) -> dict:

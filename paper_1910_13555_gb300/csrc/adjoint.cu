@@ -545,6 +545,14 @@ void adj_state_free(bst_plan *p) {
   p->adj = nullptr;
 }
 
+void adjoint_info(const bst_plan *p, int32_t *info) {
+  for (int i = 0; i < 2; ++i) {
+    const AdjSide *D = p->adj ? (i ? &p->adj->b : &p->adj->a) : nullptr;
+    info[2 * i] = D && D->staged;
+    info[2 * i + 1] = D && D->staged && D->t.tiled;
+  }
+}
+
 static void adj_build(bst_plan *p, AdjState &S, cudaStream_t s) {
   S.ar.ctx = static_cast<Ctx *>(p->ctx);
   S.ar.stream = s;

@@ -405,6 +405,13 @@ bst_status bst_plan_schedule_info(const bst_plan *plan, int32_t *info) {
   API_END
 }
 
+bst_status bst_plan_adjoint_info(const bst_plan *plan, int32_t *info) {
+  API_BEGIN
+  BST_REQUIRE(plan && info, BST_ERR_INVALID_ARG, "NULL argument");
+  bst::adjoint_info(plan, info);
+  API_END
+}
+
 bst_status bst_plan_emu_costs(bst_plan *plan, double *out) {
   API_BEGIN
   BST_REQUIRE(plan && out, BST_ERR_INVALID_ARG, "NULL argument");

@@ -429,6 +429,7 @@ void contract_finish(bst_plan *p, cudaStream_t s);
 void contract_adjoint(bst_plan *p, const double *dR, double *dT1, double *dT2, double *dRin,
                       double alpha, double beta, cudaStream_t s);
 void contract_free(bst_plan *p);
+void adjoint_info(const bst_plan *p, int32_t *info);
 void adjoint_fp64(bst_plan *p, const double *A, const double *B, const double *dC, double *dA,
                   double *dB, double alpha, cudaStream_t s);
 void scale_cin_grad(bst_plan *p, const double *dC, double *dCin, double beta, cudaStream_t s);
