@@ -99,11 +99,9 @@ __host__ __device__ __forceinline__ int tail_of(const TailCost &C) {
 template <class T>
 struct SplitSteps {
   T steps[kMaxSplit + 1] = {};
-  int wmax = 0;
   __host__ __device__ __forceinline__ void add(int w, T times = 1) {
 #pragma unroll
     for (int s = 2; s <= kMaxSplit; ++s) steps[s] += times * (T)((unsigned)(w + s - 1) / s);
-    wmax = w > wmax ? w : wmax;
   }
 };
 
@@ -154,8 +152,8 @@ __host__ __device__ __forceinline__ TileChoice choose_tile(const TailCost &C, in
 // block).
 //
 // An output of one chain over w1 elements rounds as sqrt(w1); the s partial sums of a whole-tile
-// split as sqrt(w1 / s + s), panels summed by themselves ("fresh") as sqrt(wmax + ne), at one add
-// per output and panel.  The tail split is often cheaper than a whole-tile split but leaves the
+// split as sqrt(w1 / s + s), panels summed by themselves ("fresh") as sqrt(w1 / ne + ne), at one
+// add per output and panel.  The tail split is often cheaper than a whole-tile split but leaves the
 // full rounds one chain: the relative error of 13 x 13 blocks with 60 products of 35 was 1.2e-15
 // that way, 4.4e-16 with the sums split in three.  So where a whole-tile split would pay (at
 // least 1/25 of the unsplit instructions, by the accumulators of the wide shape), it is the
@@ -189,19 +187,20 @@ __host__ __device__ inline TileChoice choose_tile(const TailCost &C, const Split
   if (!split_pays(c0, R.unsplit, w1) || 25 * (R.unsplit - c0) < R.unsplit) s0 = 1;
   R.reference = s0 > 1 ? R.unsplit - c0 : 0;
   const long long limit = s0 > 1 ? inner / (unsigned)s0 + s0 : w1 + ne;
+  const long long width = (inner + (unsigned)ne - 1) / (unsigned)ne;  // of a panel, on average
   long long chain = 0;  // the longest without a whole-tile split
   if (full > 0) {
     if (s0 > 1 && !R.fresh) {
       R.fresh = 1;
       R.cost += kFreshAdd * full * ne;
     }
-    chain = R.fresh ? S.wmax + ne : w1;
+    chain = R.fresh ? width + ne : w1;
   }
   if (R.tail > 1) {
     const long long one = inner / (unsigned)R.tail + R.tail;
     R.tail_fresh = one > limit;
     R.cost += R.tail_fresh ? kFreshAdd * ne : 0;
-    const long long t = R.tail_fresh ? (S.wmax + R.tail - 1) / R.tail + ne : one;
+    const long long t = R.tail_fresh ? (width + R.tail - 1) / R.tail + ne : one;
     chain = chain > t ? chain : t;
   }
   int best = 1, shortest = 1;
