@@ -160,9 +160,10 @@ __host__ __device__ __forceinline__ TileChoice choose_tile(const TailCost &C, in
 // reference: the tile takes the cheapest form whose chains are no longer than that split's.  Parts
 // of blocks have none (in the wide shape they would be larger), nor have panels that the slot cuts
 // to four elements, whose adds cost a third of the time (200 x 200 blocks 64 -> 84 ms).
-// Elsewhere one chain stays, except that long sums over wide panels beside a tail split are
-// fresh too (an add per 16 elements at most; the rank-3 contraction with gradients 2.1e-15, so
-// 0.8e-15, for 1 % of its time).
+// Long sums over wide panels beside a tail split are fresh in any case (an add per 16 elements at
+// most; the rank-3 contraction with gradients 2.1e-15, so 0.8e-15, for 1 % of its time): a
+// whole-tile split with longer chains takes their place only where the narrow shape's is cheaper
+// than the tail split alone.  Elsewhere one chain stays.
 template <class T>
 __host__ __device__ inline TileChoice choose_tile(const TailCost &C, const SplitSteps<T> &S, int mn,
                                                   long long ne, int smax, int tile, int slot,
@@ -173,7 +174,8 @@ __host__ __device__ inline TileChoice choose_tile(const TailCost &C, const Split
   const unsigned inner = w1 < (1ll << 31) ? (unsigned)w1 : 1u << 31;  // for the chains' lengths
   const int full = R.tail > 1 ? mn >> 5 : (mn + 31) >> 5;
   int s0 = 1;
-  long long c0 = R.unsplit;
+  long long c0 = R.unsplit, cn = R.unsplit;
+  const int narrow = split_bound(smax, mn, 32 * kNarrowR, slot);
   const int now = split_bound(smax, mn, tile, slot);
   const int most = whole && w1 > 4 * ne ? split_bound(smax, mn, 32 * kWideR, slot) : 1;
 #pragma unroll
@@ -183,11 +185,14 @@ __host__ __device__ inline TileChoice choose_tile(const TailCost &C, const Split
       c0 = c;
       s0 = s;
     }
+    if (s <= narrow && c < cn) cn = c;
   }
+  const bool narrow_pays = split_pays(cn, R.plain, w1);
   if (!split_pays(c0, R.unsplit, w1) || 25 * (R.unsplit - c0) < R.unsplit) s0 = 1;
   R.reference = s0 > 1 ? R.unsplit - c0 : 0;
-  const long long limit = s0 > 1 ? inner / (unsigned)s0 + s0 : w1 + ne;
   const long long width = (inner + (unsigned)ne - 1) / (unsigned)ne;  // of a panel, on average
+  long long limit = s0 > 1 ? inner / (unsigned)s0 + s0 : w1 + ne;
+  if (R.fresh && !narrow_pays && width + ne < limit) limit = width + ne;
   long long chain = 0;  // the longest without a whole-tile split
   if (full > 0) {
     if (s0 > 1 && !R.fresh) {

@@ -1167,8 +1167,8 @@ static bool split_opens(const SplitSums &v, bool wide);
 static void apply_split_gate(bst_plan *p, const SplitSums &sums, cudaStream_t s);
 
 // FP64 instructions of the plan's tiles in one shape, as choose_tile counts them for tiles with
-// their class's average number of products
-static double shape_cost(const bst_plan *p, const std::vector<int32_t> &smax, bool wide) {
+// their class's average number of products (slab: A is read in place as slabs)
+static double shape_cost(const bst_plan *p, const std::vector<int32_t> &smax, bool wide, bool slab) {
   const int tile = 32 * (wide ? kWideR : kNarrowR), slot_max = wide ? kWideSlot : kNarrowSlot;
   const int32_t ncls = p->Dm * p->Dn, Dk = p->Dk;
   auto rows = [&](int64_t m, int64_t n) { return m * n <= tile ? m : tile / n; };
@@ -1188,20 +1188,26 @@ static double shape_cost(const bst_plan *p, const std::vector<int32_t> &smax, bo
         const int32_t b = cls * Dk + kc;
         const int64_t cnt = (int64_t)p->h_bucket_ptr[b + 1] - p->h_bucket_ptr[b];
         if (cnt == 0) continue;
-        const int64_t k = p->k_vals[kc], np = (k + slot_max / (tr + n) - 1) / (slot_max / (tr + n));
-        const int64_t w = (k + np - 1) / np;
+        const int64_t k = p->k_vals[kc], wmax = slot_max / (tr + n);
+        const int64_t parts = (k + wmax - 1) / wmax;
+        const int64_t w = slab ? std::min(k, wmax) : (k + parts - 1) / parts;
         if (pass == 0) {
           slot = std::max(slot, (tr + n) * w);
           continue;
         }
-        for (int64_t l0 = 0; l0 < k; l0 += w) {
-          const int wl = (int)std::min(w, k - l0);
-          sum.add(wl, cnt);
+        // as k_f64_tiles cuts them: from a range's start on (the whole k, or a slab of k_i), w wide,
+        // or whole slabs
+        const int64_t ki = slab ? p->a_slab_kin[(size_t)kc] : 0;
+        const int64_t range = ki > 0 && w < ki ? ki : k, step = ki > 0 && w >= ki ? w / ki * ki : w;
+        for (int64_t l0 = 0; l0 < range; l0 += step) {
+          const int wl = (int)std::min(step, range - l0);
+          const int64_t times = cnt * (k / range);
+          sum.add(wl, times);
           for (int i = 0; i < 2; ++i)
-            for (int j = 0; j < 2; ++j) tc_sum[i][j] += cnt * ((wl + tc[i].t[j] - 1) / tc[i].t[j]);
+            for (int j = 0; j < 2; ++j) tc_sum[i][j] += times * ((wl + tc[i].t[j] - 1) / tc[i].t[j]);
+          ne += times;
         }
         w1 += cnt * k;
-        ne += cnt * np;
       }
       if (pass == 0) continue;
       for (long long &x : sum.steps) x /= nblk;
@@ -1228,14 +1234,17 @@ static double shape_cost(const bst_plan *p, const std::vector<int32_t> &smax, bo
 
 // Whether the wide shape runs a plan that the narrow one could: where its whole-tile splits (544
 // accumulators instead of 320) and wider panels save more instructions than the fourth CTA is
-// worth: with 60 products of 35, counted 1.04 times as many in the narrow shape, 10 x 10 blocks
-// take 9.33 ms narrow and 9.29 wide; 1.03, 5 x 13 blocks 6.28 and 6.35; 1.12, 5 x 23 blocks 12.1
-// and 10.7; at equal counts the wide shape takes 1.05 to 1.1 times as long.  Only long sums over small blocks can gain, and only bases of few sizes are counted (a
+// worth: with 60 products of 35, counted 1.18 times as many in the narrow shape, 5 x 23 blocks take
+// 12.2 ms narrow and 10.7 wide; 1.34, 7 x 7 blocks 5.91 and 4.82; 1.07, 13 x 13 blocks 16.6 and
+// 15.9; at equal counts the wide shape takes 1.05 to 1.1 times as long (5 x 5 2.38 and 2.59).
+// Slabs want whole slabs in a panel, so there the wider slots are worth more: blocks of 5 and 13
+// over 30 slabs (1.023) take 7.33 ms narrow and 6.54 wide, of 13 (1.030) 18.4 and 17.4, of 16
+// (1.000) 22.9 and 21.8, of 17 (0.948) 25.8 and 26.8.  Only long sums over small blocks can gain, and only bases of few sizes are counted (a
 // pass over classes and inner sizes on the host).
-constexpr double kWideGain = 1.06;
+constexpr double kWideGain = 1.06, kWideGainSlab = 1.0;
 constexpr int32_t kShapeBuckets = 1024;
 
-static bool wide_saves(const bst_plan *p, const std::vector<int32_t> &smax) {
+static bool wide_saves(const bst_plan *p, const std::vector<int32_t> &smax, bool slab) {
   if (p->nb_all > kShapeBuckets) return false;
   bool may = false;
   for (int32_t cls = 0; cls < p->Dm * p->Dn && !may; ++cls) {
@@ -1248,7 +1257,8 @@ static bool wide_saves(const bst_plan *p, const std::vector<int32_t> &smax) {
     }
     may = w1 >= kSplitMinInner * nblk;
   }
-  return may && shape_cost(p, smax, false) >= kWideGain * shape_cost(p, smax, true);
+  return may && shape_cost(p, smax, false, slab) >=
+                    (slab ? kWideGainSlab : kWideGain) * shape_cost(p, smax, true, slab);
 }
 
 static bool build_staged(bst_plan *p, cudaStream_t s) {
@@ -1276,7 +1286,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   const bool slab_fits = slab_wanted && largest <= 32 * kWideR;
   wide = wide || (slab_fits && largest > 32 * kNarrowR);
   const std::vector<int32_t> smax = class_split_bounds(p);
-  wide = wide || (!slab_fits && wide_saves(p, smax));
+  wide = wide || wide_saves(p, smax, slab_fits);
   const int tile = 32 * (wide ? kWideR : kNarrowR), slot_max = wide ? kWideSlot : kNarrowSlot;
   for (int32_t c = 0; c < ncls; ++c) {
     if (p->h_class_ptr[c + 1] == p->h_class_ptr[c]) continue;

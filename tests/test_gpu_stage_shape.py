@@ -79,6 +79,29 @@ def test_slab_reading_that_a_block_rules_out_keeps_the_narrow_shape():
     assert rel_fro(plan.result.data[:plan.result.info[2]].cpu().numpy(), ref["data"]) <= 1e-12
 
 
+# AO sizes; the inner splits of the shape that their plans take
+@pytest.mark.parametrize("sizes,splits", [((9,), {3}), ((7, 12), {2, 3, 7}), ((5, 13), {3, 5, 16}),
+                                          ((17,), {16})])
+def test_slab_reading_of_small_blocks(sizes, splits):
+    import torch
+    from paper_1910_13555_gb300 import bst
+    from paper_1910_13555_gb300.workloads import _tensor
+    rng = np.random.default_rng(4)
+    P, ao = np.full(12, 30, np.int32), np.resize(np.array(sizes, np.int32), 8)
+    every = np.stack([x.ravel() for x in np.meshgrid(range(12), range(8), range(8), indexing="ij")], 1)
+    T, U = _tensor(rng, [P, ao, ao], every), _tensor(rng, [P, ao, ao], every)
+    lib = lambda t: bst.Tensor.from_host(t.block_sizes, t.index, t.data)
+    keep = lib(T), lib(U)
+    plan = bst.contract_plan(*keep, [0, 2], [0, 1], [1], [2], None, None, 0.0)
+    plan.alloc_result()
+    assert plan.schedule_info()["slab"]
+    assert set(np.nonzero(plan.split_histogram())[0]) == splits
+    plan.execute(1.0, 0.0)
+    torch.cuda.synchronize()
+    ref = oracle.contract(T, U, [0, 2], [0, 1], [1], [2])
+    assert rel_fro(plan.result.data[:plan.result.info[2]].cpu().numpy(), ref["data"]) <= 1e-12
+
+
 @pytest.mark.parametrize("m,n,k,kb,warps", [(23, 23, 23, 60, 16), (9, 9, 35, 60, 12), (5, 13, 13, 60, 16)])
 def test_automatic_k_split_counts_the_shape_s_warps(m, n, k, kb, warps):
     import torch
