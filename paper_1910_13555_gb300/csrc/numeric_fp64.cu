@@ -1211,12 +1211,14 @@ static double shape_cost(const bst_plan *p, const std::vector<int32_t> &smax, bo
       }
       if (pass == 0) continue;
       for (long long &x : sum.steps) x /= nblk;
+      // at least one: blocks without products (from C_in) may outnumber the products
+      const int64_t panels = std::max<int64_t>(1, ne / nblk);
       for (int i = 0; i < 2; ++i) {  // whole tiles, and the last rows
         const int mn = (int)((i ? m % tr : tr) * n);
         if (mn == 0) continue;
         tc[i].w1 = w1 / nblk;
         for (int j = 0; j < 2; ++j) tc[i].c[j] += tc_sum[i][j] / nblk;
-        const TileChoice R = choose_tile(tc[i], sum, mn, ne / nblk, smax[cls], tile, (int)slot, tr == m);
+        const TileChoice R = choose_tile(tc[i], sum, mn, panels, smax[cls], tile, (int)slot, tr == m);
         const unsigned long long times = (unsigned long long)(nblk * (i ? 1 : m / tr));
         v.plain += times * R.plain;
         v.saved += times * R.saved;

@@ -58,6 +58,24 @@ def test_narrow_panels_of_row_tiles_keep_one_chain(m, n, k, kb):
     assert rel_fro(out["data"], ref["data"]) <= 1e-12
 
 
+@pytest.mark.parametrize("k,products", [(200, 4), (60, 30), (49, 99)])
+def test_fewer_products_than_blocks(k, products):
+    """C blocks that only C_in has outnumber the products, whose inner sizes make long sums all the
+    same on average."""
+    rng = np.random.default_rng(k)
+    size = lambda v, c: np.full(c, v, np.int32)
+    grid = [x.ravel().astype(np.int32) for x in np.meshgrid(range(10), range(10), indexing="ij")]
+    at = np.sort(rng.choice(100, products, replace=False)).astype(np.int32)
+    A = make_matrix(rng, size(5, 10), size(k, 100), at // 10, at)  # one product each
+    B = make_matrix(rng, size(k, 100), size(13, 10), np.arange(100, dtype=np.int32),
+                    np.arange(100, dtype=np.int32) % 10)
+    C = make_matrix(rng, size(5, 10), size(13, 10), *grid)
+    out = run_multiply(Problem(A, B, C, alpha=1.0, beta=-2.0), stacks=False)
+    ref = oracle.multiply(A, B, C, 1.0, -2.0, 0.0)
+    assert out["stats"]["n_stack"] == products and len(out["rows"]) == 100
+    assert rel_fro(out["data"], ref["data"]) <= 1e-12
+
+
 def test_slab_reading_that_a_block_rules_out_keeps_the_narrow_shape():
     import torch
     from paper_1910_13555_gb300 import bst
