@@ -1525,25 +1525,27 @@ void execute_tf32x3(bst_plan *p, const NumArgs &a, cudaStream_t s) {
     k_tf32_ents<<<nblk(nc, 256), 256, 0, s>>>(nc, p->Dk, p->run_start, p->run_len, p->kval, p->s_ab,
                                               p->s_bb, E.a_toff, E.b_toff, E.ebeg, E.tents);
     BST_CHECK_LAUNCH();
-    Arena scratch;
-    scratch.ctx = static_cast<Ctx *>(p->ctx);
-    scratch.stream = s;
-    int64_t *ubeg = nullptr;
-    if (E.nunits != nc) {
-      int64_t *cnt = scratch.alloc_n<int64_t>((size_t)nc);
-      ubeg = scratch.alloc_n<int64_t>((size_t)nc + 1);
-      k_tf32_passes<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->cls_m, p->cls_n, E.tf_cols, cnt);
-      BST_CHECK_LAUNCH();
-      exscan_i64(cnt, ubeg, nc, scratch, s);
-    }
-    k_tf32_units<<<nblk(nc, 8), 256, 0, s>>>(nc, E.ebeg, ubeg, p->C->off, p->c_cls, p->cls_m,
-                                             p->cls_n, p->c_cin, E.tf_cols, E.tdesc);
-    BST_CHECK_LAUNCH();
     // the lists serve later executes on any stream; an execute captured before they are
     // built builds them in its graph, on every replay
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     BST_CUDA(cudaStreamIsCapturing(s, &cap));
-    if (cap == cudaStreamCaptureStatusNone) {
+    const bool captured = cap != cudaStreamCaptureStatusNone;
+    Arena scratch;
+    scratch.ctx = static_cast<Ctx *>(p->ctx);
+    scratch.stream = s;
+    Arena &tmp = captured ? E.ar : scratch;  // a replay writes them again
+    int64_t *ubeg = nullptr;
+    if (E.nunits != nc) {
+      int64_t *cnt = tmp.alloc_n<int64_t>((size_t)nc);
+      ubeg = tmp.alloc_n<int64_t>((size_t)nc + 1);
+      k_tf32_passes<<<nblk(nc, 256), 256, 0, s>>>(nc, p->c_cls, p->cls_m, p->cls_n, E.tf_cols, cnt);
+      BST_CHECK_LAUNCH();
+      exscan_i64(cnt, ubeg, nc, tmp, s);
+    }
+    k_tf32_units<<<nblk(nc, 8), 256, 0, s>>>(nc, E.ebeg, ubeg, p->C->off, p->c_cls, p->cls_m,
+                                             p->cls_n, p->c_cin, E.tf_cols, E.tdesc);
+    BST_CHECK_LAUNCH();
+    if (!captured) {
       BST_CUDA(cudaStreamSynchronize(s));
       E.tf_lists = true;
     }
