@@ -10,12 +10,13 @@ namespace {
 // * MR = 10, slots of at most 896 doubles: four 4-warp CTAs per SM (at most 128
 //   registers, 4 x (2 x 4 x 896 x 8 B + 1 KB) <= 228 KB).  The FP64 pipe takes 16 SM
 //   cycles per warp FMA and idles when no resident warp has one ready: with 17
-//   accumulators and 1184-double slots 12 warps fitted and the pipe was 94 % busy on the
-//   banded product (20.8 ms); 16 warps keep it 96 % busy (18.9 ms with the tail split).  A
-//   23 x 23 block is then cut into tiles of 13 and 10 rows.
+//   accumulators and 1184-double slots 12 warps fitted and the pipe was 91 % busy on the
+//   2000 x 2000 banded product; 16 warps keep it 94 % busy (4000 x 4000: 20.8 and, with the
+//   tail split, 18.6 ms).  A 23 x 23 block is then cut into tiles of 13 and 10 rows.
 // * MR = 17, slots of 1184 doubles, three CTAs per SM ("wide"): for plans with rows of C
-//   of 321 to 544 elements, and for contractions read in place as slabs (which need whole
-//   C blocks) with blocks of 321 to 544 elements.
+//   of 321 to 544 elements, for contractions read in place as slabs (which need whole
+//   C blocks) with blocks of 321 to 544 elements, and where its splits and panels save
+//   instructions (wide_saves).
 constexpr int kNarrowR = 10, kWideR = 17;
 constexpr int kNarrowSlot = 896, kWideSlot = 1184;
 constexpr int kStageWarps = 4;    // warps per CTA

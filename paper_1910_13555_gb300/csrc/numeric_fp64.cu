@@ -464,8 +464,8 @@ __device__ __forceinline__ void slot_product_rt(const NumParams &P, const double
 // o of the round.  A warp FMA occupies the FP64 pipe for 16 cycles however few lanes are
 // active, so a 13 x 13 tile's sixth round (9 outputs) costs as much as a full one unless
 // three groups share it.  The partial sums are added once per tile (tail_reduce).  On the
-// banded product this takes the FP64 instructions from 189.0 M to 175.2 M (2000 x 2000
-// blocks), 27.9 to 30.8 useful lanes per instruction.
+// banded product this takes the FP64 instructions from 47.8 M to 44.6 M (2000 x 2000
+// blocks at 1 %, 41.7 M full ones).
 struct TailMap {
   int g, p, q;  // group (>= t: idle lane), row and column of the lane's output
 };
