@@ -448,9 +448,9 @@ void side_begin(bst_plan *p, SideBuild &B, AdjState &st, Arena &scratch, cudaStr
   // the direct kernels read the groups on every call, a schedule only while it is built
   Arena &ga = D.staged ? scratch : st.ar;
   D.grp = ga.alloc_n<int32_t>((size_t)p->T);
-  D.ptr = ga.alloc_n<int32_t>((size_t)M.nblocks + 1);
-  stable_partition(B.is_a ? p->s_ab : p->s_bb, p->T,
-                   (int32_t)std::max<int64_t>(M.nblocks, 1), D.grp, D.ptr, scratch, s);
+  const int32_t nkeys = (int32_t)std::max<int64_t>(M.nblocks, 1);  // an operand without blocks too
+  D.ptr = ga.alloc_n<int32_t>((size_t)nkeys + 1);
+  stable_partition(B.is_a ? p->s_ab : p->s_bb, p->T, nkeys, D.grp, D.ptr, scratch, s);
   if (!D.staged) return;
   AdjSched &S = B.S;
   S.nblocks = M.nblocks;
