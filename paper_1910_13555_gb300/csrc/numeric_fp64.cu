@@ -899,8 +899,8 @@ __device__ __forceinline__ int count_choice(const TileChoice &R, SplitSums &v) {
   return choice_word(R);
 }
 
-// word 7 of a tile whose split k_f64_split chooses
-constexpr int kSplitLater = -1;
+// in the cost key (below 64) of a tile whose split k_f64_split chooses
+constexpr int kSplitLater = 64;
 
 // descriptor and entries of a tile of C block c, its cost key (63 - floor(log2(flops)): a
 // stable partition on it lists costly tiles first) and its inner split, with its FP64 instruction
@@ -967,12 +967,11 @@ __device__ __forceinline__ void f64_tile_of(
   int4 *dv = reinterpret_cast<int4 *>(d);
   dv[0] = make_int4((int32_t)(c_off[c] + (int64_t)p0 * n), (int32_t)q0, (int32_t)(q - q0),
                     mt | (n << 12));
-  key[tile] = __clzll(flops + 1ull);
   // another pass over the entries costs registers that this kernel has not (plans of long row
   // tiles 38 -> 47 ms)
   const bool later = tile_may_split(tc.w1, cls_smax[cls], mt * n, tile_max, slot_elems, tr >= m);
-  const int word =
-      later ? kSplitLater : count_choice(choose_tile(tc, mt * n, (int)(q - q0)), sums);
+  key[tile] = __clzll(flops + 1ull) | (later ? kSplitLater : 0);
+  const int word = later ? 0 : count_choice(choose_tile(tc, mt * n, (int)(q - q0)), sums);
   dv[1] = make_int4(c_cin[c], p0 * n, (int32_t)c, word);
 }
 
@@ -996,19 +995,25 @@ __global__ void k_f64_tiles(int64_t ntiles, const int32_t *__restrict__ tile_c,
   add_sums(v, sums);
 }
 
-// word 7 of every tile for new bounds of the inner split; with `item`, only of the tiles that
-// k_f64_tiles left, and the work items 0 .. ntiles - 1
+// word 7 of every tile for new bounds of the inner split; with `item` and `key`, only of the tiles
+// that k_f64_tiles left, and the work items 0 .. ntiles - 1
 __global__ void k_f64_split(int64_t ntiles, const int4 *__restrict__ ents,
                             const int32_t *__restrict__ c_cls, const int32_t *__restrict__ cls_m,
                             const int32_t *__restrict__ cls_smax, int tile_max, int slot_elems,
                             int32_t *__restrict__ desc, SplitSums *__restrict__ sums,
-                            int64_t *__restrict__ item) {
+                            int64_t *__restrict__ item, int32_t *__restrict__ key) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   SplitSums v = {};
   if (t < ntiles) {
-    int32_t *d = desc + t * kF64Desc;
-    if (item) item[t] = t;
-    if (!item || d[7] == kSplitLater) {
+    bool mine = true;
+    if (item) {
+      item[t] = t;
+      const int k = key[t];
+      mine = k & kSplitLater;
+      if (mine) key[t] = k & ~kSplitLater;
+    }
+    if (mine) {
+      int32_t *d = desc + t * kF64Desc;
       const int cls = c_cls[d[6]], smax = cls_smax[cls], ne = d[2];
       const int m = d[3] & 0xfff, mn = m * ((d[3] >> 12) & 0xfff);
       TailCost tc = tail_cost(mn, smax);
@@ -1397,7 +1402,7 @@ static bool build_staged(bst_plan *p, cudaStream_t s) {
   int64_t *it0 = scratch.alloc_n<int64_t>((size_t)ntiles);
   p->titems = ar.alloc_n<int64_t>((size_t)ntiles);
   k_f64_split<<<nblk(ntiles, 128), 128, 0, s>>>(ntiles, p->fents, p->c_cls, p->cls_m, d_smax, tile,
-                                                (int)slot, p->fdesc, d_sums, it0);
+                                                (int)slot, p->fdesc, d_sums, it0, p->tkeys);
   BST_CHECK_LAUNCH();
   sort_items(it0, p->tkeys, ntiles, p->titems, scratch, s);
   SplitSums sums = {};
@@ -1473,7 +1478,7 @@ void refresh_f64_split(bst_plan *p, cudaStream_t s) {
   BST_CUDA(cudaMemsetAsync(d_sums, 0, sizeof(SplitSums), s));
   k_f64_split<<<nblk(p->n_tiles, 128), 128, 0, s>>>(p->n_tiles, p->fents, p->c_cls, p->cls_m, d_smax,
                                                    32 * (p->stage_wide ? kWideR : kNarrowR),
-                                                   p->stage_elems, p->fdesc, d_sums, nullptr);
+                                                   p->stage_elems, p->fdesc, d_sums, nullptr, nullptr);
   BST_CHECK_LAUNCH();
   SplitSums sums = {};
   {
